@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libst.so")
-SOURCES = ["kernels.cu", "band.cu", "band_blk.cu", "st_api.cu", "host_math.cpp", "host_abi.cpp", "noalloc.cu",
+SOURCES = ["kernels.cu", "band.cu", "nd.cu", "st_api.cu", "host_math.cpp", "host_abi.cpp", "noalloc.cu",
            "probe.cu", "combine_ds.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

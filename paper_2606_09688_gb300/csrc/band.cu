@@ -55,45 +55,9 @@ __global__ void k_band_form(const double* __restrict__ Kb, const double* __restr
 }
 
 // Right-looking LDL^T without pivoting of a complex-symmetric band (see
-// band.h for why no pivot is needed).  One CTA per mode; column k:
-// a_{k+i,k+j} -= a_{k+i,k} a_{k+j,k} / d_k, then l_{k+i,k} = a_{k+i,k} / d_k.
-template <typename R>
-__global__ void k_band_ldlt(cx<R>* __restrict__ F, BandLayout L, int* err) {
-  extern __shared__ unsigned char smem_raw[];
-  cx<R>* col = reinterpret_cast<cx<R>*>(smem_raw);
-  const int q = blockIdx.x;
-  const int bw = L.bw, ld = L.ld;
-  const int64_t nrow = L.nrow;
-  cx<R>* Fq = F + (int64_t)q * L.mstride;
-  for (int64_t k = 0; k < nrow; ++k) {
-    __syncthreads();
-    for (int t = threadIdx.x; t <= bw; t += blockDim.x) col[t] = (k + t < nrow) ? Fq[k * ld + t] : mk<R>(0, 0);
-    __syncthreads();
-    const cx<R> d = col[0];
-    if (!(d.re * d.re + d.im * d.im > R(0))) {
-      if (threadIdx.x == 0) atomicExch(err, 1);
-      return;
-    }
-    const cx<R> dinv = cdiv(mk<R>(1, 0), d);
-    const int m = (int)((nrow - 1 - k) < (int64_t)bw ? (nrow - 1 - k) : bw);
-    // pairs (ii, jj) with 1 <= jj <= ii <= m, enumerated row by row of the lower triangle
-    const int npairs = m * (m + 1) / 2;
-    for (int p = threadIdx.x; p < npairs; p += blockDim.x) {
-      int ii = (int)((sqrtf(8.0f * p + 1.0f) - 1.0f) * 0.5f);
-      while (ii * (ii + 1) / 2 > p) --ii;
-      while ((ii + 1) * (ii + 2) / 2 <= p) ++ii;
-      const int jj = p - ii * (ii + 1) / 2;  // 0 <= jj <= ii
-      const int i1 = ii + 1, j1 = jj + 1;
-      cx<R>& tgt = Fq[(k + j1) * ld + (i1 - j1)];
-      tgt = tgt - (col[i1] * col[j1]) * dinv;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x + 1; t <= m; t += blockDim.x) Fq[k * ld + t] = col[t] * dinv;
-    if (threadIdx.x == 0) Fq[k * ld] = dinv;  // the solve multiplies by 1/d_k
-  }
-}
-
-// The same factorisation with the active window in shared memory: column c
+// band.h for why no pivot is needed), one CTA per mode, column k:
+// a_{k+i,k+j} -= a_{k+i,k} a_{k+j,k} / d_k, then l_{k+i,k} = a_{k+i,k} / d_k, with
+// the active window in shared memory: column c
 // of the trailing matrix (rows c..c+bw) lives in slot c mod P, P = bw + 1,
 // entry t at win[slot * P + t].  At column k every pair 1 <= j <= i <= m
 // takes a_{k+i,k+j} -= (a_{k+i,k} / d_k) a_{k+j,k}; thread (i, p) owns row
@@ -221,71 +185,6 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(256)
     }
     __syncthreads();
     slot0 = slot0 + 1 == P ? 0 : slot0 + 1;
-  }
-}
-
-// The global-memory factorisation spread over a cluster of kLdltCluster CTAs
-// per mode (bands whose window does not fit in shared memory): every CTA
-// reads column k, updates its share of the pairs (i, j) (column offsets
-// j = 1 + rank, 1 + rank + kLdltCluster * NP, ...), and one cluster barrier
-// (release / acquire) per column makes the updates visible before column
-// k + 1 is read; rank 0 then stores column k of L (no CTA reads row k again).
-// Every CTA sees the same pivot, so a zero pivot returns all of them together.
-constexpr int kLdltCluster = 4;
-template <typename R>
-__global__ void __cluster_dims__(kLdltCluster, 1, 1) __launch_bounds__(256)
-    k_band_ldlt_cl(cx<R>* __restrict__ F, BandLayout L, int RI, int NP, int* err) {
-  extern __shared__ unsigned char smem_raw[];
-  cx<R>* col = reinterpret_cast<cx<R>*>(smem_raw);
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int q = blockIdx.x / kLdltCluster;
-  const int bw = L.bw, ld = L.ld;
-  const int64_t nrow = L.nrow;
-  cx<R>* Fq = F + (int64_t)q * L.mstride;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int p = tid / RI;
-  const int jstep = NP * kLdltCluster;
-  for (int64_t k = 0; k < nrow; ++k) {
-    for (int t = tid; t <= bw; t += nth) col[t] = (k + t < nrow) ? Fq[k * ld + t] : mk<R>(0, 0);
-    __syncthreads();
-    const cx<R> d = col[0];
-    if (!(d.re * d.re + d.im * d.im > R(0))) {
-      if (tid == 0 && rank == 0) atomicExch(err, 1);
-      return;
-    }
-    const cx<R> dinv = cdiv(mk<R>(1, 0), d);
-    const int m = (int)((nrow - 1 - k) < (int64_t)bw ? (nrow - 1 - k) : bw);
-    // row offsets i = 1 + tid mod RI, + RI, ... (bands wider than the CTA take several)
-    for (int i = 1 + tid % RI; i <= m; i += RI) {
-      const cx<R> u = col[i] * dinv;
-      int j = 1 + rank + kLdltCluster * p;
-      // four column offsets at a time: their four target words are loaded
-      // before any is stored (distinct columns), so four requests are in flight
-      for (; j + 3 * jstep <= i; j += 4 * jstep) {
-        cx<R>* tg[4];
-        cx<R> v[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) tg[r] = Fq + (k + j + r * jstep) * ld + (i - j - r * jstep);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = *tg[r];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const cx<R> a = col[j + r * jstep];
-          *tg[r] = mk<R>(fma(-u.re, a.re, fma(u.im, a.im, v[r].re)), fma(-u.re, a.im, fma(-u.im, a.re, v[r].im)));
-        }
-      }
-      for (; j <= i; j += jstep) {
-        cx<R>& tgt = Fq[(k + j) * ld + (i - j)];
-        const cx<R> a = col[j];
-        tgt = mk<R>(fma(-u.re, a.re, fma(u.im, a.im, tgt.re)), fma(-u.re, a.im, fma(-u.im, a.re, tgt.im)));
-      }
-    }
-    cluster.sync();
-    // column k of L (1/d_k in slot 0) by rank 0, after every CTA has read it
-    if (rank == 0)
-      for (int t = tid; t <= m; t += nth) Fq[k * ld + t] = t == 0 ? dinv : col[t] * dinv;
-    __syncthreads();
   }
 }
 
@@ -782,123 +681,6 @@ __global__ void __launch_bounds__(32 * SLOTS) k_band_solve_mw(const cx<R>* __res
   }
 }
 
-// Wide bands (3D grids: bw = n^2 + n + 1 up to 1024): the fixed-slot solve
-// with one warp per 32-row slot of a window padded to W = 32 * NW >= bw rows
-// (NW = ceil(bw / 32) warps; window offsets beyond bw have zero coupling), the
-// band offsets computed at run time instead of unrolled.  Rows are staged in
-// chunks of C rows (C divides 32) by bulk copies; the finished row of each
-// step is passed through shared memory with one block barrier per row.
-template <typename R>
-__global__ void __launch_bounds__(1024) k_band_solve_mwg(const cx<R>* __restrict__ F, const cx<R>* __restrict__ G,
-                                                         BandLayout L, int C, const cx<R>* __restrict__ b,
-                                                         cx<R>* __restrict__ x, const CocgScal* __restrict__ scal,
-                                                         int64_t vstride, int* err) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int q = blockIdx.x;
-  if (scal != nullptr && !scal[q].active) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5, W = 32 * NW;
-  const int bw = L.bw, ld = L.ld, nrow = (int)L.nrow;
-  const size_t stage_elems = (size_t)C * ld;
-  cx<R>* stage0 = reinterpret_cast<cx<R>*>(smem);
-  cx<R>* stage1 = stage0 + stage_elems;
-  cx<R>* ybuf = stage1 + stage_elems;  // 2 entries, written by other threads between barriers
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ybuf + 2);
-  if (threadIdx.x == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  unsigned phase[2] = {0u, 0u};
-  const int nchunks = (nrow + C - 1) / C;
-  cx<R>* dst = x + (int64_t)q * vstride;
-  const cx<R> zero = mk<R>(0, 0);
-  for (int pass = 0; pass < 2; ++pass) {
-    const cx<R>* Mq = (pass == 0 ? F : G) + (int64_t)q * L.mstride;
-    const cx<R>* src = pass == 0 ? b + (int64_t)q * vstride : dst;
-    auto chunk = [&](int c, int& klo, int& cnt) {
-      const int k0 = c * C;
-      cnt = min(C, nrow - k0);
-      klo = pass == 0 ? k0 : nrow - k0 - cnt;
-    };
-    auto issue = [&](int c) {
-      int klo, cnt;
-      chunk(c, klo, cnt);
-      cx<R>* st = (c & 1) ? stage1 : stage0;
-      const unsigned bytes = (unsigned)((size_t)cnt * ld * sizeof(cx<R>));
-      mbar_expect_tx(&bar[c & 1], bytes);
-      bulk_g2s(st, Mq + (int64_t)klo * ld, bytes, &bar[c & 1]);
-    };
-    auto at = [&](int rp) -> cx<R> {
-      if (rp >= nrow) return zero;
-      return src[pass == 0 ? rp : nrow - 1 - rp];
-    };
-    if (threadIdx.x == 0) {
-      issue(0);
-      if (nchunks > 1) issue(1);
-    }
-    cx<R> v = at(lane + 32 * warp);
-    cx<R> bcur = at(lane + W), bnext = at(32 + lane + W);  // rows entering during groups 0 and 1
-    if (threadIdx.x == 0) ybuf[1] = v;
-    __syncthreads();
-    cx<R> y = ybuf[1];
-    bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
-      ok = mbar_wait_bounded(&bar[c & 1], phase[c & 1]);
-      if (!__syncthreads_and(ok)) {
-        ok = false;
-        break;
-      }
-      phase[c & 1] ^= 1u;
-      int klo, cnt;
-      chunk(c, klo, cnt);
-      const cx<R>* st = (c & 1) ? stage1 : stage0;
-      for (int r = 0; r < cnt; ++r) {
-        const int kp = c * C + r, i = kp & 31, g = kp >> 5;
-        if (i == 0 && g > 0) {
-          bcur = bnext;
-          bnext = at(32 * (g + 1) + lane + W);
-        }
-        const int sg = g % NW;
-        const cx<R>* row = st + (size_t)(pass == 0 ? r : cnt - 1 - r) * ld;
-        if (warp == sg && lane == i) {
-          const int k = pass == 0 ? kp : nrow - 1 - kp;
-          dst[k] = pass == 0 ? y * row[0] : y;
-        }
-        int t;
-        cx<R> base = v;
-        if (warp == sg) {
-          if (lane == i) {
-            t = W;  // the row entering the window
-            base = bcur;
-          } else {
-            t = lane - i + (lane < i ? W : 0);
-          }
-        } else {
-          const int dd = warp - sg;
-          t = lane - i + 32 * (dd < 0 ? dd + NW : dd);
-        }
-        const cx<R> a = t <= bw ? row[t] : zero;
-        v = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, base.re)), fma(-a.re, y.im, fma(-a.im, y.re, base.im)));
-        const int nslot = i < 31 ? sg : (sg + 1 == NW ? 0 : sg + 1);
-        if (warp == nslot && lane == ((i + 1) & 31)) ybuf[kp & 1] = v;
-        __syncthreads();
-        y = ybuf[kp & 1];
-      }
-      __syncthreads();
-      if (threadIdx.x == 0 && c + 2 < nchunks) issue(c + 2);
-    }
-    if (!ok) {
-      if (threadIdx.x == 0) {
-        atomicExch(err, 2);
-        for (int c2 = 0; c2 < 2; ++c2) mbar_wait_bounded(&bar[c2], phase[c2]);
-      }
-      return;
-    }
-    __syncthreads();
-  }
-}
-
 std::mutex g_attr_mu;  // launches come from several host threads (one per component)
 
 template <typename R, int SLOTS> void set_smem_attr(size_t bytes) {
@@ -915,15 +697,6 @@ template <typename R, int SLOTS> void set_smem_attr_mw(size_t bytes) {
   std::lock_guard<std::mutex> lock(g_attr_mu);
   if (bytes > done) {
     cudaFuncSetAttribute(k_band_solve_mw<R, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    done = bytes;
-  }
-}
-
-template <typename R> void set_smem_attr_mwg(size_t bytes) {
-  static size_t done = 0;
-  std::lock_guard<std::mutex> lock(g_attr_mu);
-  if (bytes > done) {
-    cudaFuncSetAttribute(k_band_solve_mwg<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     done = bytes;
   }
 }
@@ -1001,12 +774,6 @@ void launch_band_factor(cx<R>* F, cx<R>* G, const BandLayout& L, int nmodes, int
     const size_t bytes = dsm_bytes(L.bw, 8, sizeof(cx<R>));
     set_smem_attr_ldlt_dsm<R, 8>(bytes);
     k_band_ldlt_dsm<R, 8><<<nmodes * 8, RI * NP, bytes, s>>>(F, L, RI, NP, err);
-  } else if (L.bw <= 1024) {
-    // global memory, four CTAs per mode (the 31^3 grids: half bandwidth 993)
-    const int RI = L.bw <= 256 ? (L.bw + 31) / 32 * 32 : 256, NP = 256 / RI;
-    k_band_ldlt_cl<R><<<nmodes * kLdltCluster, RI * NP, (L.bw + 1) * sizeof(cx<R>), s>>>(F, L, RI, NP, err);
-  } else {
-    k_band_ldlt<R><<<nmodes, 256, (L.bw + 1) * sizeof(cx<R>), s>>>(F, L, err);
   }
   k_band_rows<R><<<dim3(blocks_for(L.nrow * L.ld), nmodes), kBlock, 0, s>>>(F, G, L);
   note_launches(2);
@@ -1023,29 +790,21 @@ bool launch_band_solve(const cx<R>* F, const cx<R>* G, const BandLayout& L, cons
                        const CocgScal* scal, int nmodes, int64_t vstride, int* err, cudaStream_t s) {
   // power-of-two bandwidths (the 2D grids): fixed-slot kernel with 32-row chunks
   const size_t smem32 = 2 * (size_t)32 * L.ld * sizeof(cx<R>) + 2 * sizeof(uint64_t);
-  if (sizeof(R) == 8 && smem32 + 2 * sizeof(cx<R>) <= 160 * 1024 && (L.bw == 64 || L.bw == 128)) {
+  if (sizeof(R) == 8 && smem32 + 2 * sizeof(cx<R>) <= 160 * 1024 && L.bw == 64) {
     // FP64: spread each mode over bw / 32 warps (one FP64 pipe per warp)
     const size_t sm = smem32 + 2 * sizeof(cx<R>);
-    if (L.bw == 64) {
-      set_smem_attr_mw<R, 2>(sm);
-      k_band_solve_mw<R, 2><<<nmodes, 64, sm, s>>>(F, G, L, b, x, scal, vstride, err);
-    } else {
-      set_smem_attr_mw<R, 4>(sm);
-      k_band_solve_mw<R, 4><<<nmodes, 128, sm, s>>>(F, G, L, b, x, scal, vstride, err);
-    }
+    set_smem_attr_mw<R, 2>(sm);
+    k_band_solve_mw<R, 2><<<nmodes, 64, sm, s>>>(F, G, L, b, x, scal, vstride, err);
     note_launches(1);
     return true;
   }
-  if (smem32 <= 160 * 1024 && (L.bw == 32 || L.bw == 64 || L.bw == 128)) {
+  if (smem32 <= 160 * 1024 && (L.bw == 32 || L.bw == 64)) {
     if (L.bw == 32) {
       set_smem_attr_p2<R, 1>(smem32);
       k_band_solve_p2<R, 1><<<nmodes, 32, smem32, s>>>(F, G, L, b, x, scal, vstride, err);
-    } else if (L.bw == 64) {
+    } else {
       set_smem_attr_p2<R, 2>(smem32);
       k_band_solve_p2<R, 2><<<nmodes, 32, smem32, s>>>(F, G, L, b, x, scal, vstride, err);
-    } else {
-      set_smem_attr_p2<R, 4>(smem32);
-      k_band_solve_p2<R, 4><<<nmodes, 32, smem32, s>>>(F, G, L, b, x, scal, vstride, err);
     }
     note_launches(1);
     return true;
@@ -1058,20 +817,9 @@ bool launch_band_solve(const cx<R>* F, const cx<R>* G, const BandLayout& L, cons
   } else if (L.bw <= 64) {
     set_smem_attr<R, 2>(smem);
     k_band_solve_w<R, 2><<<nmodes, 32, smem, s>>>(F, G, L, C, b, x, scal, vstride, err);
-  } else if (L.bw <= 128) {
-    set_smem_attr<R, 4>(smem);
-    k_band_solve_w<R, 4><<<nmodes, 32, smem, s>>>(F, G, L, C, b, x, scal, vstride, err);
   } else if (L.bw <= 256) {
     set_smem_attr<R, 8>(smem);
     k_band_solve_w<R, 8><<<nmodes, 32, smem, s>>>(F, G, L, C, b, x, scal, vstride, err);
-  } else if (L.bw <= 1024) {
-    // wide 3D bands: one warp per 32-row slot of the padded window
-    const int nw = (L.bw + 31) / 32;
-    int cw = 32;
-    while (cw > 1 && 2 * (size_t)cw * L.ld * sizeof(cx<R>) > 160 * 1024) cw >>= 1;
-    const size_t smw = 2 * (size_t)cw * L.ld * sizeof(cx<R>) + 2 * sizeof(cx<R>) + 2 * sizeof(uint64_t);
-    set_smem_attr_mwg<R>(smw);
-    k_band_solve_mwg<R><<<nmodes, 32 * nw, smw, s>>>(F, G, L, cw, b, x, scal, vstride, err);
   } else {
     return false;
   }

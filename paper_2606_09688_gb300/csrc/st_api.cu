@@ -35,6 +35,7 @@
 #include "band.h"
 #include "host_math.h"
 #include "kernels.h"
+#include "nd.h"
 #include <nvtx3/nvToolsExt.h>
 
 using namespace st;
@@ -185,7 +186,8 @@ template <typename R> struct Work {
   cx<R>* band = nullptr;               // F factors, nsel x mstride
   cx<R>* bandG = nullptr;              // G (rows of L), nsel x mstride
   cx<R>* cinv = nullptr;               // coarsest-level inverses, nsel x n x n (small coarse grids)
-  cx<R>* blk = nullptr;                // tile streams of the blocked solve, nsel x tstride (bw <= 128)
+  cx<R>* nd = nullptr;                 // nested dissection matrices, nsel x mstride
+  cx<R>* ndu = nullptr;                // its update values, nsel x ustride
   bool ready = false;
 };
 
@@ -215,7 +217,7 @@ struct Component {
   int64_t nrowc = 0;
   int bw = 0;
   BandLayout bl{};
-  BlkLayout bk{};  // blocked-solve layout of bl (rt = 0: too wide)
+  const NdPlan* nd = nullptr;  // nested dissection of the directly solved grid, or nullptr (banded factors)
   std::vector<double> Kband, Mband;
   double* Kb = nullptr;
   double* Mb = nullptr;
@@ -287,6 +289,7 @@ struct st_handle {
   DevMem mem;
   std::map<int, std::unique_ptr<SpaceLevel>> space;
   std::map<int, std::unique_ptr<TimeData>> time;
+  std::map<std::pair<int, int>, std::unique_ptr<NdPlan>> nd;  // per (spatial level, leaf size)
   std::vector<std::unique_ptr<Component>> comps;
   int nterm_rows = 0;  // n_terms + 2
   double* part = nullptr;
@@ -432,11 +435,11 @@ st_status fail(st_handle* h, st_status code, const std::string& msg) {
   } while (0)
 
 enum KClass {
-  KC_STENCIL = 0, KC_JACOBI, KC_MG_RESID, KC_RESTRICT, KC_PROLONG, KC_BAND_SOLVE, KC_REDUCE, KC_UPDATE,
+  KC_STENCIL = 0, KC_JACOBI, KC_MG_RESID, KC_RESTRICT, KC_PROLONG, KC_DIRECT, KC_REDUCE, KC_UPDATE,
   KC_TRANSFORM, KC_RESIDUAL64, KC_NORM, KC_RHS, KC_SPACE_EIG, KC_COMBINE, KC_SETUP, KC_DENSE_COARSE, KC_COUNT
 };
 const char* const kClassName[KC_COUNT] = {"stencil_apply", "jacobi_smooth", "mg_residual", "mg_restrict",
-                                          "mg_prolong", "band_solve", "cocg_reduce", "cocg_update",
+                                          "mg_prolong", "direct_solve", "cocg_reduce", "cocg_update",
                                           "time_transform", "st_residual_fp64", "norm_fp64", "rhs_assemble",
                                           "space_eigenbasis", "combine_level", "setup", "coarse_inverse"};
 
@@ -796,6 +799,25 @@ double system_norm_bound(const Component& c) {
   return n2(tl.A) * mnorm + n2(tl.B) * knorm;
 }
 
+// Nested dissection plan of a level for nmodes modes, built once per handle.
+st_status nd_of(st_handle* h, const MGLevel& l, int nmodes, size_t rsize, const NdPlan** out) {
+  const int leaf = nd_leaf(l.geo, nmodes, rsize);
+  std::unique_ptr<NdPlan>& slot = h->nd[std::make_pair(l.j, leaf)];
+  if (!slot) {
+    auto p = std::make_unique<NdPlan>(nd_plan(l.geo, leaf));
+    p->idx = h->alloc<int>((size_t)p->nidx);
+    p->map = h->alloc<int>((size_t)p->nidx * 2);
+    p->nb = h->alloc<int>((size_t)p->nnb);
+    ST_NEED(h, p->idx);
+    ST_NEED(h, p->map);
+    ST_NEED(h, p->nb);
+    launch_nd_index(*p, h->stream);
+    slot = std::move(p);
+  }
+  *out = slot.get();
+  return ST_OK;
+}
+
 st_status setup_component(st_handle* h, Component& c) {
   const st_problem& p = h->prob;
   c.nx = c.sl->geo.nnodes;
@@ -959,11 +981,20 @@ st_status setup_component(st_handle* h, Component& c) {
   c.bl = band_layout(c.nrowc, c.bw);
   c.bl.wait = (long long)h->opt.wait_cycles;
   c.bl.stall = h->opt.inject_stall;
-  assemble_band(lc.geo, lc.sc, lc.c2h, c.Kband, c.Mband, c.bw);
-  c.Kb = h->upload(c.Kband);
-  c.Mb = h->upload(c.Mband);
-  ST_NEED(h, c.Kb);
-  ST_NEED(h, c.Mb);
+  // directly solved grids and coarsest grids too large for an explicit inverse
+  // by nested dissection; the banded factors serve the explicit inverses and
+  // the fault injection of the single-warp banded solve (bands above 128)
+  const bool stall = h->opt.inject_stall != 0 && c.bw > 128 && c.bw <= kMaxCoarseBand;
+  if ((c.direct || c.nrowc > kMaxDenseCoarse) && !stall) {
+    st_status s = nd_of(h, lc, c.nsel, c.inner64 ? 8 : 4, &c.nd);
+    if (s != ST_OK) return s;
+  } else {
+    assemble_band(lc.geo, lc.sc, lc.c2h, c.Kband, c.Mband, c.bw);
+    c.Kb = h->upload(c.Kband);
+    c.Mb = h->upload(c.Mband);
+    ST_NEED(h, c.Kb);
+    ST_NEED(h, c.Mb);
+  }
   c.scal = h->alloc<CocgScal>(c.nsel);
   c.part = h->alloc<double>((size_t)c.nsel * 304 * 2);
   ST_NEED(h, c.scal);
@@ -1045,14 +1076,32 @@ template <typename R> st_status prepare_work(st_handle* h, Component& c) {
     }
   }
   // coarsest-level factorisations, one per mode
-  w.band = h->alloc<cx<R>>((size_t)c.nsel * c.bl.mstride);
-  w.bandG = h->alloc<cx<R>>((size_t)c.nsel * c.bl.mstride);
-  ST_NEED(h, w.band);
-  ST_NEED(h, w.bandG);
   ST_CUDA(h, cudaEventRecord(h->entry_ev, h->stream));
   ST_CUDA(h, cudaStreamWaitEvent(c.cs, h->entry_ev, 0));
-  launch_band_form<R>(c.Kb, c.Mb, c.lamP64, w.band, c.bl, c.nsel, c.cs);
-  launch_band_factor<R>(w.band, w.bandG, c.bl, c.nsel, c.cerr, c.cs);
+  if (c.nd != nullptr) {
+    w.nd = h->alloc<cx<R>>((size_t)(c.nsel * c.nd->mstride));
+    w.ndu = h->alloc<cx<R>>((size_t)(c.nsel * c.nd->ustride));
+    ST_NEED(h, w.nd);
+    ST_NEED(h, w.ndu);
+    // workspace of the fronts, returned to the stream's pool after use
+    const size_t wsb = (size_t)c.nsel * c.nd->work_elems * sizeof(cx<R>);
+    if (h->opt.mem_cap_bytes > 0 && h->mem.bytes + wsb > (size_t)h->opt.mem_cap_bytes)
+      return fail(h, ST_ERR_OOM, "device allocation failed");
+    cx<R>* ws = nullptr;
+    if (cudaMallocAsync(reinterpret_cast<void**>(&ws), wsb, c.cs) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(h, ST_ERR_OOM, "device allocation failed");
+    }
+    launch_nd_factor<R>(*c.nd, c.mg.back().sc, c.mg.back().c2d, c.lamP64, c.nsel, w.nd, ws, c.cerr, c.cs);
+    ST_CUDA(h, cudaFreeAsync(ws, c.cs));
+  } else {
+    w.band = h->alloc<cx<R>>((size_t)c.nsel * c.bl.mstride);
+    w.bandG = h->alloc<cx<R>>((size_t)c.nsel * c.bl.mstride);
+    ST_NEED(h, w.band);
+    ST_NEED(h, w.bandG);
+    launch_band_form<R>(c.Kb, c.Mb, c.lamP64, w.band, c.bl, c.nsel, c.cs);
+    launch_band_factor<R>(w.band, w.bandG, c.bl, c.nsel, c.cerr, c.cs);
+  }
   if constexpr (sizeof(R) == 8) {
     // FP64 sweeps are bound by the FP64 pipe: the damped inverse diagonal of
     // every smoothed level and mode is formed once (the complex reciprocal is
@@ -1065,13 +1114,6 @@ template <typename R> st_status prepare_work(st_handle* h, Component& c) {
       launch_jacobi_dinv<R>(lv.geo, lv.sc, lv.c2d, c.lamP64, omega_of(lv.geo.d), c.nsel, lv.geo.nnodes, dv, c.cs);
       lv.sc.dinv = dv;
     }
-  }
-  c.bk = blk_layout(c.bl);
-  if (c.bk.rt > 0 && (c.direct || c.bl.nrow > kMaxDenseCoarse)) {
-    // banded solves in every step: blocked solve with precomputed block inverses
-    w.blk = h->alloc<cx<R>>((size_t)c.nsel * c.bk.tstride);
-    ST_NEED(h, w.blk);
-    launch_band_blk_prepare<R>(w.band, c.bl, c.bk, w.blk, c.nsel, c.cs);
   }
   if (!c.direct && c.bl.nrow <= kMaxDenseCoarse) {
     // multigrid coarsest level: explicit inverses, column j = the banded
@@ -1101,16 +1143,22 @@ template <typename R> const cx<R>* plam_of(const Component& c);
 template <> const cx<double>* plam_of<double>(const Component& c) { return c.lamP64; }
 template <> const cx<float>* plam_of<float>(const Component& c) { return c.lamP32; }
 
-// Banded solve of every active mode of the component's direct grid: the
-// blocked solve when its tile streams exist, the row-by-row kernels otherwise.
+// Direct solve of every active mode of the component's direct grid: nested
+// dissection, or the single-warp banded solve when fault injection asks for it.
 template <typename R>
-bool band_solve(Component& c, const cx<R>* b, cx<R>* x, const CocgScal* scal, int64_t vstride, cudaStream_t s) {
+bool direct_solve(Component& c, const cx<R>* b, cx<R>* x, const CocgScal* scal, int64_t vstride, cudaStream_t s) {
   Work<R>& w = work_of<R>(c);
-  if (w.blk != nullptr) {
-    launch_band_solve_blk<R>(w.band, c.bl, c.bk, w.blk, b, x, scal, c.nsel, vstride, c.cerr, s);
+  if (w.nd != nullptr) {
+    launch_nd_solve<R>(*c.nd, w.nd, b, x, w.ndu, scal, c.nsel, vstride, s);
     return true;
   }
   return launch_band_solve<R>(w.band, w.bandG, c.bl, b, x, scal, c.nsel, vstride, c.cerr, s);
+}
+
+// Algorithmic bytes and flops of one mode's direct solve.
+double direct_flops(const Component& c) { return c.nd != nullptr ? c.nd->solve_flops : (double)c.nrowc * c.bw * 16.0; }
+double direct_bytes(const Component& c, double cs) {
+  return (c.nd != nullptr ? c.nd->solve_flops / 8.0 : 2.0 * c.nrowc * c.bl.ld) * cs + 3.0 * c.nrowc * cs;
 }
 
 double omega_of(int d) { return d == 1 ? kOmega1D : (d == 2 ? kOmega2D : kOmega3D); }
@@ -1134,8 +1182,8 @@ cx<R>* vcycle(st_handle* h, Component& c, int l, const cx<R>* b, cx<R>* xa, cx<R
       PROF(h, s, KC_DENSE_COARSE, (int64_t)(n), m * (double)n * (n + 2.0) * cs, m * (double)n * n * 8.0,
            launch_dense_coarse<R>(w.cinv, n, b, xb, c.scal, c.nsel, n, s));
     } else {
-      PROF(h, s, KC_BAND_SOLVE, (int64_t)(n), m * (double)n * (2.0 * c.bl.ld * cs + 3 * cs),
-           m * (double)n * c.bw * 16.0, band_solve<R>(c, b, xb, c.scal, n, s));
+      PROF(h, s, KC_DIRECT, (int64_t)(n), m * direct_bytes(c, cs), m * direct_flops(c),
+           direct_solve<R>(c, b, xb, c.scal, n, s));
     }
     return xb;
   }
@@ -1308,8 +1356,8 @@ template <typename R> st_status inner_solve(st_handle* h, Component& c, int& ite
   c.nactive = c.nsel;
   if (c.direct) {
     const double m = c.nsel;
-    PROF(h, s, KC_BAND_SOLVE, (int64_t)(n), m * (double)n * (2.0 * c.bl.ld * cs + 3 * cs), m * (double)n * c.bw * 16.0,
-         band_solve<R>(c, w.G, w.X, nullptr, n, s));
+    PROF(h, s, KC_DIRECT, (int64_t)(n), m * direct_bytes(c, cs), m * direct_flops(c),
+         direct_solve<R>(c, w.G, w.X, nullptr, n, s));
     return ccheck(c, "direct band solve");
   }
   const int max_iter = h->opt.max_iter > 0 ? h->opt.max_iter : 1000;
@@ -1611,7 +1659,7 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
       Work<R>& w = work_of<R>(c);
       launch_fwd_transform<R>(io.Wf, c.Rv, w.G, c.nsel, c.nt, c.nx, c.cs);
       if (c.direct) {
-        band_solve<R>(c, w.G, w.X, nullptr, c.nx, c.cs);
+        direct_solve<R>(c, w.G, w.X, nullptr, c.nx, c.cs);
       } else {
         c.nactive = c.nsel;
         cocg_start<R>(h, c);
@@ -2296,7 +2344,7 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
       return ST_ERR_CUDA;
     }
     if (herr != 0) {
-      g_create_error = "zero pivot in a banded LDL^T factorisation";
+      g_create_error = "zero pivot in the factorisation of a spatial problem";
       return ST_ERR_NUMERIC;
     }
   }
