@@ -110,8 +110,10 @@ typedef struct {
                        for FP64 inner solves, 1e-4 for FP32) */
   int max_direct_rows;  /* spatial grids with at most this many unknowns
                            (and a band of at most 1024) are solved by the
-                           banded direct method, larger ones by multigrid-
-                           preconditioned COCG (0 = default 32768) */
+                           direct method (nested dissection), larger ones by
+                           multigrid-preconditioned COCG; 0 = default: grids
+                           of at most 32768 unknowns, and larger ones whose
+                           factorisation is cheap (2D: up to 255 x 255) */
   int autotune;         /* stencil launch shapes (time modes per thread, CTA
                            size) timed per grid size and mode count at setup,
                            before the COCG graphs are captured, and kept for the
@@ -120,9 +122,9 @@ typedef struct {
                             (0 = no cap); an allocation beyond it fails with
                             ST_ERR_OOM, as a real allocation failure would */
   int64_t wait_cycles;  /* cycle budget of each bounded copy wait in the
-                           single-warp banded solves (grids with a half
-                           bandwidth above 128 that are not power-of-two
-                           bands): 0 = 2^31, about one second; a wait that runs
+                           single-warp banded solves (which fault injection
+                           selects for grids with a half bandwidth of 129 to
+                           256): 0 = 2^31, about one second; a wait that runs
                            out makes the solve return ST_ERR_TIMEOUT */
   int inject_stall;     /* fault injection for failure tests: 1 = the first
                            factor-row copy of every single-warp banded solve is

@@ -51,12 +51,20 @@ struct Phase {
   Phase& operator=(const Phase&) = delete;
 };
 
-constexpr int kMaxDirectRows = 32768;  // largest grid solved by the banded direct method (3D: 31^3)
+constexpr int kMaxDirectRows = 32768;  // grids up to this size are solved directly (3D: 31^3) ...
+// ... and larger ones whose factorisation for all modes takes at most this
+// many flops.  The line lies between 255^2 (1.8 GF a mode, at most 9 modes in
+// the 2D configurations) and 511^2 (15 GF a mode).  Solve of a component, MG ->
+// direct: 255^2 FP64 9 modes 9.6 -> 1.36 ms, 3 modes 3.07 -> 0.68 ms, FP32 9
+// modes 5.4 -> 2.2 ms; 511^2 FP64 5 modes 11.9 -> 2.7 ms, but the set-up grows
+// by 0.24 s for 12 ms a solve (255^2: 0.03 s for 11 ms); 511^2 FP32 5.3 -> 4.5 ms
+// alone (four sweeps in place of three) and nothing for the whole step.
+constexpr double kDirectFactorFlops = 2.5e10;
 constexpr int64_t kCoarseFloor = 1024;     // multigrid coarsening stops at the largest grid of at most this size
 constexpr int64_t kMaxDenseCoarse = 4096;  // coarsest multigrid grids up to this size use an explicit inverse
 constexpr int kMaxBandWidth = 1024;    // widest band the warp solve supports
 constexpr int kMaxCoarseBand = 256;    // widest band of a multigrid coarsest grid
-constexpr int64_t kMaxCoarseRows = 16384;  // largest multigrid coarsest grid
+constexpr int64_t kMaxCoarseRows = 32768;  // largest multigrid coarsest grid
 constexpr int kModeSMaxNx = 1024;      // dense spatial eigenbasis limit
 constexpr int kModeTMaxNt = 129;       // time eigenbasis used up to this many time unknowns
 constexpr double kKappaFP32 = 2.0e5;   // cond(V) above which inner solves stay in FP64
@@ -747,15 +755,18 @@ int choose_coarse(const st_problem& p, const Component& c, int64_t max_direct) {
   while (jc < c.jx && kmax * L / (1 << jc) > kThetaMG) ++jc;
   auto fits = [&](int j) {
     const Geo g = make_geo(p.d, j);
-    return g.nnodes <= max_direct && band_width(g) <= kMaxBandWidth;
+    if (max_direct > 0) return g.nnodes <= max_direct && band_width(g) <= kMaxBandWidth;
+    if (g.nnodes <= kMaxDirectRows) return true;
+    return nd_plan(g, nd_leaf(g, c.nsel, c.inner64 ? 8 : 4)).factor_flops * c.nsel <= kDirectFactorFlops;
   };
-  if (fits(c.jx)) return c.jx;  // the banded direct solve beats a V-cycle with a large coarse grid
-  // a coarsest multigrid grid is solved once per V-cycle: keep it within the
-  // fast banded solves (band <= kMaxCoarseBand); modes it cannot resolve get
-  // the shifted V-cycle
+  if (fits(c.jx)) return c.jx;
+  // a coarsest multigrid grid is solved once per V-cycle: at most kMaxCoarseRows
+  // unknowns (3D 31^3: 0.25 ms for 9 modes against 5 ms an iteration that the
+  // unresolved modes of 63^3 lose with 15^3: 158 -> 33 iterations); modes it
+  // cannot resolve get the shifted V-cycle
   auto fits_coarse = [&](int j) {
     const Geo g = make_geo(p.d, j);
-    return fits(j) && g.nnodes <= kMaxCoarseRows && band_width(g) <= kMaxCoarseBand;
+    return g.nnodes <= kMaxCoarseRows && fits(j);
   };
   int jmax = 1;  // largest level the coarse banded solve handles
   while (jmax + 1 <= c.jx && fits_coarse(jmax + 1)) ++jmax;
@@ -911,7 +922,7 @@ st_status setup_component(st_handle* h, Component& c) {
   // time eigenbasis
   c.nsel = c.td->eig.nsel;
   c.inner64 = (h->opt.precision == ST_FP64) || (c.td->eig.cond_est > kKappaFP32);
-  c.jc = choose_coarse(p, c, h->opt.max_direct_rows > 0 ? (int64_t)h->opt.max_direct_rows : kMaxDirectRows);
+  c.jc = choose_coarse(p, c, (int64_t)h->opt.max_direct_rows);
   c.direct = (c.jc == c.jx);
   // multigrid hierarchy jx -> jc (level 0 uses the sampled c^2)
   c.mg.clear();
