@@ -757,6 +757,9 @@ int choose_coarse(const st_problem& p, const Component& c, int64_t max_direct) {
     const Geo g = make_geo(p.d, j);
     if (max_direct > 0) return g.nnodes <= max_direct && band_width(g) <= kMaxBandWidth;
     if (g.nnodes <= kMaxDirectRows) return true;
+    // 1D grids this fine are too ill-conditioned for FP32 factors (2^16 cells: 8
+    // sweeps against 6 with multigrid)
+    if (p.d == 1 && !c.inner64) return false;
     return nd_plan(g, nd_leaf(g, c.nsel, c.inner64 ? 8 : 4)).factor_flops * c.nsel <= kDirectFactorFlops;
   };
   if (fits(c.jx)) return c.jx;
