@@ -933,53 +933,141 @@ __global__ void k_activate(CocgScal* scal, int nmodes) {
 }
 
 // --------------------------------------------------------- time transforms
-constexpr int kQB = 4;
+// FP64 on both paths, so bound by the FP64 pipe (2 multiply-adds a clock and SM)
+// on large grids: a thread takes one node and QB outputs (the 3, 5 or 9
+// time modes or rows of the finest grids in one pass, so that every input is
+// read and, from FP32, converted once), two FP64 multiply-adds per complex
+// coefficient.  On small grids latency bounds them: a CTA takes 32 nodes and QB
+// outputs, its warps share the inputs and meet in shared memory.
+constexpr int kTransWarps = 8;
 
-template <typename R>
+template <typename R, int QB>
 __global__ void __launch_bounds__(kBlock) k_fwd_transform(const cx<double>* __restrict__ W,
                                                           const double* __restrict__ Rt, cx<R>* __restrict__ G,
                                                           int nsel, int nt, int64_t nx) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= nx) return;
-  const int q0 = blockIdx.y * kQB;
-  cx<double> acc[kQB];
+  const int q0 = blockIdx.y * QB;
+  cx<double> acc[QB];
 #pragma unroll
-  for (int u = 0; u < kQB; ++u) acc[u] = mk<double>(0, 0);
+  for (int u = 0; u < QB; ++u) acc[u] = mk<double>(0, 0);
   for (int i = 0; i < nt; ++i) {
     const double r = Rt[(int64_t)i * nx + a];
 #pragma unroll
-    for (int u = 0; u < kQB; ++u)
+    for (int u = 0; u < QB; ++u)
       if (q0 + u < nsel) acc[u] = fma_s(r, W[(int64_t)(q0 + u) * nt + i], acc[u]);
   }
 #pragma unroll
-  for (int u = 0; u < kQB; ++u)
+  for (int u = 0; u < QB; ++u)
     if (q0 + u < nsel) G[(int64_t)(q0 + u) * nx + a] = mk<R>((R)acc[u].re, (R)acc[u].im);
 }
 
-template <typename R>
+template <typename R, int QB>
+__global__ void __launch_bounds__(32 * kTransWarps) k_fwd_transform_split(const cx<double>* __restrict__ W,
+                                                                          const double* __restrict__ Rt,
+                                                                          cx<R>* __restrict__ G, int nsel, int nt,
+                                                                          int64_t nx) {
+  __shared__ cx<double> part[kTransWarps][QB][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t a = (int64_t)blockIdx.x * 32 + lane;
+  const int q0 = blockIdx.y * QB;
+  cx<double> acc[QB];
+#pragma unroll
+  for (int u = 0; u < QB; ++u) acc[u] = mk<double>(0, 0);
+  if (a < nx) {
+#pragma unroll 2
+    for (int i = warp; i < nt; i += kTransWarps) {
+      const double r = Rt[(int64_t)i * nx + a];
+#pragma unroll
+      for (int u = 0; u < QB; ++u)
+        if (q0 + u < nsel) acc[u] = fma_s(r, W[(int64_t)(q0 + u) * nt + i], acc[u]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < QB; ++u) part[warp][u][lane] = acc[u];
+  __syncthreads();
+  for (int e = threadIdx.x; e < QB * 32; e += 32 * kTransWarps) {
+    const int u = e >> 5, l = e & 31;
+    const int64_t al = (int64_t)blockIdx.x * 32 + l;
+    if (q0 + u >= nsel || al >= nx) continue;
+    cx<double> v = part[0][u][l];
+#pragma unroll
+    for (int w = 1; w < kTransWarps; ++w) v = v + part[w][u][l];
+    G[(int64_t)(q0 + u) * nx + al] = mk<R>((R)v.re, (R)v.im);
+  }
+}
+
+// U += Re(V X); V carries the weights (1 or 2) of the folded conjugate modes.
+template <typename R, int QB>
 __global__ void __launch_bounds__(kBlock) k_back_transform(const cx<double>* __restrict__ V,
-                                                           const double* __restrict__ wq,
                                                            const cx<R>* __restrict__ X, double* __restrict__ U,
                                                            int nsel, int nt, int64_t nx) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= nx) return;
-  const int i0 = blockIdx.y * kQB;
-  double acc[kQB];
+  const int i0 = blockIdx.y * QB;
+  double acc[QB];
 #pragma unroll
-  for (int u = 0; u < kQB; ++u) acc[u] = 0.0;
+  for (int u = 0; u < QB; ++u) acc[u] = 0.0;
   for (int q = 0; q < nsel; ++q) {
     const cx<R> xr = X[(int64_t)q * nx + a];
-    const double xre = (double)xr.re, xim = (double)xr.im, w = wq[q];
+    const double xre = (double)xr.re, xim = (double)xr.im;
 #pragma unroll
-    for (int u = 0; u < kQB; ++u)
+    for (int u = 0; u < QB; ++u)
       if (i0 + u < nt) {
         const cx<double> v = V[(int64_t)(i0 + u) * nsel + q];
-        acc[u] = fma(w, v.re * xre - v.im * xim, acc[u]);
+        acc[u] = fma(v.re, xre, fma(-v.im, xim, acc[u]));
       }
   }
 #pragma unroll
-  for (int u = 0; u < kQB; ++u)
+  for (int u = 0; u < QB; ++u)
     if (i0 + u < nt) U[(int64_t)(i0 + u) * nx + a] += acc[u];
+}
+
+template <typename R, int QB>
+__global__ void __launch_bounds__(32 * kTransWarps) k_back_transform_split(const cx<double>* __restrict__ V,
+                                                                           const cx<R>* __restrict__ X,
+                                                                           double* __restrict__ U, int nsel, int nt,
+                                                                           int64_t nx) {
+  __shared__ double part[kTransWarps][QB][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t a = (int64_t)blockIdx.x * 32 + lane;
+  const int i0 = blockIdx.y * QB;
+  double acc[QB];
+#pragma unroll
+  for (int u = 0; u < QB; ++u) acc[u] = 0.0;
+  if (a < nx) {
+#pragma unroll 2
+    for (int q = warp; q < nsel; q += kTransWarps) {
+      const cx<R> xr = X[(int64_t)q * nx + a];
+      const double xre = (double)xr.re, xim = (double)xr.im;
+#pragma unroll
+      for (int u = 0; u < QB; ++u)
+        if (i0 + u < nt) {
+          const cx<double> v = V[(int64_t)(i0 + u) * nsel + q];
+          acc[u] = fma(v.re, xre, fma(-v.im, xim, acc[u]));
+        }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < QB; ++u) part[warp][u][lane] = acc[u];
+  __syncthreads();
+  for (int e = threadIdx.x; e < QB * 32; e += 32 * kTransWarps) {
+    const int u = e >> 5, l = e & 31;
+    const int64_t al = (int64_t)blockIdx.x * 32 + l;
+    if (i0 + u >= nt || al >= nx) continue;
+    double v = part[0][u][l];
+#pragma unroll
+    for (int w = 1; w < kTransWarps; ++w) v += part[w][u][l];
+    U[(int64_t)(i0 + u) * nx + al] += v;
+  }
+}
+
+// A thread per node fills the device from about two CTAs per SM on; below
+// that the split kernel, four outputs a CTA.
+constexpr int kTransSplitQB = 4;
+inline bool transform_split(int64_t nx, int nout, int nin) {
+  const int qb = nout > 5 ? 9 : (nout > 3 ? 5 : 3);
+  return nin >= 4 && (int64_t)blocks_for(nx) * ((nout + qb - 1) / qb) < 304;
 }
 
 // ------------------------------------------------------- FP64 residual, loads
@@ -1038,59 +1126,96 @@ __global__ void __launch_bounds__(kBlock) k_stencil_real2(Geo g, StencilCoef sc,
 // pentadiagonal); row j-2 is complete after step j.  Chunks (the grid's y)
 // only matter for small grids with many time rows; they recompute the two
 // rows of halo on either side.
+// The same pass sums ||R||^2 and ||U||^2: every CTA leaves its partial sums in
+// `part`, and the last one to finish (counter `done`, which wraps back to 0)
+// adds them up in a fixed order into nrm2[0..1], with the component's error
+// word as nrm2[2].
 template <int D>
 __global__ void __launch_bounds__(kBlock) k_residual_fused(Geo g, StencilCoef sc, const double* __restrict__ c2,
                                                            const double* __restrict__ U,
                                                            const double* __restrict__ F,
                                                            const double* __restrict__ Aband,
                                                            const double* __restrict__ Bband,
-                                                           double* __restrict__ Rout, int nt, int chunk) {
+                                                           double* __restrict__ Rout, int nt, int chunk,
+                                                           double* __restrict__ part, unsigned* __restrict__ done,
+                                                           const int* __restrict__ err, double* __restrict__ nrm2) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= g.nnodes) return;
-  const int jb = blockIdx.y * chunk, je = min(nt, jb + chunk);
-  const int64_t nx = g.nnodes;
-  constexpr int NS = ipow3(D);
-  int i[3] = {0, 0, 0};
-  decode<D>(a, g, i);
-  double kr[NS];
-  cell_sums<D, double>(c2, g.N, i, kr);
+  double rr = 0.0, uu = 0.0;
+  if (a < g.nnodes) {
+    const int jb = blockIdx.y * chunk, je = min(nt, jb + chunk);
+    const int64_t nx = g.nnodes;
+    constexpr int NS = ipow3(D), CEN = (NS - 1) / 2;
+    int i[3] = {0, 0, 0};
+    decode<D>(a, g, i);
+    double kr[NS];
+    cell_sums<D, double>(c2, g.N, i, kr);
 #pragma unroll
-  for (int s = 0; s < NS; ++s) kr[s] *= sc.ke[s];
-  int off[NS];
-  unsigned valid = 0u;
+    for (int s = 0; s < NS; ++s) kr[s] *= sc.ke[s];
+    int off[NS];
+    unsigned valid = 0u;
 #pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    int64_t o;
-    if (neighbour<D>(i, s, g.n, o)) valid |= 1u << s;
-    off[s] = (int)o;
-  }
-  double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // rows j-2 .. j+2
-  for (int j = max(0, jb - 2); j <= je + 1; ++j) {
-    if (j < nt) {
-      const double* uj = U + (int64_t)j * nx + a;
-      double ku = 0.0, mu = 0.0;
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        if ((valid >> s) & 1u) {
-          const double v = uj[off[s]];
-          ku = fma(kr[s], v, ku);
-          mu = fma(sc.mtot[s], v, mu);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const int r = j - 2 + k;  // A(r, j) sits at Aband[r * 5 + (j - r) + 2]
-        if (r >= 0 && r < nt) {
-          const int e = r * 5 + 4 - k;
-          acc[k] = fma(-__ldg(Aband + e), mu, fma(-__ldg(Bband + e), ku, acc[k]));
-        }
-      }
+    for (int s = 0; s < NS; ++s) {
+      int64_t o;
+      if (neighbour<D>(i, s, g.n, o)) valid |= 1u << s;
+      off[s] = (int)o;
     }
-    const int done = j - 2;
-    if (done >= jb && done < je) Rout[(int64_t)done * nx + a] = F[(int64_t)done * nx + a] + acc[0];
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // rows j-2 .. j+2
+    for (int j = max(0, jb - 2); j <= je + 1; ++j) {
+      if (j < nt) {
+        const double* uj = U + (int64_t)j * nx + a;
+        double ku = 0.0, mu = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = acc[k + 1];
-    acc[4] = 0.0;
+        for (int s = 0; s < NS; ++s) {
+          if ((valid >> s) & 1u) {
+            const double v = uj[off[s]];
+            ku = fma(kr[s], v, ku);
+            mu = fma(sc.mtot[s], v, mu);
+            if (s == CEN && j >= jb && j < je) uu = fma(v, v, uu);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const int r = j - 2 + k;  // A(r, j) sits at Aband[r * 5 + (j - r) + 2]
+          if (r >= 0 && r < nt) {
+            const int e = r * 5 + 4 - k;
+            acc[k] = fma(-__ldg(Aband + e), mu, fma(-__ldg(Bband + e), ku, acc[k]));
+          }
+        }
+      }
+      const int fin = j - 2;
+      if (fin >= jb && fin < je) {
+        const double r = F[(int64_t)fin * nx + a] + acc[0];
+        Rout[(int64_t)fin * nx + a] = r;
+        rr = fma(r, r, rr);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[k] = acc[k + 1];
+      acc[4] = 0.0;
+    }
+  }
+  __shared__ bool last;
+  const cx<double> s = block_sum(mk<double>(rr, uu));
+  const unsigned nblk = gridDim.x * gridDim.y;
+  if (threadIdx.x == 0) {
+    const unsigned blk = blockIdx.y * gridDim.x + blockIdx.x;
+    part[2 * (size_t)blk] = s.re;
+    part[2 * (size_t)blk + 1] = s.im;
+    __threadfence();
+    last = atomicInc(done, nblk - 1) == nblk - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  cx<double> t = mk<double>(0.0, 0.0);
+  for (unsigned e = threadIdx.x; e < nblk; e += kBlock) {
+    t.re += __ldcg(part + 2 * (size_t)e);
+    t.im += __ldcg(part + 2 * (size_t)e + 1);
+  }
+  t = block_sum(t);
+  if (threadIdx.x == 0) {
+    nrm2[0] = t.re;
+    nrm2[1] = t.im;
+    nrm2[2] = (double)err[0];
   }
 }
 
@@ -1708,32 +1833,68 @@ template <typename R>
 void launch_fwd_transform(const cx<double>* W, const double* Rt, cx<R>* G, int nsel, int nt, int64_t nx,
                           cudaStream_t s) {
   count(1);
-  k_fwd_transform<R><<<dim3(blocks_for(nx), (nsel + kQB - 1) / kQB), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+  if (transform_split(nx, nsel, nt)) {
+    constexpr int QB = kTransSplitQB;
+    k_fwd_transform_split<R, QB><<<dim3(blocks_for(nx, 32), (nsel + QB - 1) / QB), 32 * kTransWarps, 0, s>>>(
+        W, Rt, G, nsel, nt, nx);
+  } else if (nsel > 5) {
+    k_fwd_transform<R, 9><<<dim3(blocks_for(nx), (nsel + 8) / 9), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+  } else if (nsel > 3) {
+    k_fwd_transform<R, 5><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+  } else {
+    k_fwd_transform<R, 3><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+  }
 }
 
 template <typename R>
-void launch_back_transform(const cx<double>* V, const double* wq, const cx<R>* X, double* U, int nsel, int nt,
-                           int64_t nx, cudaStream_t s) {
+void launch_back_transform(const cx<double>* V, const cx<R>* X, double* U, int nsel, int nt, int64_t nx,
+                           cudaStream_t s) {
   count(1);
-  k_back_transform<R><<<dim3(blocks_for(nx), (nt + kQB - 1) / kQB), kBlock, 0, s>>>(V, wq, X, U, nsel, nt, nx);
+  if (transform_split(nx, nt, nsel)) {
+    constexpr int QB = kTransSplitQB;
+    k_back_transform_split<R, QB><<<dim3(blocks_for(nx, 32), (nt + QB - 1) / QB), 32 * kTransWarps, 0, s>>>(
+        V, X, U, nsel, nt, nx);
+  } else if (nt > 5) {
+    k_back_transform<R, 9><<<dim3(blocks_for(nx), (nt + 8) / 9), kBlock, 0, s>>>(V, X, U, nsel, nt, nx);
+  } else if (nt > 3) {
+    k_back_transform<R, 5><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(V, X, U, nsel, nt, nx);
+  } else {
+    k_back_transform<R, 3><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(V, X, U, nsel, nt, nx);
+  }
+}
+
+// Time rows per thread: a chunk pays four halo rows.  Small grids take short
+// chunks (a row costs about 0.8 us of latency), large ones all rows: the
+// estimate adds that latency to the FP64 multiply-adds (2 x 3^d + 10 a row)
+// at 608 a ns.
+static int residual_chunk(const Geo& g, int nt) {
+  const double row_us = (2.0 * ipow3(g.d) + 10.0) / 608.0e3 * (double)g.nnodes * nt;
+  int best = nt;
+  double tbest = 1e300;
+  for (int c = 1;; c = c < nt ? std::min(2 * c, nt) : nt) {
+    const double t = 0.8 * (c + 4) + row_us * (1.0 + (c < nt ? 4.0 / c : 0.0));
+    if (t < tbest && (int64_t)blocks_for(g.nnodes) * ((nt + c - 1) / c) <= 65535) {
+      tbest = t;
+      best = c;
+    }
+    if (c == nt) break;
+  }
+  return best;
+}
+
+int64_t residual_blocks(const Geo& g, int nt) {
+  const int chunk = residual_chunk(g, nt);
+  return (int64_t)blocks_for(g.nnodes) * ((nt + chunk - 1) / chunk);
 }
 
 void launch_residual(const Geo& g, const StencilCoef& sc, const double* c2, const double* U, const double* F,
-                     const double* Aband, const double* Bband, double* KU, double* MU, double* Rout, int nt,
-                     cudaStream_t s) {
+                     const double* Aband, const double* Bband, double* Rout, int nt, double* part, unsigned* done,
+                     const int* err, double* nrm2, cudaStream_t s) {
   count(1);
-  (void)KU;
-  (void)MU;
-  // time chunks of at least 8 rows, as many as it takes to give the grid
-  // about two CTAs per SM
-  const unsigned bx = blocks_for(g.nnodes);
-  int nch = (int)std::min<int64_t>((nt + 7) / 8, (304 + (int64_t)bx - 1) / bx);
-  nch = std::max(nch, 1);
-  const int chunk = (nt + nch - 1) / nch;
-  const dim3 grid(bx, (nt + chunk - 1) / chunk);
-  if (g.d == 1) k_residual_fused<1><<<grid, kBlock, 0, s>>>(g, sc, c2, U, F, Aband, Bband, Rout, nt, chunk);
-  else if (g.d == 2) k_residual_fused<2><<<grid, kBlock, 0, s>>>(g, sc, c2, U, F, Aband, Bband, Rout, nt, chunk);
-  else k_residual_fused<3><<<grid, kBlock, 0, s>>>(g, sc, c2, U, F, Aband, Bband, Rout, nt, chunk);
+  const int chunk = residual_chunk(g, nt);
+  const dim3 grid(blocks_for(g.nnodes), (nt + chunk - 1) / chunk);
+  auto kern = g.d == 1 ? k_residual_fused<1> : (g.d == 2 ? k_residual_fused<2> : k_residual_fused<3>);
+  kern<<<grid, kBlock, 0, s>>>(g, sc, c2, U, F, Aband, Bband, Rout, nt, chunk, part, done, err, nrm2);
 }
 
 void launch_norm2(const double* v, int64_t n, double* part, double* out, cudaStream_t s) {
@@ -2086,8 +2247,7 @@ void note_launches(int k) { count(k); }
                                     int64_t, double, int, cudaStream_t, const double*);                              \
   template void launch_update_p<R>(cx<R>*, const cx<R>*, const CocgScal*, int, int64_t, int64_t, int, cudaStream_t);      \
   template void launch_fwd_transform<R>(const cx<double>*, const double*, cx<R>*, int, int, int64_t, cudaStream_t);  \
-  template void launch_back_transform<R>(const cx<double>*, const double*, const cx<R>*, double*, int, int, int64_t, \
-                                         cudaStream_t);                                                              \
+  template void launch_back_transform<R>(const cx<double>*, const cx<R>*, double*, int, int, int64_t, cudaStream_t); \
   template void launch_dense_coarse<R>(const cx<R>*, int64_t, const cx<R>*, cx<R>*, const CocgScal*, int, int64_t,   \
                                        cudaStream_t);                                                                \
   template void launch_identity<R>(cx<R>*, int64_t, cudaStream_t);                                              \

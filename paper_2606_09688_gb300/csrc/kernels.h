@@ -101,18 +101,22 @@ void launch_refine_decide(RefineRec* rec, const double* nrm2, const double* fn2,
                           cudaGraphConditionalHandle h, InnerTol it, cudaStream_t s);
 
 // Time transforms of the eigenbasis method (FP64 matrices):
-// G[q][a] = sum_i W[q][i] R[i][a];  U[i][a] += sum_q w_q Re(V[i][q] X[q][a]).
+// G[q][a] = sum_i W[q][i] R[i][a];  U[i][a] += sum_q Re(V[i][q] X[q][a]) (V with
+// the weights of the folded conjugate modes).
 template <typename R>
 void launch_fwd_transform(const cx<double>* W, const double* Rt, cx<R>* G, int nsel, int nt, int64_t nx,
                           cudaStream_t s);
 template <typename R>
-void launch_back_transform(const cx<double>* V, const double* wq, const cx<R>* X, double* U, int nsel, int nt,
-                           int64_t nx, cudaStream_t s);
+void launch_back_transform(const cx<double>* V, const cx<R>* X, double* U, int nsel, int nt, int64_t nx,
+                           cudaStream_t s);
 
-// FP64 space-time residual R = F - (A (x) M + B (x) K) U (banded time factors).
+// FP64 space-time residual R = F - (A (x) M + B (x) K) U (banded time factors)
+// with nrm2 = (||R||^2, ||U||^2, err[0]) (device).  part: 2 x residual_blocks
+// doubles of scratch; done: a zeroed counter, left zeroed.
+int64_t residual_blocks(const Geo& g, int nt);
 void launch_residual(const Geo& g, const StencilCoef& sc, const double* c2, const double* U, const double* F,
-                     const double* Aband, const double* Bband, double* KU, double* MU, double* Rout, int nt,
-                     cudaStream_t s);
+                     const double* Aband, const double* Bband, double* Rout, int nt, double* part, unsigned* done,
+                     const int* err, double* nrm2, cudaStream_t s);
 // Sum of squares of a real vector (deterministic), result to out[0] (device).
 void launch_norm2(const double* v, int64_t n, double* part, double* out, cudaStream_t s);
 

@@ -173,8 +173,7 @@ struct TimeData {
   cx<double>* W = nullptr;  // nsel x nt
   cx<double>* V = nullptr;  // nt x nsel
   cx<double>* VT = nullptr;  // nsel x nt: forward transform of the adjoint systems
-  cx<double>* WT = nullptr;  // nt x nsel: their back transform
-  double* wq = nullptr;
+  cx<double>* WT = nullptr;  // nt x nsel: their back transform (V and WT carry the weights of folded conjugate modes)
   cx<double>* lam64 = nullptr;
   cx<float>* lam32 = nullptr;
   double* rhs_coef = nullptr;  // (nterm + 2) x nt
@@ -209,8 +208,7 @@ struct Component {
   double* F = nullptr;
   double* U = nullptr;
   double* Rv = nullptr;
-  double* KU = nullptr;
-  double* MU = nullptr;
+  double* KU = nullptr;  // space eigenbasis: the transformed residual
   double* Fg_all = nullptr;  // general source, time-projected on all nodes (nt x nall), or nullptr
   ds* Uds[2] = {nullptr, nullptr};  // coef (U + u0) as pairs for the combination (nt x nx), two buffers
   ds* Lds = nullptr;                 // coef u0 on all nodes as pairs, or nullptr (written once)
@@ -258,8 +256,9 @@ struct Component {
   // reduction scratch, so that independent components overlap on the GPU.
   cudaStream_t cs = nullptr;
   cudaEvent_t done = nullptr;
-  double* cpart = nullptr;
-  double* cscalar = nullptr;
+  double* cpart = nullptr;     // partial sums of the norms
+  double* cscalar = nullptr;   // ||R||^2, ||U||^2, the error word (launch_residual)
+  unsigned* cdone = nullptr;   // its counter of finished blocks
   double* cscalar_h = nullptr;  // pinned
   int* cerr = nullptr;
   int64_t d2h = 0;
@@ -841,13 +840,11 @@ st_status setup_component(st_handle* h, Component& c) {
   c.F = h->alloc<double>(n);
   c.U = h->alloc<double>(n);
   c.Rv = h->alloc<double>(n);
-  c.KU = h->alloc<double>(n);
-  c.MU = h->alloc<double>(n);
+  if (c.method == 1) c.KU = h->alloc<double>(n);
   ST_NEED(h, c.F);
   ST_NEED(h, c.U);
   ST_NEED(h, c.Rv);
-  ST_NEED(h, c.KU);
-  ST_NEED(h, c.MU);
+  if (c.method == 1) ST_NEED(h, c.KU);
   if (p.f_general != nullptr) {
     // time-projected general source on all nodes: sum_q Q[i][q] f(x, t_q)
     const std::vector<double> pts = node_points(p, c.jx);
@@ -1421,18 +1418,14 @@ st_status assemble_rhs(st_handle* h, Component& c) {
   return ccheck(c, "rhs");
 }
 
-// ||a|| and ||b|| (2-norms) with one synchronisation.
-st_status read_norm2(st_handle* h, Component& c, const double* a, const double* b, int64_t n, double& na, double& nb) {
-  PROF(h, c.cs, KC_NORM, (int64_t)(n), (double)n * 8.0, 2.0 * n, launch_norm2(a, n, c.cpart, c.cscalar, c.cs));
-  PROF(h, c.cs, KC_NORM, (int64_t)(n), (double)n * 8.0, 2.0 * n, launch_norm2(b, n, c.cpart, c.cscalar + 1, c.cs));
-  int serr = 0;
-  ST_CUDAC(c, cudaMemcpyAsync(&serr, c.cerr, sizeof(int), cudaMemcpyDeviceToHost, c.cs));
-  ST_CUDAC(c, cudaMemcpyAsync(c.cscalar_h, c.cscalar, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.cs));
-  c.d2h += (int64_t)(2 * sizeof(double) + sizeof(int));
+// ||R|| and ||U|| of the last residual, with one copy and synchronisation.
+st_status read_norm2(Component& c, double& rn, double& un) {
+  ST_CUDAC(c, cudaMemcpyAsync(c.cscalar_h, c.cscalar, 3 * sizeof(double), cudaMemcpyDeviceToHost, c.cs));
+  c.d2h += (int64_t)(3 * sizeof(double));
   ST_CUDAC(c, cudaStreamSynchronize(c.cs));
-  na = std::sqrt(c.cscalar_h[0]);
-  nb = std::sqrt(c.cscalar_h[1]);
-  if (serr) return cfail(c, ST_ERR_TIMEOUT, "a bounded copy wait in the banded solve timed out");
+  rn = std::sqrt(c.cscalar_h[0]);
+  un = std::sqrt(c.cscalar_h[1]);
+  if (c.cscalar_h[2] != 0.0) return cfail(c, ST_ERR_TIMEOUT, "a bounded copy wait in the banded solve timed out");
   return ccheck(c, "norm");
 }
 
@@ -1477,7 +1470,7 @@ st_status sweep_time_eig(st_handle* h, Component& c, const SolveIO& io, const do
   st_status s = inner_solve<R>(h, c, iters);
   if (s != ST_OK) return s;
   PROF(h, c.cs, KC_TRANSFORM, (int64_t)(c.nx), 2.0 * c.nt * nx * 8.0 + c.nsel * nx * cs, 4.0 * c.nsel * c.nt * nx,
-       launch_back_transform<R>(io.Vb, c.td->wq, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs));
+       launch_back_transform<R>(io.Vb, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs));
   return ccheck(c, "time transforms");
 }
 
@@ -1544,10 +1537,10 @@ st_status solve_one(st_handle* h, Component& c, const SolveIO& io, bool adjoint)
     c.info.sweeps = sw + 1;
     PROF(h, c.cs, KC_RESIDUAL64, (int64_t)(c.nx), 7.0 * (double)n * 8.0 + (double)c.sl->geo.ncells * 8.0,
          (double)n * (4.0 * ipow3(c.sl->geo.d) + 20.0),
-         launch_residual(c.sl->geo, c.sl->sc, c.sl->c2d, io.sol, io.rhs, io.Ab, io.Bb, c.KU, c.MU, c.Rv, c.nt,
-                         c.cs));
+         launch_residual(c.sl->geo, c.sl->sc, c.sl->c2d, io.sol, io.rhs, io.Ab, io.Bb, c.Rv, c.nt, c.cpart, c.cdone,
+                         c.cerr, c.cscalar, c.cs));
     double rn = 0.0, un = 0.0;
-    if ((s = read_norm2(h, c, c.Rv, io.sol, (int64_t)n, rn, un)) != ST_OK) return s;
+    if ((s = read_norm2(c, rn, un)) != ST_OK) return s;
     c.info.max_inner_iters = std::max(c.info.max_inner_iters, iters);
     rel = rn / fn;
     eta = rn / (c.Snorm * un + fn);
@@ -1682,11 +1675,10 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
           ok(capture_add_while(c.cs, hi, &inner), "inner node");
         }
       }
-      launch_back_transform<R>(io.Vb, c.td->wq, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs);
+      launch_back_transform<R>(io.Vb, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs);
     }
-    launch_residual(c.sl->geo, c.sl->sc, c.sl->c2d, io.sol, io.rhs, io.Ab, io.Bb, c.KU, c.MU, c.Rv, c.nt, c.cs);
-    launch_norm2(c.Rv, n, c.cpart, c.cscalar, c.cs);
-    launch_norm2(io.sol, n, c.cpart, c.cscalar + 1, c.cs);
+    launch_residual(c.sl->geo, c.sl->sc, c.sl->c2d, io.sol, io.rhs, io.Ab, io.Bb, c.Rv, c.nt, c.cpart, c.cdone,
+                    c.cerr, c.cscalar, c.cs);
     launch_refine_decide(c.rec, c.cscalar, c.fn2, c.Snorm, tol, max_sweeps, iterative ? c.scal : nullptr, c.nsel,
                          c.cerr, hs, c.itol_rule, c.cs);
     cudaGraph_t out = nullptr;
@@ -1767,14 +1759,17 @@ st_status setup_context(st_handle* h, Component& c) {
   ST_CUDA(h, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
   ST_CUDA(h, cudaStreamCreateWithPriority(&c.cs, cudaStreamNonBlocking, prio_hi));
   ST_CUDA(h, cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming));
-  c.cpart = h->alloc<double>(304);
-  c.cscalar = h->alloc<double>(2);
+  c.cpart = h->alloc<double>((size_t)std::max<int64_t>(304, 2 * residual_blocks(c.sl->geo, c.nt)));
+  c.cscalar = h->alloc<double>(3);
   c.cerr = h->alloc<int>(1);
+  c.cdone = h->alloc<unsigned>(1);
   ST_NEED(h, c.cpart);
   ST_NEED(h, c.cscalar);
   ST_NEED(h, c.cerr);
+  ST_NEED(h, c.cdone);
+  ST_CUDA(h, cudaMemsetAsync(c.cdone, 0, sizeof(unsigned), h->stream));
   ST_CUDA(h, cudaMemsetAsync(c.cerr, 0, sizeof(int), h->stream));
-  ST_CUDA(h, cudaMallocHost(&c.cscalar_h, 2 * sizeof(double)));
+  ST_CUDA(h, cudaMallocHost(&c.cscalar_h, 3 * sizeof(double)));
   if (c.method == 0) {
     st_status s = c.inner64 ? prepare_work<double>(h, c) : prepare_work<float>(h, c);
     if (s != ST_OK) return s;
@@ -2294,7 +2289,11 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
       std::vector<cx<double>> Wc((size_t)ns * ntt), Vc((size_t)ntt * ns), lc(ns);
       std::vector<cx<float>> lf(ns);
       for (size_t e = 0; e < Wc.size(); ++e) Wc[e] = mk(td.eig.W[e].real(), td.eig.W[e].imag());
-      for (size_t e = 0; e < Vc.size(); ++e) Vc[e] = mk(td.eig.V[e].real(), td.eig.V[e].imag());
+      // the back transforms V and W^T with the weights (1 or 2, exact) of the folded conjugate modes
+      for (size_t e = 0; e < Vc.size(); ++e) {
+        const double wt = td.eig.weight[e % ns];
+        Vc[e] = mk(wt * td.eig.V[e].real(), wt * td.eig.V[e].imag());
+      }
       for (int q = 0; q < ns; ++q) {
         lc[q] = mk(td.eig.lam[q].real(), td.eig.lam[q].imag());
         lf[q] = mk((float)td.eig.lam[q].real(), (float)td.eig.lam[q].imag());
@@ -2306,8 +2305,10 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
       std::vector<cx<double>> VTc((size_t)ns * ntt), WTc((size_t)ntt * ns);
       for (int q = 0; q < ns; ++q)
         for (int j = 0; j < ntt; ++j) {
-          VTc[(size_t)q * ntt + j] = Vc[(size_t)j * ns + q];
-          WTc[(size_t)j * ns + q] = Wc[(size_t)q * ntt + j];
+          const std::complex<double> v = td.eig.V[(size_t)j * ns + q], w = td.eig.W[(size_t)q * ntt + j];
+          const double wt = td.eig.weight[q];
+          VTc[(size_t)q * ntt + j] = mk(v.real(), v.imag());
+          WTc[(size_t)j * ns + q] = mk(wt * w.real(), wt * w.imag());
         }
       td.VT = hp->upload(VTc);
       td.WT = hp->upload(WTc);
@@ -2317,8 +2318,7 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
       }
       td.lam64 = hp->upload(lc);
       td.lam32 = hp->upload(lf);
-      td.wq = hp->upload(td.eig.weight);
-      if (!td.W || !td.V || !td.lam64 || !td.lam32 || !td.wq) {
+      if (!td.W || !td.V || !td.lam64 || !td.lam32) {
         g_create_error = "device allocation failed";
         return ST_ERR_OOM;
       }

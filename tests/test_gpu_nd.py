@@ -62,3 +62,19 @@ def test_many_modes_and_one_node_per_leaf():
         for k, info in enumerate(s.components()):
             ref = osolve.solve_component(p, info.jx, info.jt, method="schur")
             assert np.linalg.norm(s.coeffs(k) - ref) / np.linalg.norm(ref) < 1e-10
+
+
+@pytest.mark.parametrize("jx,jt", [(17, 1), (17, 3), (14, 6)])
+def test_long_grids_backward_error(jx, jt):
+    """131071 nodes with 3 and 9 time rows (time transforms with a thread per node, all outputs in one
+    pass) and 16383 with 65 (transforms with split inputs, several time chunks of the residual): the oracle's
+    own normwise backward error, bound 1e-12 as in the full-size tests."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2606_09688_gb300 import Solver
+    p = _problem(1, jx, jt)
+    with Solver(p) as s:
+        assert s.solve(0).status == 0
+        U = s.coeffs(0)
+    assert osolve.backward_error(p, jx, jt, U) < 1e-12
