@@ -131,10 +131,12 @@ typedef struct {
                            never issued, so its bounded wait runs out after
                            wait_cycles and the solve returns ST_ERR_TIMEOUT;
                            0 = off (default) */
-  int device_loop;      /* 0 = host-driven solves (default): the refinement
-                           sweeps and, for multigrid components, graph launches
-                           of 4 COCG iterations with a host check of
-                           convergence after each; k = 4, 8 or 16 = every
+  int device_loop;      /* 0 (default): components without an inner iteration
+                           (direct and space-eigenbasis solves) are one CUDA
+                           graph launch each, as below; multigrid components
+                           are host-driven, with graph launches of 4 COCG
+                           iterations and a host check of convergence after
+                           each; k = 4, 8 or 16 = every
                            forward solve is one CUDA graph launch: the sweeps
                            run in a conditional WHILE node whose stopping test
                            (the backward error, the sweep limit, status words)

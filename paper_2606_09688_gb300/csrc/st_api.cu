@@ -1488,10 +1488,10 @@ st_status sweep_space_eig(st_handle* h, Component& c, const SolveIO& io, const d
 }
 
 st_status enqueue_graph_solve(st_handle* h, Component& c);
-bool graph_solves(const st_handle* h);
+bool graph_solve(const st_handle* h, const Component& c);
 
 st_status solve_one(st_handle* h, Component& c, const SolveIO& io, bool adjoint) {
-  if (!adjoint && graph_solves(h) && c.g_solve != nullptr) return enqueue_graph_solve(h, c);
+  if (!adjoint && graph_solve(h, c)) return enqueue_graph_solve(h, c);
   st_status s = ST_OK;
   if (!adjoint && (s = assemble_rhs(h, c)) != ST_OK) return s;
   const size_t n = (size_t)c.nx * c.nt;
@@ -1747,7 +1747,13 @@ st_status finish_graph_solve(st_handle* h, Component& c) {
   return st;
 }
 
-bool graph_solves(const st_handle* h) { return h->opt.device_loop > 0 && !h->prof_on; }
+// The forward solve of the component is one graph launch (not while profiling).
+bool graph_solve(const st_handle* h, const Component& c) { return c.g_solve != nullptr && !h->prof_on; }
+
+// Waits for those of the listed components whose graph solve is pending (one
+// host synchronisation) and sets their status.
+st_status join_pending(st_handle* h, const std::vector<Component*>& cs, std::vector<st_status>& st);
+
 
 // Execution context of a component: stream, completion event, reduction
 // scratch, and its workspace prepared for the handle's precision.
@@ -1791,7 +1797,14 @@ st_status setup_context(st_handle* h, Component& c) {
       if (s != ST_OK) return s;
     }
   }
-  if (h->opt.device_loop > 0)
+  // Solves as one graph: on request (device_loop > 0), and by default for the
+  // components without an inner iteration, whose few dozen short launches and
+  // one host round trip per sweep (a thread each, 15 to 20 us) cost as much as
+  // their kernels: nine 1D components 0.57 -> 0.27 ms.  Long iterative solves
+  // stay host-driven: a graph occupies one of the device's few launch queues
+  // until it ends, and short solves behind it wait (2D n = 12: 52.8 against
+  // 53.6 ms with every solve as a graph).
+  if (h->opt.device_loop > 0 || c.method == 1 || c.direct)
     return (c.method == 0 && !c.inner64) ? capture_solve_graph<float>(h, c) : capture_solve_graph<double>(h, c);
   return ST_OK;
 }
@@ -1809,6 +1822,23 @@ st_status join_graph_solves(st_handle* h, const std::vector<Component*>& cs, std
     const st_status r = finish_graph_solve(h, *cs[i]);
     if (st[i] == ST_OK) st[i] = r;
   }
+  return ST_OK;
+}
+
+st_status join_pending(st_handle* h, const std::vector<Component*>& cs, std::vector<st_status>& st) {
+  std::vector<Component*> pc;
+  std::vector<st_status> ps;
+  std::vector<size_t> at;
+  for (size_t i = 0; i < cs.size(); ++i)
+    if (cs[i]->rec_pending) {
+      pc.push_back(cs[i]);
+      ps.push_back(st[i]);
+      at.push_back(i);
+    }
+  if (pc.empty()) return ST_OK;
+  const st_status js = join_graph_solves(h, pc, ps);
+  if (js != ST_OK) return js;
+  for (size_t j = 0; j < at.size(); ++j) st[at[j]] = ps[j];
   return ST_OK;
 }
 
@@ -2066,6 +2096,13 @@ void enqueue_comb_level(st_handle* h, const st_handle::CombTables& t, int lev, i
   }
 }
 
+// Component indices by decreasing size: the finest components are the critical path.
+void largest_first(const st_handle* h, std::vector<int>& k) {
+  std::stable_sort(k.begin(), k.end(), [&](int a, int b) {
+    return h->comps[a]->nx * h->comps[a]->nt > h->comps[b]->nx * h->comps[b]->nt;
+  });
+}
+
 // Forward (S U = F) or adjoint (S^T L = G) solves of components k0..k1-1.
 // Component streams start after the work already queued on the handle's
 // stream; independent components run concurrently, one host thread and one
@@ -2084,22 +2121,22 @@ st_status run_solves(st_handle* h, int k0, int k1, bool adjoint, st_solve_info* 
     Component& c = *h->comps[i];
     st[i - k0] = solve_one(h, c, adjoint ? adjoint_io(c) : forward_io(c), adjoint);
   };
-  // graph solves: every component enqueued from this thread, one wait for all
-  const bool graphs = !adjoint && graph_solves(h);
-  if (k1 - k0 > 1 && !h->prof_on && !graphs) {
-    std::vector<std::thread> pool;
-    pool.reserve(k1 - k0);
-    for (int i = k0; i < k1; ++i) pool.emplace_back(run, i);
-    for (auto& t : pool) t.join();
-  } else {
-    for (int i = k0; i < k1; ++i) run(i);
-  }
-  if (graphs) {
-    std::vector<Component*> cs;
-    for (int i = k0; i < k1; ++i) cs.push_back(h->comps[i].get());
-    st_status js = join_graph_solves(h, cs, st);
-    if (js != ST_OK) return js;
-  }
+  // graph solves are enqueued from this thread, largest first, with one wait
+  // for all; host-driven ones run on a thread each, started before them
+  std::vector<int> host, graph;
+  for (int i = k0; i < k1; ++i) (!adjoint && graph_solve(h, *h->comps[i]) ? graph : host).push_back(i);
+  largest_first(h, graph);
+  std::vector<std::thread> pool;
+  if (host.size() + graph.size() > 1 && !h->prof_on)
+    for (int i : host) pool.emplace_back(run, i);
+  for (int i : graph) run(i);
+  if (pool.empty())
+    for (int i : host) run(i);
+  for (auto& t : pool) t.join();
+  std::vector<Component*> cs;
+  for (int i = k0; i < k1; ++i) cs.push_back(h->comps[i].get());
+  st_status js = join_pending(h, cs, st);
+  if (js != ST_OK) return js;
   st_status worst = ST_OK;
   st_solve_info agg{};
   for (int i = k0; i < k1; ++i) {
@@ -2423,31 +2460,30 @@ st_status st_solve_batch(st_handle* const* hs, int n, int max_threads, st_solve_
   }
   std::stable_sort(tasks.begin(), tasks.end(), [](const Task& a, const Task& b) { return a.cost > b.cost; });
   std::vector<st_status> st(tasks.size(), ST_OK);
-  bool graphs = true;
-  for (int i = 0; i < n; ++i) graphs = graphs && graph_solves(hs[i]);
-  if (graphs) {
-    // every component's solve is one graph: all enqueued from this thread,
-    // largest first, then one host synchronisation for the whole batch
+  // graph solves: all enqueued from this thread, largest first; host-driven
+  // ones over a bounded pool of threads started before them; then one host
+  // synchronisation for the graph solves of the whole batch
+  std::vector<size_t> host, graph;
+  for (size_t t = 0; t < tasks.size(); ++t)
+    (graph_solve(tasks[t].h, *tasks[t].h->comps[tasks[t].k]) ? graph : host).push_back(t);
+  auto solve_task = [&](size_t t) {
+    Component& c = *tasks[t].h->comps[tasks[t].k];
+    st[t] = solve_one(tasks[t].h, c, forward_io(c), false);
+  };
+  std::atomic<size_t> next{0};
+  auto worker = [&]() {
+    for (size_t e = next.fetch_add(1); e < host.size(); e = next.fetch_add(1)) solve_task(host[e]);
+  };
+  const int nth = (int)std::min<size_t>(host.size(), max_threads > 0 ? (size_t)max_threads : (size_t)32);
+  std::vector<std::thread> pool;
+  for (int i = 0; i < nth; ++i) pool.emplace_back(worker);
+  for (size_t t : graph) solve_task(t);
+  for (auto& th : pool) th.join();
+  {
     std::vector<Component*> cs;
-    for (size_t t = 0; t < tasks.size(); ++t) {
-      Component& c = *tasks[t].h->comps[tasks[t].k];
-      st[t] = solve_one(tasks[t].h, c, forward_io(c), false);
-      cs.push_back(&c);
-    }
-    st_status js = join_graph_solves(hs[0], cs, st);
+    for (const Task& t : tasks) cs.push_back(t.h->comps[t.k].get());
+    st_status js = join_pending(hs[0], cs, st);
     if (js != ST_OK) return js;
-  } else {
-    std::atomic<size_t> next{0};
-    auto worker = [&]() {
-      for (size_t t = next.fetch_add(1); t < tasks.size(); t = next.fetch_add(1)) {
-        Component& c = *tasks[t].h->comps[tasks[t].k];
-        st[t] = solve_one(tasks[t].h, c, forward_io(c), false);
-      }
-    };
-    const int nth = (int)std::min<size_t>(tasks.size(), max_threads > 0 ? (size_t)max_threads : (size_t)32);
-    std::vector<std::thread> pool;
-    for (int i = 0; i < nth; ++i) pool.emplace_back(worker);
-    for (auto& th : pool) th.join();
   }
   st_status worst = ST_OK;
   st_solve_info agg{};
@@ -2569,28 +2605,27 @@ st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_d
     }
     cv.notify_all();
   };
-  // graph solves are enqueued inline (they return at once); host-driven
-  // solves run on a thread each, except when profiling
-  const bool graphs = graph_solves(h);
+  // host-driven solves run on a thread each (inline, level by level, when
+  // profiling); graph solves are enqueued inline, largest first (the finest
+  // components are the step's critical path), and return at once
+  std::vector<char> graph(nc, 0);
+  std::vector<int> byc;
+  for (int i = 0; i < nc; ++i)
+    if ((graph[i] = graph_solve(h, *h->comps[i]) ? 1 : 0)) byc.push_back(i);
   std::vector<std::thread> pool;
-  if (graphs) {
-    // largest first: the finest components are the step's critical path
-    std::vector<int> byc(nc);
-    for (int i = 0; i < nc; ++i) byc[i] = i;
-    std::stable_sort(byc.begin(), byc.end(), [&](int a, int b) {
-      return h->comps[a]->nx * h->comps[a]->nt > h->comps[b]->nx * h->comps[b]->nt;
-    });
-    for (int i : byc) run(i);
-  } else if (!h->prof_on) {
+  if (!h->prof_on) {
     pool.reserve(nc);
-    for (int i = 0; i < nc; ++i) pool.emplace_back(run, i);
+    for (int i = 0; i < nc; ++i)
+      if (!graph[i]) pool.emplace_back(run, i);
   }
+  largest_first(h, byc);
+  for (int i : byc) run(i);
   bool failed = false;
   for (int lev = t->jmin; lev <= jx_star; ++lev) {
     const int c0 = t->first[lev], c1 = t->first[lev + 1];
     for (int o = c0; o < c1 && !failed; ++o) {
       const int k = t->order[o];
-      if (graphs) {
+      if (graph[k]) {
         // enqueued above
       } else if (h->prof_on) {
         run(k);
@@ -2609,20 +2644,12 @@ st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_d
     if (le != nullptr) cudaEventRecord(le, h->stream);
   }
   for (auto& th : pool) th.join();
-  if (graphs) {
-    // one host synchronisation: the solves' records (the levels may still run)
+  {
+    // one host synchronisation: the records of the graph solves (the levels may still run)
     std::vector<Component*> cs;
-    std::vector<st_status> gst;
-    std::vector<int> idx;
-    for (int i = 0; i < nc; ++i)
-      if (done[i] && h->comps[i]->rec_pending) {
-        cs.push_back(h->comps[i].get());
-        gst.push_back(st[i]);
-        idx.push_back(i);
-      }
-    st_status js = join_graph_solves(h, cs, gst);
+    for (auto& c : h->comps) cs.push_back(c.get());
+    st_status js = join_pending(h, cs, st);
     if (js != ST_OK) return js;
-    for (size_t j = 0; j < idx.size(); ++j) st[idx[j]] = gst[j];
   }
   st_status worst = ST_OK;
   st_solve_info agg{};
