@@ -1546,39 +1546,53 @@ template <typename R> __global__ void k_identity(cx<R>* __restrict__ I, int64_t 
 
 // ----------------------------------------------- receiver misfit gradient
 
-__global__ void __launch_bounds__(kBlock) k_receiver_eval(const CombComp* __restrict__ comps, int ncomp,
+// One thread per receiver, target time and component (blockIdx.z), the
+// components' values added up in component order by k_receiver_sum: a thread
+// that walked all components waited out their loads one after another.
+__global__ void __launch_bounds__(kBlock) k_receiver_eval(const CombComp* __restrict__ comps,
                                                           const RecCorner* __restrict__ rc, int nrec, int ncorner,
                                                           const double* __restrict__ tbv,
-                                                          const int* __restrict__ tspan, int nts,
-                                                          double* __restrict__ out) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
-  if (r >= nrec) return;
-  double val = 0.0;
-  for (int c = 0; c < ncomp; ++c) {
-    const CombComp cc = comps[c];
-    const int n = (1 << cc.jx) - 1, nt = (1 << cc.jt) + 1;
-    int64_t nx = n;  // interior nodes of the component grid (ncorner = 2^d)
-    for (int k = 2; k < ncorner; k <<= 1) nx *= n;
-    const int span = tspan[(int64_t)c * nts + s];
-    const double* tb = tbv + ((int64_t)c * nts + s) * 3;
-    double vc = 0.0;
-    for (int e = 0; e < ncorner; ++e) {
-      const RecCorner q = rc[((int64_t)c * nrec + r) * ncorner + e];
-      double u = 0.0;
-      if (q.interior >= 0)
-        for (int t = 0; t < 3; ++t) {
-          const int row = span + t - 1;
-          if (row >= 0 && row < nt) u = fma(tb[t], cc.U[(int64_t)row * nx + q.interior], u);
-        }
-      if (cc.lift != nullptr) u += cc.lift[q.all];
-      vc = fma(q.w, u, vc);
+                                                          const int* __restrict__ tspan, int nts, int c0,
+                                                          double* __restrict__ part) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (int64_t)nts * nrec) return;
+  const int s = (int)(e / nrec), r = (int)(e - (int64_t)s * nrec), c = c0 + blockIdx.z;
+  const CombComp cc = comps[c];
+  const int n = (1 << cc.jx) - 1, nt = (1 << cc.jt) + 1;
+  int64_t nx = n;  // interior nodes of the component grid (ncorner = 2^d)
+  for (int k = 2; k < ncorner; k <<= 1) nx *= n;
+  const int span = tspan[(int64_t)c * nts + s];
+  const double* tb = tbv + ((int64_t)c * nts + s) * 3;
+  double vc = 0.0;
+  for (int k = 0; k < ncorner; ++k) {
+    const RecCorner q = rc[((int64_t)c * nrec + r) * ncorner + k];
+    double u = 0.0;
+    if (q.interior >= 0) {
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        const int row = span + t - 1;
+        if (row >= 0 && row < nt) u = fma(tb[t], cc.U[(int64_t)row * nx + q.interior], u);
+      }
     }
-    val = fma((double)cc.coef, vc, val);
+    if (cc.lift != nullptr) u += cc.lift[q.all];
+    vc = fma(q.w, u, vc);
   }
-  out[(int64_t)s * nrec + r] = val;
+  part[(int64_t)blockIdx.z * nts * nrec + e] = vc;
 }
 
-__global__ void __launch_bounds__(kBlock) k_misfit(const double* __restrict__ vals, const double* __restrict__ dobs,
+// out (+)= sum of the group's components c0 .. c0 + ncomp - 1
+__global__ void __launch_bounds__(kBlock) k_receiver_sum(const CombComp* __restrict__ comps, int c0, int ncomp,
+                                                         const double* __restrict__ part, int64_t n,
+                                                         double* __restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  double val = c0 > 0 ? out[e] : 0.0;
+#pragma unroll 4
+  for (int c = 0; c < ncomp; ++c) val = fma((double)comps[c0 + c].coef, part[(int64_t)c * n + e], val);
+  out[e] = val;
+}
+
+__global__ void __launch_bounds__(1024) k_misfit(const double* __restrict__ vals, const double* __restrict__ dobs,
                                                    int nts, int nrec, double T, double* __restrict__ wm,
                                                    double* __restrict__ Jout) {
   const double dt = T / (double)(nts - 1);
@@ -1594,37 +1608,56 @@ __global__ void __launch_bounds__(kBlock) k_misfit(const double* __restrict__ va
   if (threadIdx.x == 0) Jout[0] = 0.5 * t.re;
 }
 
-// ehat[i][r] = sum_s psi_i(t_s) wm[s][r] (one thread per receiver, no races)
-__global__ void k_adj_time_project(const double* __restrict__ wm, int nts, int nrec, const double* __restrict__ tb,
-                                   const int* __restrict__ tspan, int nt, double* __restrict__ ehat) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrec) return;
-  for (int i = 0; i < nt; ++i) ehat[(int64_t)i * nrec + r] = 0.0;
-  for (int s = 0; s < nts; ++s) {
-    const double m = wm[(int64_t)s * nrec + r];
-    for (int t = 0; t < 3; ++t) {
-      const int row = tspan[s] + t - 1;
-      if (row >= 0 && row < nt) ehat[(int64_t)row * nrec + r] = fma(tb[s * 3 + t], m, ehat[(int64_t)row * nrec + r]);
-    }
+// Adjoint right-hand sides of all components (blockIdx.y = component, one
+// thread per time row i and receiver r):
+//   e = sum_s psi_i(t_s) wm[s][r],  G_i += coef e (multilinear weights of x_r).
+// Row i only meets the target times of its three intervals, so the thread
+// walks those (a walk over all times by one thread per receiver took 0.3 ms a
+// component at 257 times).
+__global__ void __launch_bounds__(kBlock) k_adj_rhs(const double* __restrict__ wm, int nts, int jt_star, int nrec,
+                                                    const AdjComp* __restrict__ comps, const double* __restrict__ tbv,
+                                                    const int* __restrict__ tspan, const RecCorner* __restrict__ rc,
+                                                    int ncorner) {
+  const AdjComp c = comps[blockIdx.y];
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int nt = (1 << c.jt) + 1;
+  if (e >= (int64_t)nt * nrec) return;
+  const int i = (int)(e / nrec), r = (int)(e - (int64_t)i * nrec);
+  const double* tb = tbv + (int64_t)blockIdx.y * nts * 3;
+  const int* span = tspan + (int64_t)blockIdx.y * nts;
+  // target times whose interval is i-1, i or i+1 (the last one also holds t = T)
+  int s0, s1;
+  if (jt_star >= c.jt) {
+    const int gap = 1 << (jt_star - c.jt);
+    s0 = (i - 1) * gap;
+    s1 = (i + 2) * gap;
+  } else {
+    const int m = 1 << (c.jt - jt_star);
+    s0 = (i - 1) / m;
+    s1 = (i + 1) / m + 1;
   }
-}
-
-__global__ void k_adj_scatter(const double* __restrict__ ehat, int nrec, int nt, const RecCorner* __restrict__ rc,
-                              int ncorner, double coef, int64_t nx, double* __restrict__ G) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
-  if (r >= nrec || i >= nt) return;
-  const double v = coef * ehat[(int64_t)i * nrec + r];
-  for (int e = 0; e < ncorner; ++e) {
-    const RecCorner q = rc[(int64_t)r * ncorner + e];
-    if (q.interior >= 0) atomicAdd(&G[(int64_t)i * nx + q.interior], q.w * v);
+  s0 = max(s0, 0);
+  s1 = min(s1, nts - 1);
+  double acc = 0.0;
+#pragma unroll 4
+  for (int s = s0; s <= s1; ++s) {
+    const int t = i + 1 - span[s];
+    if (t >= 0 && t <= 2) acc = fma(tb[s * 3 + t], wm[(int64_t)s * nrec + r], acc);
   }
+  const double v = (double)c.coef * acc;
+  const RecCorner* q = rc + ((int64_t)blockIdx.y * nrec + r) * ncorner;
+  for (int k = 0; k < ncorner; ++k)
+    if (q[k].interior >= 0) atomicAdd(&c.G[(int64_t)i * c.nx + q[k].interior], q[k].w * v);
 }
 
 // One thread per cell of the level: g_e = -sum_i L_i|_e^T K_ref Z_i|_e with
 // Z_i = sum_j B[i][j] U_j, then P^T onto the parameter nodes.
+// Time rows are split over blockIdx.y (a few cells with many rows would
+// otherwise be one long serial walk); the five rows of U that a row reaches
+// roll through registers.
 template <int D>
 __global__ void __launch_bounds__(kBlock) k_grad_c2(Geo g, double lo0, double lo1, double lo2, double h0, double h1,
-                                                    double h2, int nt, const double* __restrict__ Bband,
+                                                    double h2, int nt, int chunk, const double* __restrict__ Bband,
                                                     const double* __restrict__ U, const double* __restrict__ L,
                                                     ElemK ke, ParamGrid pg, double* __restrict__ dc2) {
   constexpr int NC = 1 << D;
@@ -1654,19 +1687,35 @@ __global__ void __launch_bounds__(kBlock) k_grad_c2(Geo g, double lo0, double lo
     node[c] = in ? idx : -1;
   }
   const int64_t nx = g.nnodes;
-  double acc = 0.0;
-  for (int i = 0; i < nt; ++i) {
-    double Z[NC], Lv[NC];
+  const int i0 = blockIdx.y * chunk, i1 = min(nt, i0 + chunk);
+  double w[5][NC];  // rows i-2 .. i+2 of U
+#pragma unroll
+  for (int t = 0; t < 5; ++t)
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      double z = 0.0;
-      if (node[c] >= 0)
-        for (int t = -2; t <= 2; ++t) {
-          const int j = i + t;
-          if (j >= 0 && j < nt) z = fma(Bband[i * 5 + t + 2], U[(int64_t)j * nx + node[c]], z);
-        }
-      Z[c] = z;
+      const int j = i0 - 3 + t;  // shifted by one: the loop advances the window first
+      w[t][c] = (t > 0 && j >= 0 && j < nt && node[c] >= 0) ? U[(int64_t)j * nx + node[c]] : 0.0;
+    }
+  double acc = 0.0;
+  for (int i = i0; i < i1; ++i) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) w[t][c] = w[t + 1][c];
+    double Lv[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      w[4][c] = (i + 2 < nt && node[c] >= 0) ? U[(int64_t)(i + 2) * nx + node[c]] : 0.0;
       Lv[c] = node[c] >= 0 ? L[(int64_t)i * nx + node[c]] : 0.0;
+    }
+    double Z[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) Z[c] = 0.0;
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+      const double bt = Bband[i * 5 + t];  // zero beyond the matrix
+#pragma unroll
+      for (int c = 0; c < NC; ++c) Z[c] = fma(bt, w[t][c], Z[c]);
     }
 #pragma unroll
     for (int p = 0; p < NC; ++p) {
@@ -1684,12 +1733,20 @@ __global__ void __launch_bounds__(kBlock) k_grad_c2(Geo g, double lo0, double lo
   for (int c = 0; c < NC; ++c) atomicAdd(&dc2[pn[c]], -acc * pw[c]);
 }
 
+// v[a] = sum_i b[i] L_i[a]: 32 nodes per CTA, the rows split over its warps.
 __global__ void __launch_bounds__(kBlock) k_grad_g_v(int nt, int64_t nx, const double* __restrict__ b,
                                                      const double* __restrict__ L, double* __restrict__ v) {
-  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= nx) return;
+  __shared__ double part[kBlock / 32][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t a = (int64_t)blockIdx.x * 32 + lane;
   double acc = 0.0;
-  for (int i = 0; i < nt; ++i) acc = fma(b[i], L[(int64_t)i * nx + a], acc);
+  if (a < nx)
+    for (int i = warp; i < nt; i += kBlock / 32) acc = fma(b[i], L[(int64_t)i * nx + a], acc);
+  part[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || a >= nx) return;
+#pragma unroll
+  for (int w = 1; w < kBlock / 32; ++w) acc += part[w][lane];
   v[a] = acc;
 }
 
@@ -2139,41 +2196,54 @@ template <typename R> void launch_identity(cx<R>* I, int64_t n, cudaStream_t s) 
   k_identity<R><<<blocks_for(n * n), kBlock, 0, s>>>(I, n);
 }
 
+int receiver_group(int64_t n, int ncomp) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(ncomp, ((int64_t)1 << 23) / n));
+}
+
 void launch_receiver_eval(const CombComp* comps, int ncomp, const RecCorner* rc, int nrec, int ncorner,
-                          const double* tbv, const int* tspan, int nts, double* out, cudaStream_t s) {
-  count(1);
-  k_receiver_eval<<<dim3((nrec + kBlock - 1) / kBlock, nts), kBlock, 0, s>>>(comps, ncomp, rc, nrec, ncorner, tbv,
-                                                                             tspan, nts, out);
+                          const double* tbv, const int* tspan, int nts, double* part, double* out, cudaStream_t s) {
+  const int64_t n = (int64_t)nts * nrec;
+  const int grp = receiver_group(n, ncomp);
+  for (int c0 = 0; c0 < ncomp; c0 += grp) {
+    const int nc = std::min(grp, ncomp - c0);
+    count(2);
+    k_receiver_eval<<<dim3(blocks_for(n), 1, nc), kBlock, 0, s>>>(comps, rc, nrec, ncorner, tbv, tspan, nts, c0, part);
+    k_receiver_sum<<<blocks_for(n), kBlock, 0, s>>>(comps, c0, nc, part, n, out);
+  }
 }
 
 void launch_misfit(const double* vals, const double* dobs, int nts, int nrec, double T, double* wm, double* Jout,
                    cudaStream_t s) {
   count(1);
-  k_misfit<<<1, kBlock, 0, s>>>(vals, dobs, nts, nrec, T, wm, Jout);
+  k_misfit<<<1, 1024, 0, s>>>(vals, dobs, nts, nrec, T, wm, Jout);
 }
 
-void launch_adjoint_rhs(const double* wm, int nts, int nrec, const double* tb, const int* tspan, int nt,
-                        const RecCorner* rc, int ncorner, double coef, int64_t nx, double* ehat, double* G,
+void launch_adjoint_rhs(const double* wm, int nts, int jt_star, int nrec, const AdjComp* comps, int ncomp,
+                        int max_nt, const double* tbv, const int* tspan, const RecCorner* rc, int ncorner,
                         cudaStream_t s) {
-  count(2);
-  k_adj_time_project<<<(nrec + 63) / 64, 64, 0, s>>>(wm, nts, nrec, tb, tspan, nt, ehat);
-  k_adj_scatter<<<dim3((nrec + 63) / 64, nt), 64, 0, s>>>(ehat, nrec, nt, rc, ncorner, coef, nx, G);
+  count(1);
+  k_adj_rhs<<<dim3(blocks_for((int64_t)max_nt * nrec), ncomp), kBlock, 0, s>>>(wm, nts, jt_star, nrec, comps, tbv,
+                                                                             tspan, rc, ncorner);
 }
 
 void launch_grad_c2(const Geo& g, const double* lo, int nt, const double* Bband, const double* U, const double* L,
                     const ElemK& ke, const ParamGrid& pg, double* dc2, cudaStream_t s) {
   count(1);
   const double h0 = pg.h[0] * pg.Np / g.N, h1 = pg.h[1] * pg.Np / g.N, h2 = pg.h[2] * pg.Np / g.N;
-  const unsigned grid = blocks_for(g.ncells);
-  if (g.d == 1) k_grad_c2<1><<<grid, kBlock, 0, s>>>(g, lo[0], lo[1], lo[2], h0, h1, h2, nt, Bband, U, L, ke, pg, dc2);
-  else if (g.d == 2) k_grad_c2<2><<<grid, kBlock, 0, s>>>(g, lo[0], lo[1], lo[2], h0, h1, h2, nt, Bband, U, L, ke, pg, dc2);
-  else k_grad_c2<3><<<grid, kBlock, 0, s>>>(g, lo[0], lo[1], lo[2], h0, h1, h2, nt, Bband, U, L, ke, pg, dc2);
+  // time chunks: about four CTAs per SM in all, at least four rows each
+  const unsigned bx = blocks_for(g.ncells);
+  const int nch = (int)std::min<int64_t>((nt + 3) / 4, std::max<int64_t>(1, 608 / (int64_t)bx));
+  const int chunk = (nt + nch - 1) / nch;
+  const dim3 grid(bx, (nt + chunk - 1) / chunk);
+  if (g.d == 1) k_grad_c2<1><<<grid, kBlock, 0, s>>>(g, lo[0], lo[1], lo[2], h0, h1, h2, nt, chunk, Bband, U, L, ke, pg, dc2);
+  else if (g.d == 2) k_grad_c2<2><<<grid, kBlock, 0, s>>>(g, lo[0], lo[1], lo[2], h0, h1, h2, nt, chunk, Bband, U, L, ke, pg, dc2);
+  else k_grad_c2<3><<<grid, kBlock, 0, s>>>(g, lo[0], lo[1], lo[2], h0, h1, h2, nt, chunk, Bband, U, L, ke, pg, dc2);
 }
 
 void launch_grad_g(const Geo& g, const double* lo, const StencilCoef& sc, int nt, const double* b, const double* L,
                    double* v, const ParamGrid& pg, double* dg, cudaStream_t s) {
   count(2);
-  k_grad_g_v<<<blocks_for(g.nnodes), kBlock, 0, s>>>(nt, g.nnodes, b, L, v);
+  k_grad_g_v<<<blocks_for(g.nnodes, 32), kBlock, 0, s>>>(nt, g.nnodes, b, L, v);
   const double h0 = pg.h[0] * pg.Np / g.N, h1 = pg.h[1] * pg.Np / g.N, h2 = pg.h[2] * pg.Np / g.N;
   int64_t nall = 1;
   for (int k = 0; k < g.d; ++k) nall *= (g.N + 1);

@@ -196,15 +196,23 @@ struct RecCorner {
 struct ElemK {
   double k[64];
 };
-// out[s][r] = sum_c coef_c u_c(x_r, t_s) for all target times s (nts) and receivers r.
+// out[s][r] = sum_c coef_c u_c(x_r, t_s) for all target times s (nts) and
+// receivers r; part: scratch of receiver_group(nts x nrec, ncomp) x nts x nrec
+// doubles (at most 64 MB, or one component's values where those are more).
+int receiver_group(int64_t n, int ncomp);
 void launch_receiver_eval(const CombComp* comps, int ncomp, const RecCorner* rc, int nrec, int ncorner,
-                          const double* tbv, const int* tspan, int nts, double* out, cudaStream_t s);
+                          const double* tbv, const int* tspan, int nts, double* part, double* out, cudaStream_t s);
 // wm[s][r] = w_s (vals - dobs)[s][r] with trapezoid weights on [0, T]; J = 1/2 sum w_s e^2 -> Jout[0].
 void launch_misfit(const double* vals, const double* dobs, int nts, int nrec, double T, double* wm, double* Jout,
                    cudaStream_t s);
-// G (nt x nx) += coef sum_s sum_r psi_i(t_s) phi_a(x_r) wm[s][r] for one component (G zeroed by the caller).
-void launch_adjoint_rhs(const double* wm, int nts, int nrec, const double* tb, const int* tspan, int nt,
-                        const RecCorner* rc, int ncorner, double coef, int64_t nx, double* ehat, double* G,
+// G_c (nt x nx) += coef sum_s sum_r psi_i(t_s) phi_a(x_r) wm[s][r] for every component c (G zeroed by the caller).
+struct AdjComp {
+  double* G;
+  int64_t nx;
+  int jt, coef;
+};
+void launch_adjoint_rhs(const double* wm, int nts, int jt_star, int nrec, const AdjComp* comps, int ncomp,
+                        int max_nt, const double* tbv, const int* tspan, const RecCorner* rc, int ncorner,
                         cudaStream_t s);
 // dc2 (param nodes) += P^T g with g_e = -sum_ij B[i][j] L_i^T K_e U_j per cell e of the level.
 void launch_grad_c2(const Geo& g, const double* lo, int nt, const double* Bband, const double* U, const double* L,

@@ -248,6 +248,7 @@ struct Component {
   // adjoint state (receiver misfit gradient): right-hand side and solution, n_t x n_x
   double* Gadj = nullptr;
   double* Lam = nullptr;
+  double* gv = nullptr;  // n_x: the time-summed adjoint of the source gradient
   bool adj_solved = false;
   double Snorm = 0.0;  // upper bound of ||A (x) M + B (x) K||_2
   st_solve_info info{};
@@ -346,8 +347,9 @@ struct st_handle {
     double* vals = nullptr;       // nts x nrec
     double* wm = nullptr;         // weighted misfit, nts x nrec
     double* J = nullptr;          // 1
-    double* ehat = nullptr;       // max nt x nrec
-    double* gv = nullptr;         // max nx
+    double* part = nullptr;       // receiver values of a group of components
+    AdjComp* adj = nullptr;       // adjoint right-hand sides, in component order (first gradient)
+    int max_nt = 1;
   } rec;
 
   // Optional per-kernel-class timing: CUDA events recorded on the handle's
@@ -1910,9 +1912,9 @@ st_status build_receivers(st_handle* h, int jt_star, const double* x, int nrec) 
   R.vals = h->alloc<double>((size_t)nts * nrec);
   R.wm = h->alloc<double>((size_t)nts * nrec);
   R.J = h->alloc<double>(1);
-  R.ehat = h->alloc<double>((size_t)max_nt * nrec);
-  R.gv = h->alloc<double>((size_t)max_nx);
-  if (!R.comps || !R.rc || !R.tb || !R.span || !R.vals || !R.wm || !R.J || !R.ehat || !R.gv)
+  R.part = h->alloc<double>((size_t)receiver_group((int64_t)nts * nrec, ncomp) * nts * nrec);
+  R.max_nt = max_nt;
+  if (!R.comps || !R.rc || !R.tb || !R.span || !R.vals || !R.wm || !R.J || !R.part)
     return fail(h, ST_ERR_OOM, "device allocation failed");
   R.jt = jt_star;
   R.nrec = nrec;
@@ -2696,7 +2698,7 @@ st_status st_receiver_values(st_handle* h, int jt_star, const double* x_rec, int
   st_status s = build_receivers(h, jt_star, x_rec, n_rec);
   if (s != ST_OK) return s;
   const st_handle::RecTables& R = h->rec;
-  launch_receiver_eval(R.comps, (int)h->comps.size(), R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, out_dev, h->stream);
+  launch_receiver_eval(R.comps, (int)h->comps.size(), R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.part, out_dev, h->stream);
   return check_launch(h, "receiver values");
 }
 
@@ -2715,9 +2717,9 @@ st_status st_misfit_gradient(st_handle* h, int jt_star, const double* x_rec, int
     if (!c->solved) return fail(h, ST_ERR_STATE, "gradient before every component is solved");
   st_status s = build_receivers(h, jt_star, x_rec, n_rec);
   if (s != ST_OK) return s;
-  const st_handle::RecTables& R = h->rec;
+  st_handle::RecTables& R = h->rec;
   const int ncomp = (int)h->comps.size();
-  launch_receiver_eval(R.comps, ncomp, R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.vals, h->stream);
+  launch_receiver_eval(R.comps, ncomp, R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.part, R.vals, h->stream);
   launch_misfit(R.vals, d_obs_dev, R.nts, n_rec, p.T, R.wm, R.J, h->stream);
   // adjoint right-hand sides G_k = coef_k E_k^T (w * e)
   for (int c = 0; c < ncomp; ++c) {
@@ -2726,13 +2728,22 @@ st_status st_misfit_gradient(st_handle* h, int jt_star, const double* x_rec, int
     if (k.Gadj == nullptr) {
       k.Gadj = h->alloc<double>(n);
       k.Lam = h->alloc<double>(n);
-      if (!k.Gadj || !k.Lam) return fail(h, ST_ERR_OOM, "device allocation failed");
+      k.gv = h->alloc<double>((size_t)k.nx);
+      if (!k.Gadj || !k.Lam || !k.gv) return fail(h, ST_ERR_OOM, "device allocation failed");
     }
     ST_CUDA(h, cudaMemsetAsync(k.Gadj, 0, n * sizeof(double), h->stream));
-    launch_adjoint_rhs(R.wm, R.nts, n_rec, R.tb + (size_t)c * R.nts * 3, R.span + (size_t)c * R.nts, k.nt,
-                       R.rc + (size_t)c * n_rec * R.ncorner, R.ncorner, (double)k.coef, k.nx, R.ehat, k.Gadj,
-                       h->stream);
   }
+  if (R.adj == nullptr) {
+    std::vector<AdjComp> ac(ncomp);
+    for (int c = 0; c < ncomp; ++c) {
+      const Component& k = *h->comps[c];
+      ac[c] = AdjComp{k.Gadj, k.nx, k.jt, k.coef};
+    }
+    R.adj = h->upload(ac);
+    ST_NEED(h, R.adj);
+    ST_CUDA(h, cudaStreamSynchronize(h->stream));  // the host table goes out of scope
+  }
+  launch_adjoint_rhs(R.wm, R.nts, jt_star, n_rec, R.adj, ncomp, R.max_nt, R.tb, R.span, R.rc, R.ncorner, h->stream);
   if ((s = check_launch(h, "adjoint right-hand sides")) != ST_OK) return s;
   // adjoint solves S_k^T L_k = G_k, all components concurrently
   s = run_solves(h, 0, ncomp, true, info);
@@ -2749,12 +2760,17 @@ st_status st_misfit_gradient(st_handle* h, int jt_star, const double* x_rec, int
   for (int k = 0; k < p.d; ++k) np *= (pg.Np + 1);
   ST_CUDA(h, cudaMemsetAsync(dc2_dev, 0, np * sizeof(double), h->stream));
   ST_CUDA(h, cudaMemsetAsync(dg_dev, 0, np * sizeof(double), h->stream));
+  // every component's reductions on its own stream, after the zeroing above
+  ST_CUDA(h, cudaEventRecord(h->entry_ev, h->stream));
   for (int c = 0; c < ncomp; ++c) {
     Component& k = *h->comps[c];
     const ElemK ke = element_stiffness(p.d, k.sl->h);
-    launch_grad_c2(k.sl->geo, pg.lo, k.nt, k.td->Bband, k.U, k.Lam, ke, pg, dc2_dev, h->stream);
+    ST_CUDA(h, cudaStreamWaitEvent(k.cs, h->entry_ev, 0));
+    launch_grad_c2(k.sl->geo, pg.lo, k.nt, k.td->Bband, k.U, k.Lam, ke, pg, dc2_dev, k.cs);
     if (p.n_terms >= 1)
-      launch_grad_g(k.sl->geo, pg.lo, k.sl->sc, k.nt, k.td->rhs_coef, k.Lam, R.gv, pg, dg_dev, h->stream);
+      launch_grad_g(k.sl->geo, pg.lo, k.sl->sc, k.nt, k.td->rhs_coef, k.Lam, k.gv, pg, dg_dev, k.cs);
+    ST_CUDA(h, cudaEventRecord(k.done, k.cs));
+    ST_CUDA(h, cudaStreamWaitEvent(h->stream, k.done, 0));
   }
   ST_CUDA(h, cudaMemcpyAsync(h->scalar_h, R.J, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   ST_CUDA(h, cudaStreamSynchronize(h->stream));
