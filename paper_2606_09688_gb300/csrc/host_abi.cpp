@@ -43,7 +43,7 @@ st_status st_host_time_eig(int jt, double T, int* nsel, double* lam, double* con
   TimeLevel tl;
   build_time_level(jt, T, tl);
   TimeEig e;
-  if (!time_eig(tl, e)) return ST_ERR_NUMERIC;
+  if (!time_eig(tl, e, true)) return ST_ERR_NUMERIC;
   *nsel = e.nsel;
   for (int q = 0; q < e.nsel; ++q) {
     lam[2 * q] = e.lam[q].real();
@@ -59,7 +59,7 @@ st_status st_host_time_eig_p(int jt, double T, int p, int* nsel, double* lam, do
   TimeLevel tl;
   build_time_level_p(jt, T, p, tl);
   TimeEig e;
-  if (!time_eig(tl, e)) return ST_ERR_NUMERIC;
+  if (!time_eig(tl, e, true)) return ST_ERR_NUMERIC;
   *nsel = e.nsel;
   for (int q = 0; q < e.nsel; ++q) {
     lam[2 * q] = e.lam[q].real();

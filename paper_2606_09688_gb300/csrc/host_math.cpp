@@ -214,13 +214,27 @@ bool lu_solve_real(int n, std::vector<double> A, std::vector<double>& Bm, int nr
       for (int j = 0; j < nrhs; ++j) Bm[(size_t)i * nrhs + j] -= l * Bm[(size_t)k * nrhs + j];
     }
   }
-  for (int k = n - 1; k >= 0; --k)
-    for (int j = 0; j < nrhs; ++j) {
-      double s = Bm[(size_t)k * nrhs + j];
-      for (int i = k + 1; i < n; ++i) s -= A[(size_t)k * n + i] * Bm[(size_t)i * nrhs + j];
-      Bm[(size_t)k * nrhs + j] = s / A[(size_t)k * n + k];
+  for (int k = n - 1; k >= 0; --k) {
+    for (int i = k + 1; i < n; ++i) {
+      const double a = A[(size_t)k * n + i];
+      if (a == 0.0) continue;
+      for (int j = 0; j < nrhs; ++j) Bm[(size_t)k * nrhs + j] -= a * Bm[(size_t)i * nrhs + j];
     }
+    for (int j = 0; j < nrhs; ++j) Bm[(size_t)k * nrhs + j] /= A[(size_t)k * n + k];
+  }
   return true;
+}
+
+// y -= l x on n consecutive complex numbers.
+static void sub_scaled(int n, cplx l, const cplx* x, cplx* y) {
+  const double lr = l.real(), li = l.imag();
+  const double* a = reinterpret_cast<const double*>(x);
+  double* b = reinterpret_cast<double*>(y);
+  for (int j = 0; j < 2 * n; j += 2) {
+    const double xr = a[j], xi = a[j + 1];
+    b[j] -= lr * xr - li * xi;
+    b[j + 1] -= lr * xi + li * xr;
+  }
 }
 
 bool lu_inverse_cplx(int n, std::vector<cplx> A, std::vector<cplx>& Ainv) {
@@ -239,16 +253,14 @@ bool lu_inverse_cplx(int n, std::vector<cplx> A, std::vector<cplx>& Ainv) {
     for (int i = k + 1; i < n; ++i) {
       const cplx l = A[(size_t)i * n + k] / A[(size_t)k * n + k];
       if (l == cplx(0.0)) continue;
-      for (int j = k + 1; j < n; ++j) A[(size_t)i * n + j] -= l * A[(size_t)k * n + j];
-      for (int j = 0; j < n; ++j) Ainv[(size_t)i * n + j] -= l * Ainv[(size_t)k * n + j];
+      sub_scaled(n - k - 1, l, &A[(size_t)k * n + k + 1], &A[(size_t)i * n + k + 1]);
+      sub_scaled(n, l, &Ainv[(size_t)k * n], &Ainv[(size_t)i * n]);
     }
   }
-  for (int k = n - 1; k >= 0; --k)
-    for (int j = 0; j < n; ++j) {
-      cplx s = Ainv[(size_t)k * n + j];
-      for (int i = k + 1; i < n; ++i) s -= A[(size_t)k * n + i] * Ainv[(size_t)i * n + j];
-      Ainv[(size_t)k * n + j] = s / A[(size_t)k * n + k];
-    }
+  for (int k = n - 1; k >= 0; --k) {
+    for (int i = k + 1; i < n; ++i) sub_scaled(n, A[(size_t)k * n + i], &Ainv[(size_t)i * n], &Ainv[(size_t)k * n]);
+    for (int j = 0; j < n; ++j) Ainv[(size_t)k * n + j] /= A[(size_t)k * n + k];
+  }
   return true;
 }
 
@@ -312,33 +324,39 @@ bool complex_schur(int n, std::vector<cplx>& H, std::vector<cplx>& Z) {
       givens(h(k, k), h(k + 1, k), c, s);
       cs[k] = c;
       sn[k] = s;
-      for (int j = k; j < n; ++j) {
-        const cplx x = h(k, j), y = h(k + 1, j);
-        h(k, j) = c * x + s * y;
-        h(k + 1, j) = -std::conj(s) * x + c * y;
+      const double sr = s.real(), si = s.imag();
+      double* hx = reinterpret_cast<double*>(&h(k, 0));
+      double* hy = reinterpret_cast<double*>(&h(k + 1, 0));
+      for (int j = 2 * k; j < 2 * n; j += 2) {
+        const double xr = hx[j], xi = hx[j + 1], yr = hy[j], yi = hy[j + 1];
+        hx[j] = c * xr + (sr * yr - si * yi);
+        hx[j + 1] = c * xi + (sr * yi + si * yr);
+        hy[j] = c * yr - (sr * xr + si * xi);
+        hy[j + 1] = c * yi - (sr * xi - si * xr);
       }
     }
-    for (int k = l; k < hi; ++k) {
-      const double c = cs[k];
-      const cplx s = sn[k];
-      const int rmax = std::min(k + 2, hi);
-      for (int i = 0; i <= rmax; ++i) {
-        const cplx x = h(i, k), y = h(i, k + 1);
-        h(i, k) = c * x + std::conj(s) * y;
-        h(i, k + 1) = -s * x + c * y;
+    // the columns of H and Z row by row: row i of H takes the rotations that
+    // reach it (k >= i - 2), every row of Z all of them
+    auto rotate_row = [&](cplx* row, int k0) {
+      double xr = row[k0].real(), xi = row[k0].imag();
+      for (int k = k0; k < hi; ++k) {
+        const double c = cs[k], sr = sn[k].real(), si = sn[k].imag();
+        const double yr = row[k + 1].real(), yi = row[k + 1].imag();
+        row[k] = cplx(c * xr + (sr * yr + si * yi), c * xi + (sr * yi - si * yr));
+        const double zr = (si * xi - sr * xr) + c * yr, zi = c * yi - (sr * xi + si * xr);
+        xr = zr;
+        xi = zi;
       }
-      for (int i = 0; i < n; ++i) {
-        const cplx x = Z[(size_t)i * n + k], y = Z[(size_t)i * n + k + 1];
-        Z[(size_t)i * n + k] = c * x + std::conj(s) * y;
-        Z[(size_t)i * n + k + 1] = -s * x + c * y;
-      }
-    }
+      row[hi] = cplx(xr, xi);
+    };
+    for (int i = 0; i <= hi; ++i) rotate_row(&H[(size_t)i * n], std::max(l, i - 2));
+    for (int i = 0; i < n; ++i) rotate_row(&Z[(size_t)i * n], l);
     for (int k = l; k <= hi; ++k) h(k, k) += mu;
   }
   return true;
 }
 
-bool time_eig(const TimeLevel& tl, TimeEig& out) {
+bool time_eig(const TimeLevel& tl, TimeEig& out, bool diagnose) {
   const int n = tl.nt;
   // C = B^{-1} A
   std::vector<double> C = tl.A;
@@ -346,7 +364,7 @@ bool time_eig(const TimeLevel& tl, TimeEig& out) {
   // Householder reduction to upper Hessenberg form, Q accumulated.
   std::vector<double> Hm = C, Qm((size_t)n * n, 0.0);
   for (int i = 0; i < n; ++i) Qm[(size_t)i * n + i] = 1.0;
-  std::vector<double> v(n);
+  std::vector<double> v(n), sums(n);
   for (int k = 0; k + 2 < n; ++k) {
     double alpha = 0.0;
     for (int i = k + 1; i < n; ++i) alpha += Hm[(size_t)i * n + k] * Hm[(size_t)i * n + k];
@@ -360,12 +378,12 @@ bool time_eig(const TimeLevel& tl, TimeEig& out) {
     for (int i = k + 1; i < n; ++i) vn += v[i] * v[i];
     if (vn == 0.0) continue;
     // H <- (I - 2vv^T/vn) H (I - 2vv^T/vn);  Q <- Q (I - 2vv^T/vn)
-    for (int j = 0; j < n; ++j) {
-      double s = 0.0;
-      for (int i = k + 1; i < n; ++i) s += v[i] * Hm[(size_t)i * n + j];
-      s *= 2.0 / vn;
-      for (int i = k + 1; i < n; ++i) Hm[(size_t)i * n + j] -= s * v[i];
-    }
+    std::fill(sums.begin(), sums.end(), 0.0);
+    for (int i = k + 1; i < n; ++i)
+      for (int j = 0; j < n; ++j) sums[j] += v[i] * Hm[(size_t)i * n + j];
+    for (int j = 0; j < n; ++j) sums[j] *= 2.0 / vn;
+    for (int i = k + 1; i < n; ++i)
+      for (int j = 0; j < n; ++j) Hm[(size_t)i * n + j] -= sums[j] * v[i];
     for (int i = 0; i < n; ++i) {
       double s = 0.0;
       for (int j = k + 1; j < n; ++j) s += Hm[(size_t)i * n + j] * v[j];
@@ -390,16 +408,26 @@ bool time_eig(const TimeLevel& tl, TimeEig& out) {
     std::fill(y.begin(), y.end(), cplx(0.0));
     y[k] = 1.0;
     for (int j = k - 1; j >= 0; --j) {
-      cplx s = 0.0;
-      for (int l = j + 1; l <= k; ++l) s += Hc[(size_t)j * n + l] * y[l];
+      double ar = 0.0, ai = 0.0;
+      for (int l = j + 1; l <= k; ++l) {
+        const cplx t = Hc[(size_t)j * n + l];
+        ar += t.real() * y[l].real() - t.imag() * y[l].imag();
+        ai += t.real() * y[l].imag() + t.imag() * y[l].real();
+      }
+      const cplx s(ar, ai);
       cplx den = Hc[(size_t)j * n + j] - lam[k];
       if (std::abs(den) < 1e-14 * tnorm) den = 1e-14 * tnorm;
       y[j] = -s / den;
     }
     double nrm = 0.0;
     for (int i = 0; i < n; ++i) {
-      cplx s = 0.0;
-      for (int l = 0; l <= k; ++l) s += Zc[(size_t)i * n + l] * y[l];
+      double ar = 0.0, ai = 0.0;
+      for (int l = 0; l <= k; ++l) {
+        const cplx t = Zc[(size_t)i * n + l];
+        ar += t.real() * y[l].real() - t.imag() * y[l].imag();
+        ai += t.real() * y[l].imag() + t.imag() * y[l].real();
+      }
+      const cplx s(ar, ai);
       Vall[(size_t)i * n + k] = s;
       nrm += std::norm(s);
     }
@@ -468,10 +496,9 @@ bool time_eig(const TimeLevel& tl, TimeEig& out) {
   for (int q = 0; q < out.nsel; ++q) {
     const int cq = col_of[q];
     for (int i = 0; i < n; ++i) out.V[(size_t)i * out.nsel + q] = Vf[(size_t)i * n + cq];
-    for (int j = 0; j < n; ++j) {
-      cplx s = 0.0;
-      for (int l = 0; l < n; ++l) s += Vinv[(size_t)cq * n + l] * Binv[(size_t)l * n + j];
-      out.W[(size_t)q * n + j] = s;
+    for (int l = 0; l < n; ++l) {
+      const cplx v = Vinv[(size_t)cq * n + l];
+      for (int j = 0; j < n; ++j) out.W[(size_t)q * n + j] += v * Binv[(size_t)l * n + j];
     }
   }
   // Diagnostics: 1-norm condition estimate and eigen-residual of the full V.
@@ -486,6 +513,7 @@ bool time_eig(const TimeLevel& tl, TimeEig& out) {
     n1i = std::max(n1i, si);
   }
   out.cond_est = n1 * n1i;
+  if (!diagnose) return true;
   double rr = 0.0, cn = 0.0, vn = 0.0;
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) {

@@ -61,9 +61,9 @@ struct TimeEig {
   std::vector<cplx> W;             // nsel x nt
   std::vector<double> weight;      // 1 (real) or 2 (complex pair)
   double cond_est = 0.0;           // ||V||_1 ||V^{-1}||_1 of the full V
-  double resid = 0.0;              // ||C V - V Lam||_F / (||C||_F ||V||_F)
+  double resid = 0.0;              // ||C V - V Lam||_F / (||C||_F ||V||_F), when asked for
 };
-bool time_eig(const TimeLevel& tl, TimeEig& out);
+bool time_eig(const TimeLevel& tl, TimeEig& out, bool diagnose = false);
 
 // Dense real linear algebra helpers.
 bool lu_solve_real(int n, std::vector<double> A, std::vector<double>& B, int nrhs);  // B <- A^{-1} B

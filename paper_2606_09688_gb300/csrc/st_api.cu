@@ -22,12 +22,14 @@
 #include <cstdlib>
 #include <cstdio>
 #include <cstring>
+#include <future>
 #include <map>
 #include <memory>
 #include <mutex>
 #include <thread>
 #include <tuple>
 #include <string>
+#include <system_error>
 #include <vector>
 
 #include "../../include/st.h"
@@ -376,13 +378,12 @@ struct st_handle {
   }
 
   ~st_handle() {
-    if (scalar_h) cudaFreeHost(scalar_h);
+    if (pinned) cudaFreeHost(pinned);
     for (auto& c : comps) {
+      if (!c) continue;  // set-up ended early
       if (c->g_init) cudaGraphExecDestroy(c->g_init);
       if (c->g_iter) cudaGraphExecDestroy(c->g_iter);
       if (c->g_solve) cudaGraphExecDestroy(c->g_solve);
-      if (c->cscalar_h) cudaFreeHost(c->cscalar_h);
-      if (c->rec_h) cudaFreeHost(c->rec_h);
       if (c->cs) cudaStreamDestroy(c->cs);
       if (c->done) cudaEventDestroy(c->done);
     }
@@ -397,18 +398,51 @@ struct st_handle {
     for (auto e : ev_pool) cudaEventDestroy(e);
   }
 
+  // Device memory of the handle.  Requests of up to a quarter of a block are
+  // cut from blocks of 2 to 32 MB: a handle makes a few hundred of them, and a
+  // cudaMalloc and a cudaFree each cost as much as the set-up kernels of a small
+  // component.  With a memory cap every request is allocated by itself, so that
+  // no more than the cap is ever taken.
   template <typename T> T* alloc(size_t n) {
     std::lock_guard<std::mutex> lock(alloc_mu);
-    void* p = nullptr;
     if (n == 0) n = 1;
-    if (opt.mem_cap_bytes > 0 && mem.bytes + n * sizeof(T) > (size_t)opt.mem_cap_bytes) return nullptr;
-    if (cudaMalloc(&p, n * sizeof(T)) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
+    const size_t want = n * sizeof(T), rounded = (want + 255) & ~(size_t)255;
+    const bool capped = opt.mem_cap_bytes > 0;
+    if (capped && mem.bytes + want > (size_t)opt.mem_cap_bytes) return nullptr;
+    void* p = nullptr;
+    if (!capped && rounded <= block_next / 4) {
+      if (rounded > block_left) {
+        if (cudaMalloc(&p, block_next) != cudaSuccess) {
+          cudaGetLastError();
+          return nullptr;
+        }
+        mem.ptrs.push_back(p);
+        block = static_cast<char*>(p);
+        block_left = block_next;
+        block_next = std::min<size_t>(4 * block_next, (size_t)32 << 20);
+      }
+      p = block;
+      block += rounded;
+      block_left -= rounded;
+    } else {
+      if (cudaMalloc(&p, want) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      mem.ptrs.push_back(p);
     }
-    mem.ptrs.push_back(p);
-    mem.bytes += n * sizeof(T);
+    mem.bytes += want;
     return static_cast<T*>(p);
+  }
+  char* block = nullptr;
+  size_t block_left = 0, block_next = (size_t)2 << 20;
+  // Page-locked words of the components (norms and records read back), one allocation per handle.
+  char* pinned = nullptr;
+  size_t pinned_used = 0;
+  template <typename T> T* pinned_alloc(size_t n) {
+    T* p = reinterpret_cast<T*>(pinned + pinned_used);
+    pinned_used += (n * sizeof(T) + 63) & ~(size_t)63;
+    return p;
   }
   template <typename T> T* upload(const std::vector<T>& v) {
     T* p = alloc<T>(v.size());
@@ -1628,7 +1662,7 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
   c.fn2 = h->alloc<double>(1);
   ST_NEED(h, c.rec);
   ST_NEED(h, c.fn2);
-  ST_CUDA(h, cudaMallocHost(&c.rec_h, sizeof(RefineRec)));
+  c.rec_h = h->pinned_alloc<RefineRec>(1);
   int prio_lo = 0, prio_hi = 0;
   ST_CUDA(h, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
   cudaGraph_t g = nullptr, sweep = nullptr, inner = nullptr;
@@ -1777,7 +1811,7 @@ st_status setup_context(st_handle* h, Component& c) {
   ST_NEED(h, c.cdone);
   ST_CUDA(h, cudaMemsetAsync(c.cdone, 0, sizeof(unsigned), h->stream));
   ST_CUDA(h, cudaMemsetAsync(c.cerr, 0, sizeof(int), h->stream));
-  ST_CUDA(h, cudaMallocHost(&c.cscalar_h, 3 * sizeof(double)));
+  c.cscalar_h = h->pinned_alloc<double>(3);
   if (c.method == 0) {
     st_status s = c.inner64 ? prepare_work<double>(h, c) : prepare_work<float>(h, c);
     if (s != ST_OK) return s;
@@ -1863,12 +1897,10 @@ st_status build_receivers(st_handle* h, int jt_star, const double* x, int nrec) 
   std::vector<RecCorner> rc((size_t)ncomp * nrec * nc);
   std::vector<double> tb((size_t)ncomp * nts * 3);
   std::vector<int> sp((size_t)ncomp * nts);
-  int64_t max_nx = 1;
   int max_nt = 1;
   for (int c = 0; c < ncomp; ++c) {
     const Component& k = *h->comps[c];
     cc[c] = CombComp{k.U, k.sl->lift, k.jx, k.jt, k.coef, 0};
-    max_nx = std::max(max_nx, k.nx);
     max_nt = std::max(max_nt, k.nt);
     const int N = 1 << k.jx, n = N - 1;
     for (int r = 0; r < nrec; ++r) {
@@ -2280,10 +2312,12 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
     g_create_error = "event creation failed";
     return ST_ERR_CUDA;
   }
-  if (cudaMallocHost(&hp->scalar_h, sizeof(double)) != cudaSuccess) {
+  static_assert(sizeof(RefineRec) <= 64, "one 64-byte slot per record");
+  if (cudaMallocHost(&hp->pinned, 64 * (size_t)(1 + 2 * (2 * p.J + 1))) != cudaSuccess) {
     g_create_error = "pinned allocation failed";
     return ST_ERR_CUDA;
   }
+  hp->scalar_h = hp->pinned_alloc<double>(1);
   // Components of Eq. (19)
   std::vector<std::tuple<int, int, int>> cl;
   {
@@ -2291,7 +2325,38 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
     st_host_components(p.J, p.mx, p.mt, lst.data());
     for (int k = 0; k < 2 * p.J + 1; ++k) cl.emplace_back(lst[3 * k], lst[3 * k + 1], lst[3 * k + 2]);
   }
+  // The time eigenbases (host, 0.1 to 10 ms each) are computed on threads of
+  // their own while the spatial levels are sampled and uploaded.
+  auto space_method = [&](int jx, int jt) {
+    return (1 << jt) + 1 > kModeTMaxNt && make_geo(p.d, jx).nnodes <= kModeSMaxNx;
+  };
+  std::map<int, std::future<std::unique_ptr<TimeEig>>> eigs;
   for (auto& t : cl) {
+    const int jx = std::get<0>(t), jt = std::get<1>(t);
+    if (space_method(jx, jt) || eigs.count(jt)) continue;
+    const double T = p.T;
+    auto job = [jt, T]() -> std::unique_ptr<TimeEig> {
+      TimeLevel tl;
+      build_time_level(jt, T, tl);
+      auto e = std::make_unique<TimeEig>();
+      if (!time_eig(tl, *e)) e.reset();
+      return e;
+    };
+    try {
+      eigs[jt] = std::async(std::launch::async, job);
+    } catch (const std::system_error&) {  // no thread to be had
+      eigs[jt] = std::async(std::launch::deferred, job);
+    }
+  }
+  // components with few time levels first: their set-up overlaps the largest
+  // eigenbasis, which takes longest
+  std::vector<int> sorder(cl.size());
+  for (size_t k = 0; k < cl.size(); ++k) sorder[k] = (int)k;
+  std::stable_sort(sorder.begin(), sorder.end(),
+                   [&](int a, int b) { return std::get<1>(cl[a]) < std::get<1>(cl[b]); });
+  hp->comps.resize(cl.size());
+  for (int kc : sorder) {
+    const std::tuple<int, int, int>& t = cl[kc];
     const int jx = std::get<0>(t), jt = std::get<1>(t);
     if (!hp->space.count(jx)) {
       auto sl = std::make_unique<SpaceLevel>();
@@ -2303,9 +2368,7 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
       hp->space[jx] = std::move(sl);
       trace.mark("space levels");
     }
-    const int nt = (1 << jt) + 1;
-    const int64_t nx = make_geo(p.d, jx).nnodes;
-    const bool space_eig = nt > kModeTMaxNt && nx <= kModeSMaxNx;
+    const bool space_eig = space_method(jx, jt);
     if (!hp->time.count(jt)) {
       auto td = std::make_unique<TimeData>();
       st_status s = setup_time_level(hp, jt, *td);
@@ -2318,10 +2381,12 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
     }
     TimeData& td = *hp->time[jt];
     if (!space_eig && !td.have_eig) {
-      if (!time_eig(td.tl, td.eig)) {
+      const std::unique_ptr<TimeEig> e = eigs[jt].get();
+      if (!e) {
         g_create_error = "eigen-decomposition of the time matrices failed";
         return ST_ERR_NUMERIC;
       }
+      td.eig = std::move(*e);
       td.have_eig = true;
       // upload
       const int ns = td.eig.nsel, ntt = td.tl.nt;
@@ -2376,10 +2441,10 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
     trace.mark("component context");
     if (s != ST_OK) {
       g_create_error = hp->err;
-      hp->comps.push_back(std::move(c));  // released with the handle
+      hp->comps[kc] = std::move(c);  // released with the handle
       return s;
     }
-    hp->comps.push_back(std::move(c));
+    hp->comps[kc] = std::move(c);
   }
   if (cudaStreamSynchronize(hp->stream) != cudaSuccess) {
     g_create_error = "stream synchronisation failed during setup";
