@@ -62,8 +62,13 @@ constexpr int kMaxDirectRows = 32768;  // grids up to this size are solved direc
 // by 0.24 s for 12 ms a solve (255^2: 0.03 s for 11 ms); 511^2 FP32 5.3 -> 4.5 ms
 // alone (four sweeps in place of three) and nothing for the whole step.
 constexpr double kDirectFactorFlops = 2.5e10;
-constexpr int64_t kCoarseFloor = 1024;     // multigrid coarsening stops at the largest grid of at most this size
-constexpr int64_t kMaxDenseCoarse = 4096;  // coarsest multigrid grids up to this size use an explicit inverse
+// Multigrid coarsening stops at the largest grid of at most this size: 2D 127^2,
+// solved by nested dissection (n = 12 step, down to 31^2 with its explicit inverse
+// -> 127^2: FP64 41.4 -> 38.2 ms, FP32 19.0 -> 18.2 ms: 12 against 14 iterations and
+// three levels of launches fewer; 63^2 54 / 21 ms with an explicit inverse, 255^2
+// 41.5 / 19.9 ms); 1D and 3D 1024.
+constexpr int64_t kCoarseFloor = 1024, kCoarseFloor2D = 16384;
+constexpr int64_t kMaxDenseCoarse = 1024;  // coarsest multigrid grids up to this size use an explicit inverse
 constexpr int kMaxBandWidth = 1024;    // widest band the warp solve supports
 constexpr int kMaxCoarseBand = 256;    // widest band of a multigrid coarsest grid
 constexpr int64_t kMaxCoarseRows = 32768;  // largest multigrid coarsest grid
@@ -71,8 +76,25 @@ constexpr int kModeSMaxNx = 1024;      // dense spatial eigenbasis limit
 constexpr int kModeTMaxNt = 129;       // time eigenbasis used up to this many time unknowns
 constexpr double kKappaFP32 = 2.0e5;   // cond(V) above which inner solves stay in FP64
 constexpr double kThetaMG = 1.25;      // coarsest-grid resolution: k h_c <= theta
-constexpr double kShiftMG = 0.5;       // imaginary shift (x |Re lam|) of modes the coarsest grid cannot resolve
-constexpr double kOmega2D = 0.6, kOmega3D = 0.55, kOmega1D = 0.6;
+// Smoother weights and the imaginary shift (x |Re lam|) of modes the coarsest grid
+// cannot resolve.  The Q1 stencil's symbol over its diagonal takes the values
+// [1, 2] (1D), [3/4, 3/2] (2D) and [1/2, 3/2] (3D) on the frequencies that the
+// coarse grid does not hold.  One Jacobi sweep (FP64): near 2 / (min + max), the
+// minimiser of the largest damping factor there.  Two sweeps (FP32): the roots of
+// the Chebyshev polynomial of that interval, mirrored after the coarse correction
+// (in 3D the larger root is cut to 1.2).  Against the single weight 0.6 (3D 0.55):
+// 2D n = 12 FP64 44 -> 41.4 ms, FP32 20.3 -> 19.0 ms a step; 3D n = 10 101 -> 94 ms; and
+// with the shift 0.2 in place of 0.5 3D 94 -> 78.7 ms (63^3 x 17 rows: 30 -> 19
+// iterations; 0.1 21, 0.3 23).  Beyond k h_c = kKappaWeak the indefinite part of the
+// spectrum that these weights amplify wins (3D 63^3 x 33 rows, k h_c = 4.8, FP32: no
+// convergence, against 88 iterations), so such components keep the damped
+// weights and the larger shift.
+struct Smoother {
+  double w64[3], w32[3][2], shift;
+};
+constexpr Smoother kSmooth = {{0.667, 0.85, 0.9}, {{0.54, 0.872}, {0.72, 1.163}, {0.7, 1.2}}, 0.2};
+constexpr Smoother kSmoothWeak = {{0.6, 0.6, 0.55}, {{0.6, 0.6}, {0.6, 0.6}, {0.55, 0.55}}, 0.5};
+constexpr double kKappaWeak = 2.5;
 constexpr int kIterPerGraph = 4;  // COCG iterations between host convergence checks
 
 struct DevMem {
@@ -244,6 +266,7 @@ struct Component {
   cx<double>* lamP64 = nullptr;
   cx<float>* lamP32 = nullptr;
   int nshifted = 0;
+  const Smoother* smooth = &kSmooth;
   double* abT = nullptr;  // LU of (A + mu B)^T per spatial mode (adjoint systems)
   int* pivT = nullptr;
   int kl = 2, ku = 2;
@@ -782,11 +805,11 @@ int choose_coarse(const st_problem& p, const Component& c, int64_t max_direct) {
     kmax = std::max(kmax, std::sqrt(std::max(0.0, -c.td->eig.lam[q].real()) / c.sl->c2min));
   double L = 0.0;
   for (int k = 0; k < p.d; ++k) L = std::max(L, p.hi[k] - p.lo[k]);
-  // no coarser than the largest grid of at most kCoarseFloor nodes (its
-  // explicit inverse is cheap): below it, extra levels only add launches to
-  // every V-cycle
+  // no coarser than the largest grid of at most kCoarseFloor nodes: below it,
+  // extra levels only add launches to every V-cycle
   int jc = 2;
-  while (jc + 1 < c.jx && make_geo(p.d, jc + 1).nnodes <= kCoarseFloor) ++jc;
+  const int64_t floor = p.d == 2 ? kCoarseFloor2D : kCoarseFloor;
+  while (jc + 1 < c.jx && make_geo(p.d, jc + 1).nnodes <= floor) ++jc;
   while (jc < c.jx && kmax * L / (1 << jc) > kThetaMG) ++jc;
   auto fits = [&](int j) {
     const Geo g = make_geo(p.d, j);
@@ -1001,12 +1024,16 @@ st_status setup_component(st_handle* h, Component& c) {
     std::vector<cx<double>> lp(c.nsel);
     std::vector<cx<float>> lpf(c.nsel);
     c.nshifted = 0;
+    double kmax = 0.0;
+    for (int q = 0; q < c.nsel; ++q)
+      kmax = std::max(kmax, std::sqrt(std::max(0.0, -c.td->eig.lam[q].real()) / c.sl->c2min));
+    c.smooth = kmax * hc > kKappaWeak ? &kSmoothWeak : &kSmooth;
     for (int q = 0; q < c.nsel; ++q) {
       const std::complex<double> l = c.td->eig.lam[q];
       double im = l.imag();
       const double kq = std::sqrt(std::max(0.0, -l.real()) / c.sl->c2min);
       if (!c.direct && kq * hc > kThetaMG) {
-        im += (im >= 0.0 ? 1.0 : -1.0) * kShiftMG * std::fabs(l.real());
+        im += (im >= 0.0 ? 1.0 : -1.0) * c.smooth->shift * std::fabs(l.real());
         ++c.nshifted;
       }
       lp[q] = mk(l.real(), im);
@@ -1082,8 +1109,6 @@ st_status ccheck(Component& c, const char* where) {
 // the handle's stream), so that those of different components overlap with
 // each other and with the host work of the components set up after it; the
 // zero-pivot flag they leave in c.cerr is read at the end of st_setup.
-double omega_of(int d);
-
 template <typename R> st_status prepare_work(st_handle* h, Component& c) {
   Work<R>& w = work_of<R>(c);
   if (w.ready) return ST_OK;
@@ -1158,7 +1183,7 @@ template <typename R> st_status prepare_work(st_handle* h, Component& c) {
       MGLevel& lv = c.mg[l];
       cx<R>* dv = h->alloc<cx<R>>((size_t)c.nsel * lv.geo.nnodes);
       ST_NEED(h, dv);
-      launch_jacobi_dinv<R>(lv.geo, lv.sc, lv.c2d, c.lamP64, omega_of(lv.geo.d), c.nsel, lv.geo.nnodes, dv, c.cs);
+      launch_jacobi_dinv<R>(lv.geo, lv.sc, lv.c2d, c.lamP64, c.smooth->w64[lv.geo.d - 1], c.nsel, lv.geo.nnodes, dv, c.cs);
       lv.sc.dinv = dv;
     }
   }
@@ -1208,8 +1233,6 @@ double direct_bytes(const Component& c, double cs) {
   return (c.nd != nullptr ? c.nd->solve_flops / 8.0 : 2.0 * c.nrowc * c.bl.ld) * cs + 3.0 * c.nrowc * cs;
 }
 
-double omega_of(int d) { return d == 1 ? kOmega1D : (d == 2 ? kOmega2D : kOmega3D); }
-
 // x = B_mg b on level l: damped-Jacobi sweeps before and after the coarse
 // correction (one each way for FP64 inner solves, two for FP32); the pre- and
 // post-smoothers are the same symmetric sweep, so B_mg stays complex symmetric.
@@ -1234,7 +1257,7 @@ cx<R>* vcycle(st_handle* h, Component& c, int l, const cx<R>* b, cx<R>* xa, cx<R
     }
     return xb;
   }
-  const double om = omega_of(lv.geo.d);
+  const double om = c.smooth->w64[lv.geo.d - 1];
   const R* c2 = c2_of<R>(lv);
   const double cb = (double)lv.geo.ncells * rs;
   const MGLevel& lc = c.mg[l + 1];
@@ -1259,21 +1282,22 @@ cx<R>* vcycle(st_handle* h, Component& c, int l, const cx<R>* b, cx<R>* xa, cx<R
     return xa;
   }
   // FP32 inner solves are bound by latency and launches: V(2,2), fewer iterations
+  const double w1 = c.smooth->w32[lv.geo.d - 1][0], w2 = c.smooth->w32[lv.geo.d - 1][1];
   PROF(h, s, KC_JACOBI, (int64_t)(n), m * n * 2 * cs + cb, m * n * 30.0,
-       launch_stencil<R>(OP_JACOBI_ZERO, lv.geo, coef_of<R>(lv), c2, nullptr, b, xa, lam, c.scal, c.nsel, n, om, s));
+       launch_stencil<R>(OP_JACOBI_ZERO, lv.geo, coef_of<R>(lv), c2, nullptr, b, xa, lam, c.scal, c.nsel, n, w1, s));
   PROF(h, s, KC_JACOBI, (int64_t)(n), m * n * 3 * cs + cb, m * n * (fl + 30.0),
-       launch_stencil<R>(OP_JACOBI, lv.geo, coef_of<R>(lv), c2, xa, b, xb, lam, c.scal, c.nsel, n, om, s));
+       launch_stencil<R>(OP_JACOBI, lv.geo, coef_of<R>(lv), c2, xa, b, xb, lam, c.scal, c.nsel, n, w2, s));
   PROF(h, s, KC_MG_RESID, (int64_t)(n), m * n * 3 * cs + cb, m * n * (fl + 2.0),
-       launch_stencil<R>(OP_RESID, lv.geo, coef_of<R>(lv), c2, xb, b, rtmp, lam, c.scal, c.nsel, n, om, s));
+       launch_stencil<R>(OP_RESID, lv.geo, coef_of<R>(lv), c2, xb, b, rtmp, lam, c.scal, c.nsel, n, w1, s));
   PROF(h, s, KC_RESTRICT, (int64_t)(n), m * (n + nc) * cs, m * nc * 4.0 * ipow3(lv.geo.d),
        launch_restrict<R>(lv.geo, lc.geo, rtmp, w.bl[l + 1], c.scal, c.nsel, n, lc.geo.nnodes, s));
   cx<R>* xc = vcycle<R>(h, c, l + 1, w.bl[l + 1], w.xa[l + 1], w.xb[l + 1], w.rl[l + 1]);
   PROF(h, s, KC_PROLONG, (int64_t)(n), m * (2.0 * n + nc) * cs, m * n * 4.0 * (1 << lv.geo.d),
        launch_prolong_add<R>(lv.geo, lc.geo, xc, xb, c.scal, c.nsel, n, lc.geo.nnodes, s));
   PROF(h, s, KC_JACOBI, (int64_t)(n), m * n * 3 * cs + cb, m * n * (fl + 30.0),
-       launch_stencil<R>(OP_JACOBI, lv.geo, coef_of<R>(lv), c2, xb, b, xa, lam, c.scal, c.nsel, n, om, s));
+       launch_stencil<R>(OP_JACOBI, lv.geo, coef_of<R>(lv), c2, xb, b, xa, lam, c.scal, c.nsel, n, w2, s));
   PROF(h, s, KC_JACOBI, (int64_t)(n), m * n * 3 * cs + cb, m * n * (fl + 30.0),
-       launch_stencil<R>(OP_JACOBI, lv.geo, coef_of<R>(lv), c2, xa, b, xb, lam, c.scal, c.nsel, n, om, s));
+       launch_stencil<R>(OP_JACOBI, lv.geo, coef_of<R>(lv), c2, xa, b, xb, lam, c.scal, c.nsel, n, w1, s));
   return xb;
 }
 
@@ -1352,7 +1376,7 @@ template <typename R> st_status tune_component(st_handle* h, Component& c) {
     const size_t bytes = (size_t)c.nsel * n * sizeof(cx<R>);
     ST_CUDAC(c, cudaMemsetAsync(x, 0, bytes, c.cs));
     ST_CUDAC(c, cudaMemsetAsync(b, 0, bytes, c.cs));
-    const double om = omega_of(lv.geo.d);
+    const double om = c.smooth->w64[lv.geo.d - 1];
     const R* c2 = c2_of<R>(lv);
     const int ops[4] = {OP_JACOBI_ZERO, OP_JACOBI, OP_RESID, OP_APPLY};
     for (int op : ops) {
