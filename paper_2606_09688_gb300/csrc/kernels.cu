@@ -941,12 +941,15 @@ __global__ void k_activate(CocgScal* scal, int nmodes) {
 // outputs, its warps share the inputs and meet in shared memory.
 constexpr int kTransWarps = 8;
 
+__device__ __forceinline__ bool first_sweep(const SweepInput& f) { return f.sweep != nullptr && *f.sweep == 0; }
+
 template <typename R, int QB>
 __global__ void __launch_bounds__(kBlock) k_fwd_transform(const cx<double>* __restrict__ W,
                                                           const double* __restrict__ Rt, cx<R>* __restrict__ G,
-                                                          int nsel, int nt, int64_t nx) {
+                                                          int nsel, int nt, int64_t nx, SweepInput first) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= nx) return;
+  if (first_sweep(first)) Rt = first.F;
   const int q0 = blockIdx.y * QB;
   cx<double> acc[QB];
 #pragma unroll
@@ -966,8 +969,9 @@ template <typename R, int QB>
 __global__ void __launch_bounds__(32 * kTransWarps) k_fwd_transform_split(const cx<double>* __restrict__ W,
                                                                           const double* __restrict__ Rt,
                                                                           cx<R>* __restrict__ G, int nsel, int nt,
-                                                                          int64_t nx) {
+                                                                          int64_t nx, SweepInput first) {
   __shared__ cx<double> part[kTransWarps][QB][32];
+  if (first_sweep(first)) Rt = first.F;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t a = (int64_t)blockIdx.x * 32 + lane;
   const int q0 = blockIdx.y * QB;
@@ -997,14 +1001,16 @@ __global__ void __launch_bounds__(32 * kTransWarps) k_fwd_transform_split(const 
   }
 }
 
-// U += Re(V X); V carries the weights (1 or 2) of the folded conjugate modes.
+// U += Re(V X), in the first sweep of a device-side refinement U = Re(V X); V
+// carries the weights (1 or 2) of the folded conjugate modes.
 template <typename R, int QB>
 __global__ void __launch_bounds__(kBlock) k_back_transform(const cx<double>* __restrict__ V,
                                                            const cx<R>* __restrict__ X, double* __restrict__ U,
-                                                           int nsel, int nt, int64_t nx) {
+                                                           int nsel, int nt, int64_t nx, SweepInput first) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= nx) return;
   const int i0 = blockIdx.y * QB;
+  const bool store = first_sweep(first);
   double acc[QB];
 #pragma unroll
   for (int u = 0; u < QB; ++u) acc[u] = 0.0;
@@ -1020,18 +1026,22 @@ __global__ void __launch_bounds__(kBlock) k_back_transform(const cx<double>* __r
   }
 #pragma unroll
   for (int u = 0; u < QB; ++u)
-    if (i0 + u < nt) U[(int64_t)(i0 + u) * nx + a] += acc[u];
+    if (i0 + u < nt) {
+      double* o = U + (int64_t)(i0 + u) * nx + a;
+      *o = store ? acc[u] : *o + acc[u];
+    }
 }
 
 template <typename R, int QB>
 __global__ void __launch_bounds__(32 * kTransWarps) k_back_transform_split(const cx<double>* __restrict__ V,
                                                                            const cx<R>* __restrict__ X,
                                                                            double* __restrict__ U, int nsel, int nt,
-                                                                           int64_t nx) {
+                                                                           int64_t nx, SweepInput first) {
   __shared__ double part[kTransWarps][QB][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t a = (int64_t)blockIdx.x * 32 + lane;
   const int i0 = blockIdx.y * QB;
+  const bool store = first_sweep(first);
   double acc[QB];
 #pragma unroll
   for (int u = 0; u < QB; ++u) acc[u] = 0.0;
@@ -1058,7 +1068,8 @@ __global__ void __launch_bounds__(32 * kTransWarps) k_back_transform_split(const
     double v = part[0][u][l];
 #pragma unroll
     for (int w = 1; w < kTransWarps; ++w) v += part[w][u][l];
-    U[(int64_t)(i0 + u) * nx + al] += v;
+    double* o = U + (int64_t)(i0 + u) * nx + al;
+    *o = store ? v : *o + v;
   }
 }
 
@@ -1126,6 +1137,30 @@ __global__ void __launch_bounds__(kBlock) k_stencil_real2(Geo g, StencilCoef sc,
 // pentadiagonal); row j-2 is complete after step j.  Chunks (the grid's y)
 // only matter for small grids with many time rows; they recompute the two
 // rows of halo on either side.
+// The test that ends or continues the refinement of a component without an
+// inner iteration, taken by one thread: the outcomes of the host loop.
+__device__ __forceinline__ void refine_step(const RefineStep& p, double rr, double uu, int err) {
+  RefineRec r = *p.rec;  // zero before the first sweep
+  const double f = p.fn2[0];
+  bool more = false;
+  if (r.sweeps == 0 && !(f > 0.0 && f <= 1.7e308)) {
+    r.status = f == 0.0 ? RR_OK : RR_NUMERIC;  // F = 0: U = 0 is the solution
+  } else {
+    const double eta_prev = r.sweeps == 0 ? 1e300 : r.eta;
+    r.sweeps += 1;
+    int st = err != 0 ? RR_TIMEOUT : RR_OK;
+    const double rn = sqrt(rr), fn = sqrt(f);
+    r.rel = rn / fn;
+    r.eta = rn / (p.snorm * sqrt(uu) + fn);
+    if (st == RR_OK && !(fabs(r.rel) <= 1.7e308)) st = RR_NUMERIC;
+    more = st == RR_OK && !(r.eta <= p.tol || r.eta > 0.5 * eta_prev) && r.sweeps < p.max_sweeps;
+    r.status = st;
+  }
+  if (!more) *p.host = r;  // page-locked: the host reads it once the graph has ended
+  *p.rec = more ? r : RefineRec{};
+  cudaGraphSetConditional(p.cond, more ? 1u : 0u);
+}
+
 // The same pass sums ||R||^2 and ||U||^2: every CTA leaves its partial sums in
 // `part`, and the last one to finish (counter `done`, which wraps back to 0)
 // adds them up in a fixed order into nrm2[0..1], with the component's error
@@ -1138,7 +1173,8 @@ __global__ void __launch_bounds__(kBlock) k_residual_fused(Geo g, StencilCoef sc
                                                            const double* __restrict__ Bband,
                                                            double* __restrict__ Rout, int nt, int chunk,
                                                            double* __restrict__ part, unsigned* __restrict__ done,
-                                                           const int* __restrict__ err, double* __restrict__ nrm2) {
+                                                           const int* __restrict__ err, double* __restrict__ nrm2,
+                                                           RefineStep step) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double rr = 0.0, uu = 0.0;
   if (a < g.nnodes) {
@@ -1216,6 +1252,7 @@ __global__ void __launch_bounds__(kBlock) k_residual_fused(Geo g, StencilCoef sc
     nrm2[0] = t.re;
     nrm2[1] = t.im;
     nrm2[2] = (double)err[0];
+    if (step.rec != nullptr) refine_step(step, t.re, t.im, err[0]);
   }
 }
 
@@ -1249,12 +1286,16 @@ __global__ void __launch_bounds__(kBlock) k_rhs_assemble(const double* __restric
 // ---------------------------------------------------- space eigenbasis method
 constexpr int kTile = 16;
 
-// Y[i][a] (+)= sum_b X[i][b] P[b][a], P = Phi (trans 0) or its transpose stored row-major.
+// Y[i][a] (+)= sum_b X[i][b] P[b][a], P = Phi (trans 0) or its transpose stored
+// row-major; in the first sweep of a device-side refinement without the addition,
+// and from first.F where that is given.
 __global__ void k_gemm_right(const double* __restrict__ X, const double* __restrict__ P, double* __restrict__ Y,
-                             int nt, int64_t nx, int accumulate) {
+                             int nt, int64_t nx, int accumulate, SweepInput first) {
   __shared__ double sx[kTile][kTile + 1], sp[kTile][kTile + 1];
   const int64_t a = (int64_t)blockIdx.x * kTile + threadIdx.x;
   const int i = blockIdx.y * kTile + threadIdx.y;
+  const bool store = !accumulate || first_sweep(first);
+  if (first.F != nullptr && first_sweep(first)) X = first.F;
   double acc = 0.0;
   for (int64_t b0 = 0; b0 < nx; b0 += kTile) {
     const int64_t bx = b0 + threadIdx.x, by = b0 + threadIdx.y;
@@ -1266,8 +1307,8 @@ __global__ void k_gemm_right(const double* __restrict__ X, const double* __restr
     __syncthreads();
   }
   if (i < nt && a < nx) {
-    if (accumulate) Y[(int64_t)i * nx + a] += acc;
-    else Y[(int64_t)i * nx + a] = acc;
+    double* o = Y + (int64_t)i * nx + a;
+    *o = store ? acc : *o + acc;
   }
 }
 
@@ -1888,35 +1929,35 @@ void launch_cocg_activate(CocgScal* scal, int nmodes, cudaStream_t s) {
 
 template <typename R>
 void launch_fwd_transform(const cx<double>* W, const double* Rt, cx<R>* G, int nsel, int nt, int64_t nx,
-                          cudaStream_t s) {
+                          cudaStream_t s, const SweepInput& first) {
   count(1);
   if (transform_split(nx, nsel, nt)) {
     constexpr int QB = kTransSplitQB;
     k_fwd_transform_split<R, QB><<<dim3(blocks_for(nx, 32), (nsel + QB - 1) / QB), 32 * kTransWarps, 0, s>>>(
-        W, Rt, G, nsel, nt, nx);
+        W, Rt, G, nsel, nt, nx, first);
   } else if (nsel > 5) {
-    k_fwd_transform<R, 9><<<dim3(blocks_for(nx), (nsel + 8) / 9), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+    k_fwd_transform<R, 9><<<dim3(blocks_for(nx), (nsel + 8) / 9), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx, first);
   } else if (nsel > 3) {
-    k_fwd_transform<R, 5><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+    k_fwd_transform<R, 5><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx, first);
   } else {
-    k_fwd_transform<R, 3><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx);
+    k_fwd_transform<R, 3><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(W, Rt, G, nsel, nt, nx, first);
   }
 }
 
 template <typename R>
 void launch_back_transform(const cx<double>* V, const cx<R>* X, double* U, int nsel, int nt, int64_t nx,
-                           cudaStream_t s) {
+                           cudaStream_t s, const SweepInput& first) {
   count(1);
   if (transform_split(nx, nt, nsel)) {
     constexpr int QB = kTransSplitQB;
     k_back_transform_split<R, QB><<<dim3(blocks_for(nx, 32), (nt + QB - 1) / QB), 32 * kTransWarps, 0, s>>>(
-        V, X, U, nsel, nt, nx);
+        V, X, U, nsel, nt, nx, first);
   } else if (nt > 5) {
-    k_back_transform<R, 9><<<dim3(blocks_for(nx), (nt + 8) / 9), kBlock, 0, s>>>(V, X, U, nsel, nt, nx);
+    k_back_transform<R, 9><<<dim3(blocks_for(nx), (nt + 8) / 9), kBlock, 0, s>>>(V, X, U, nsel, nt, nx, first);
   } else if (nt > 3) {
-    k_back_transform<R, 5><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(V, X, U, nsel, nt, nx);
+    k_back_transform<R, 5><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(V, X, U, nsel, nt, nx, first);
   } else {
-    k_back_transform<R, 3><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(V, X, U, nsel, nt, nx);
+    k_back_transform<R, 3><<<dim3(blocks_for(nx), 1), kBlock, 0, s>>>(V, X, U, nsel, nt, nx, first);
   }
 }
 
@@ -1946,12 +1987,12 @@ int64_t residual_blocks(const Geo& g, int nt) {
 
 void launch_residual(const Geo& g, const StencilCoef& sc, const double* c2, const double* U, const double* F,
                      const double* Aband, const double* Bband, double* Rout, int nt, double* part, unsigned* done,
-                     const int* err, double* nrm2, cudaStream_t s) {
+                     const int* err, double* nrm2, cudaStream_t s, const RefineStep& step) {
   count(1);
   const int chunk = residual_chunk(g, nt);
   const dim3 grid(blocks_for(g.nnodes), (nt + chunk - 1) / chunk);
   auto kern = g.d == 1 ? k_residual_fused<1> : (g.d == 2 ? k_residual_fused<2> : k_residual_fused<3>);
-  kern<<<grid, kBlock, 0, s>>>(g, sc, c2, U, F, Aband, Bband, Rout, nt, chunk, part, done, err, nrm2);
+  kern<<<grid, kBlock, 0, s>>>(g, sc, c2, U, F, Aband, Bband, Rout, nt, chunk, part, done, err, nrm2, step);
 }
 
 void launch_norm2(const double* v, int64_t n, double* part, double* out, cudaStream_t s) {
@@ -1976,11 +2017,11 @@ void launch_rhs_assemble(const double* coef, const double* L, double* F, int nte
 }
 
 void launch_gemm_right(const double* X, const double* Phi, double* Y, int nt, int64_t nx, int trans, int accumulate,
-                       cudaStream_t s) {
+                       cudaStream_t s, const SweepInput& first) {
   count(1);
   (void)trans;  // the caller passes Phi or its stored transpose
   dim3 block(kTile, kTile), grid((unsigned)((nx + kTile - 1) / kTile), (nt + kTile - 1) / kTile);
-  k_gemm_right<<<grid, block, 0, s>>>(X, Phi, Y, nt, nx, accumulate);
+  k_gemm_right<<<grid, block, 0, s>>>(X, Phi, Y, nt, nx, accumulate, first);
 }
 
 // Energy of Section 6.3 on the cells of one level: for every time b,
@@ -2316,8 +2357,10 @@ void note_launches(int k) { count(k); }
   template void launch_update_xr<R>(cx<R>*, cx<R>*, const cx<R>*, const cx<R>*, CocgScal*, double*, int, int64_t,    \
                                     int64_t, double, int, cudaStream_t, const double*);                              \
   template void launch_update_p<R>(cx<R>*, const cx<R>*, const CocgScal*, int, int64_t, int64_t, int, cudaStream_t);      \
-  template void launch_fwd_transform<R>(const cx<double>*, const double*, cx<R>*, int, int, int64_t, cudaStream_t);  \
-  template void launch_back_transform<R>(const cx<double>*, const cx<R>*, double*, int, int, int64_t, cudaStream_t); \
+  template void launch_fwd_transform<R>(const cx<double>*, const double*, cx<R>*, int, int, int64_t, cudaStream_t,   \
+                                        const SweepInput&);                                                          \
+  template void launch_back_transform<R>(const cx<double>*, const cx<R>*, double*, int, int, int64_t, cudaStream_t,  \
+                                         const SweepInput&);                                                         \
   template void launch_dense_coarse<R>(const cx<R>*, int64_t, const cx<R>*, cx<R>*, const CocgScal*, int, int64_t,   \
                                        cudaStream_t);                                                                \
   template void launch_identity<R>(cx<R>*, int64_t, cudaStream_t);                                              \

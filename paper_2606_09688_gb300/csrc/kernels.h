@@ -89,6 +89,25 @@ struct RefineRec {
   int sweeps, status, max_iters, inner_bodies;
 };
 enum { RR_OK = 0, RR_NUMERIC = 1, RR_ITER_LIMIT = 2, RR_TIMEOUT = 3 };
+// The refinement test of a component without an inner iteration, taken by the
+// last block of the residual (launch_residual): rec (device) keeps the record
+// between sweeps and is zero between solves, host (page-locked) receives it when
+// the refinement ends; fn2 = ||F||^2 (device).
+struct RefineStep {
+  RefineRec* rec = nullptr;  // null: no test
+  RefineRec* host = nullptr;
+  const double* fn2 = nullptr;
+  double snorm = 0.0, tol = 0.0;
+  int max_sweeps = 0;
+  cudaGraphConditionalHandle cond{};
+};
+// What the first sweep of such a refinement does otherwise: *sweep == 0 (device)
+// makes a kernel read F instead of the residual, or overwrite its result instead
+// of adding to it, so that U = 0, R = F need no passes of their own.
+struct SweepInput {
+  const int* sweep = nullptr;  // null: a later sweep
+  const double* F = nullptr;
+};
 // Clears the record; the sweep loop runs when ||F||^2 (fn2[0]) is positive.
 void launch_refine_init(RefineRec* rec, const double* fn2, cudaGraphConditionalHandle h, InnerTol it,
                         cudaStream_t s);
@@ -101,14 +120,14 @@ void launch_refine_decide(RefineRec* rec, const double* nrm2, const double* fn2,
                           cudaGraphConditionalHandle h, InnerTol it, cudaStream_t s);
 
 // Time transforms of the eigenbasis method (FP64 matrices):
-// G[q][a] = sum_i W[q][i] R[i][a];  U[i][a] += sum_q Re(V[i][q] X[q][a]) (V with
+// G[q][a] = sum_i W[q][i] R[i][a];  U[i][a] (+)= sum_q Re(V[i][q] X[q][a]) (V with
 // the weights of the folded conjugate modes).
 template <typename R>
 void launch_fwd_transform(const cx<double>* W, const double* Rt, cx<R>* G, int nsel, int nt, int64_t nx,
-                          cudaStream_t s);
+                          cudaStream_t s, const SweepInput& first = SweepInput{});
 template <typename R>
 void launch_back_transform(const cx<double>* V, const cx<R>* X, double* U, int nsel, int nt, int64_t nx,
-                           cudaStream_t s);
+                           cudaStream_t s, const SweepInput& first = SweepInput{});
 
 // FP64 space-time residual R = F - (A (x) M + B (x) K) U (banded time factors)
 // with nrm2 = (||R||^2, ||U||^2, err[0]) (device).  part: 2 x residual_blocks
@@ -116,7 +135,7 @@ void launch_back_transform(const cx<double>* V, const cx<R>* X, double* U, int n
 int64_t residual_blocks(const Geo& g, int nt);
 void launch_residual(const Geo& g, const StencilCoef& sc, const double* c2, const double* U, const double* F,
                      const double* Aband, const double* Bband, double* Rout, int nt, double* part, unsigned* done,
-                     const int* err, double* nrm2, cudaStream_t s);
+                     const int* err, double* nrm2, cudaStream_t s, const RefineStep& step = RefineStep{});
 // Sum of squares of a real vector (deterministic), result to out[0] (device).
 void launch_norm2(const double* v, int64_t n, double* part, double* out, cudaStream_t s);
 
@@ -130,7 +149,7 @@ void launch_rhs_assemble(const double* coef, const double* L, double* F, int nte
 // Space eigenbasis method: Y = X Phi (trans = 0) or Y = X Phi^T (trans = 1),
 // X nt x nx, Phi nx x nx; then banded time solves per spatial mode.
 void launch_gemm_right(const double* X, const double* Phi, double* Y, int nt, int64_t nx, int trans, int accumulate,
-                       cudaStream_t s);
+                       cudaStream_t s, const SweepInput& first = SweepInput{});
 // Band LU factors per spatial mode a: ab[a][j][0..6] = column j of the band
 // (LAPACK band layout, kl = ku = 2, row i of column j at 4 + i - j), the
 // diagonal entry replaced by its reciprocal; piv[a][j].  Returns false (and

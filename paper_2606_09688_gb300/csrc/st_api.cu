@@ -306,6 +306,7 @@ struct Component {
   RefineRec* rec = nullptr;    // device
   RefineRec* rec_h = nullptr;  // pinned copy
   double* fn2 = nullptr;       // ||F||^2 (device)
+  bool rec_direct = false;     // the solve graph writes its record to rec_h itself
   bool rec_pending = false;    // a graph solve was enqueued; its record is not read yet
 };
 
@@ -1474,6 +1475,7 @@ st_status assemble_rhs(st_handle* h, Component& c) {
     for (int i = 0; i < c.nt; ++i)
       launch_load(c.sl->geo, c.sl->sc, c.sl->c2d, c.Fg_all + (size_t)i * c.sl->nall, c.F + (size_t)i * c.nx, 0.0,
                   1.0, 1, c.cs);
+  if (c.fn2 != nullptr) launch_norm2(c.F, c.nx * (int64_t)c.nt, c.cpart, c.fn2, c.cs);  // F is fixed after set-up
   c.f_ready = true;
   return ccheck(c, "rhs");
 }
@@ -1665,12 +1667,100 @@ cudaError_t set_kernel_priority(cudaGraph_t g, int prio) {
   return cudaSuccess;
 }
 
-// The forward solve of a component as one CUDA graph, captured on its stream:
+// The forward solve of a component without an inner iteration (direct or space
+// eigenbasis) as one CUDA graph, a single WHILE node whose condition starts true:
+//   WHILE { U (+)= S~^{-1} R; R = F - S U; ||R||^2, ||U||^2; stopping test }
+// A node costs about 4 us when its kernel is small, so the first sweep reads F and
+// overwrites U, and the residual's last block takes the norms and the stopping
+// test and writes the record to page-locked memory.
+// One pass against a graph of a prologue (U = 0, R = F, ||F||^2, condition), a
+// WHILE sweep with the test in a launch of its own and a copy of the record: 1D
+// n = 6 FP64 162 -> 124 us, 2D n = 8 FP32 545 -> 483 us, 2D box n = 9 FP64
+// 506 -> 446 us.  The first sweep outside the node, as plain graph nodes, took
+// the box to 626 us: a dozen such chains queue behind one another.
+template <typename R> st_status capture_direct_graph(st_handle* h, Component& c) {
+  const SolveIO io = forward_io(c);
+  if (c.method == 1 && time_band_smem(c.nt) > kTimeBandMaxSmem)
+    return fail(h, ST_ERR_ARG, "device solve: time band solve of this size not supported");
+  c.rec = h->alloc<RefineRec>(1);
+  c.fn2 = h->alloc<double>(1);
+  ST_NEED(h, c.rec);
+  ST_NEED(h, c.fn2);
+  c.rec_h = h->pinned_alloc<RefineRec>(1);
+  ST_CUDA(h, cudaMemsetAsync(c.rec, 0, sizeof(RefineRec), c.cs));
+  int prio_lo = 0, prio_hi = 0;
+  ST_CUDA(h, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
+  cudaGraph_t g = nullptr, sweep = nullptr, out = nullptr;
+  ST_CUDA(h, cudaGraphCreate(&g, 0));
+  RefineStep step;
+  step.rec = c.rec;
+  step.host = c.rec_h;
+  step.fn2 = c.fn2;
+  step.snorm = c.Snorm;
+  step.tol = h->opt.tol > 0 ? h->opt.tol : 1e-14;
+  step.max_sweeps = h->opt.max_sweeps > 0 ? h->opt.max_sweeps : 8;
+  const SweepInput first_in{&c.rec->sweeps, io.rhs}, first_out{&c.rec->sweeps, nullptr};
+  const char* where = "sweep node";
+  cudaError_t e = cudaGraphConditionalHandleCreate(&step.cond, g, 1, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess) {
+    cudaGraphNodeParams np{};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = step.cond;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaGraphNode_t node;
+    e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np);
+    if (e == cudaSuccess) sweep = np.conditional.phGraph_out[0];
+  }
+  const int64_t l0 = kernel_launch_count();
+  if (e == cudaSuccess) {
+    where = "sweep capture";
+    e = cudaStreamBeginCaptureToGraph(c.cs, sweep, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+  }
+  if (e == cudaSuccess) {
+    if (c.method == 1) {
+      launch_gemm_right(c.Rv, c.Phi, c.KU, c.nt, c.nx, 0, 0, c.cs, first_in);
+      launch_time_band_solve(io.lu_ab, io.lu_piv, c.KU, c.nt, c.nx, c.kl, c.ku, c.cs);
+      launch_gemm_right(c.KU, c.PhiT, io.sol, c.nt, c.nx, 1, 1, c.cs, first_out);
+    } else {
+      Work<R>& w = work_of<R>(c);
+      launch_fwd_transform<R>(io.Wf, c.Rv, w.G, c.nsel, c.nt, c.nx, c.cs, first_in);
+      direct_solve<R>(c, w.G, w.X, nullptr, c.nx, c.cs);
+      launch_back_transform<R>(io.Vb, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs, first_out);
+    }
+    launch_residual(c.sl->geo, c.sl->sc, c.sl->c2d, io.sol, io.rhs, io.Ab, io.Bb, c.Rv, c.nt, c.cpart, c.cdone, c.cerr,
+                    c.cscalar, c.cs, step);
+    e = cudaStreamEndCapture(c.cs, &out);
+  }
+  c.gs_pro_nodes = 0;
+  c.gs_sweep_nodes = kernel_launch_count() - l0;
+  c.gs_inner_nodes = 0;
+  c.rec_direct = true;
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess) {
+    where = "priority";
+    e = set_kernel_priority(sweep, prio_hi);
+  }
+  cudaGraphExec_t ge = nullptr;
+  if (e == cudaSuccess) {
+    where = "instantiation";
+    e = cudaGraphInstantiate(&ge, g, 0);
+  }
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(h, ST_ERR_CUDA, std::string("solve graph (") + where + "): " + cudaGetErrorString(e));
+  }
+  c.g_solve = ge;
+  return ST_OK;
+}
+
+// The forward solve of a multigrid component as one CUDA graph, captured on its
+// stream:
 //   U = 0, R = F, ||F||^2, condition (k_refine_init);
 //   WHILE (condition) {                       -- one refinement sweep
-//     time eigenbasis: G = W R; COCG start; WHILE (any mode active)
+//     G = W R; COCG start; WHILE (any mode active)
 //       { device_loop COCG iterations; condition }; U += Re(V X)
-//     (direct components: the banded solve; space eigenbasis: its sweep)
 //     R = F - S U; ||R||^2, ||U||^2; stopping test (k_refine_decide) }
 // The same kernels as the host-driven loop, in the same order; the host reads
 // the record (sweeps, backward error, status) once per call.
@@ -1679,9 +1769,6 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
   const int64_t n = c.nx * (int64_t)c.nt;
   const double tol = h->opt.tol > 0 ? h->opt.tol : 1e-14;
   const int max_sweeps = h->opt.max_sweeps > 0 ? h->opt.max_sweeps : 8;
-  const bool iterative = c.method == 0 && !c.direct;
-  if (c.method == 1 && time_band_smem(c.nt) > kTimeBandMaxSmem)
-    return fail(h, ST_ERR_ARG, "device solve: time band solve of this size not supported");
   c.rec = h->alloc<RefineRec>(1);
   c.fn2 = h->alloc<double>(1);
   ST_NEED(h, c.rec);
@@ -1718,28 +1805,18 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
   // one sweep
   l0 = kernel_launch_count();
   if (e == cudaSuccess && ok(cudaStreamBeginCaptureToGraph(c.cs, sweep, nullptr, nullptr, 0, mode), "sweep capture")) {
-    if (c.method == 1) {
-      launch_gemm_right(c.Rv, c.Phi, c.KU, c.nt, c.nx, 0, 0, c.cs);
-      launch_time_band_solve(io.lu_ab, io.lu_piv, c.KU, c.nt, c.nx, c.kl, c.ku, c.cs);
-      launch_gemm_right(c.KU, c.PhiT, io.sol, c.nt, c.nx, 1, 1, c.cs);
-    } else {
-      Work<R>& w = work_of<R>(c);
-      launch_fwd_transform<R>(io.Wf, c.Rv, w.G, c.nsel, c.nt, c.nx, c.cs);
-      if (c.direct) {
-        direct_solve<R>(c, w.G, w.X, nullptr, c.nx, c.cs);
-      } else {
-        c.nactive = c.nsel;
-        cocg_start<R>(h, c);
-        if (ok(cudaGraphConditionalHandleCreate(&hi, sweep, 0, cudaGraphCondAssignDefault), "inner condition")) {
-          launch_cocg_continue(c.scal, c.nsel, hi, nullptr, c.cs);
-          ok(capture_add_while(c.cs, hi, &inner), "inner node");
-        }
-      }
-      launch_back_transform<R>(io.Vb, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs);
+    Work<R>& w = work_of<R>(c);
+    launch_fwd_transform<R>(io.Wf, c.Rv, w.G, c.nsel, c.nt, c.nx, c.cs);
+    c.nactive = c.nsel;
+    cocg_start<R>(h, c);
+    if (ok(cudaGraphConditionalHandleCreate(&hi, sweep, 0, cudaGraphCondAssignDefault), "inner condition")) {
+      launch_cocg_continue(c.scal, c.nsel, hi, nullptr, c.cs);
+      ok(capture_add_while(c.cs, hi, &inner), "inner node");
     }
+    launch_back_transform<R>(io.Vb, w.X, io.sol, c.nsel, c.nt, c.nx, c.cs);
     launch_residual(c.sl->geo, c.sl->sc, c.sl->c2d, io.sol, io.rhs, io.Ab, io.Bb, c.Rv, c.nt, c.cpart, c.cdone,
                     c.cerr, c.cscalar, c.cs);
-    launch_refine_decide(c.rec, c.cscalar, c.fn2, c.Snorm, tol, max_sweeps, iterative ? c.scal : nullptr, c.nsel,
+    launch_refine_decide(c.rec, c.cscalar, c.fn2, c.Snorm, tol, max_sweeps, c.scal, c.nsel,
                          c.cerr, hs, c.itol_rule, c.cs);
     cudaGraph_t out = nullptr;
     ok(cudaStreamEndCapture(c.cs, &out), "sweep capture end");
@@ -1747,14 +1824,14 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
   c.gs_sweep_nodes = kernel_launch_count() - l0;
   // the COCG loop body
   l0 = kernel_launch_count();
-  if (e == cudaSuccess && iterative &&
+  if (e == cudaSuccess &&
       ok(cudaStreamBeginCaptureToGraph(c.cs, inner, nullptr, nullptr, 0, mode), "inner capture")) {
     for (int k = 0; k < h->opt.device_loop; ++k) cocg_iteration<R>(h, c);
     launch_cocg_continue(c.scal, c.nsel, hi, &c.rec->inner_bodies, c.cs);
     cudaGraph_t out = nullptr;
     ok(cudaStreamEndCapture(c.cs, &out), "inner capture end");
   }
-  c.gs_inner_nodes = iterative ? kernel_launch_count() - l0 : 0;
+  c.gs_inner_nodes = kernel_launch_count() - l0;
   if (e == cudaSuccess) ok(cudaGetLastError(), "captured launches");
   if (e == cudaSuccess) ok(set_kernel_priority(g, prio_hi), "priority");
   if (e == cudaSuccess) ok(set_kernel_priority(sweep, prio_hi), "priority");
@@ -1770,14 +1847,15 @@ template <typename R> st_status capture_solve_graph(st_handle* h, Component& c) 
   return ST_OK;
 }
 
-// Enqueues a component's forward solve as its graph, then the copy of its record.
+// Enqueues a component's forward solve as its graph; its record is on the host
+// once the stream has passed it.
 st_status enqueue_graph_solve(st_handle* h, Component& c) {
   st_status s = assemble_rhs(h, c);
   if (s != ST_OK) return s;
   c.info = st_solve_info{};
   c.info.status = ST_OK;
   ST_CUDAC(c, cudaGraphLaunch(c.g_solve, c.cs));
-  ST_CUDAC(c, cudaMemcpyAsync(c.rec_h, c.rec, sizeof(RefineRec), cudaMemcpyDeviceToHost, c.cs));
+  if (!c.rec_direct) ST_CUDAC(c, cudaMemcpyAsync(c.rec_h, c.rec, sizeof(RefineRec), cudaMemcpyDeviceToHost, c.cs));
   c.d2h += (int64_t)sizeof(RefineRec);
   note_launches((int)c.gs_pro_nodes);
   c.rec_pending = true;
@@ -1864,8 +1942,9 @@ st_status setup_context(st_handle* h, Component& c) {
   // stay host-driven: a graph occupies one of the device's few launch queues
   // until it ends, and short solves behind it wait (2D n = 12: 52.8 against
   // 53.6 ms with every solve as a graph).
-  if (h->opt.device_loop > 0 || c.method == 1 || c.direct)
-    return (c.method == 0 && !c.inner64) ? capture_solve_graph<float>(h, c) : capture_solve_graph<double>(h, c);
+  const bool fp32 = c.method == 0 && !c.inner64;
+  if (c.method == 1 || c.direct) return fp32 ? capture_direct_graph<float>(h, c) : capture_direct_graph<double>(h, c);
+  if (h->opt.device_loop > 0) return fp32 ? capture_solve_graph<float>(h, c) : capture_solve_graph<double>(h, c);
   return ST_OK;
 }
 
