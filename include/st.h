@@ -261,9 +261,11 @@ st_status st_misfit_gradient(st_handle* h, int jt_star, const double* x_rec, int
  * other value accepted), where the combined solution is Q1 in space, and the
  * integrals are taken exactly per cell with c^2 cellwise at that level's cell
  * centres.  Requires every component solved (ST_ERR_STATE); ST_ERR_ARG for
- * times outside [0, T] or another jx_eval; device memory for the levels and
- * tables is taken with cudaMallocAsync on the handle's stream (ST_ERR_OOM if
- * that fails).  Synchronises the handle's stream. */
+ * times outside [0, T] or another jx_eval.  The levels of a batch of times and
+ * the tables take at most 72 MiB of device memory that stays with the handle; a
+ * single time of a larger grid, and every call of a handle with mem_cap_bytes,
+ * takes it with cudaMallocAsync on the handle's stream (ST_ERR_OOM if that
+ * fails).  Synchronises the handle's stream. */
 st_status st_energy(st_handle* h, const double* times, int ntimes, int jx_eval, double* energy_out);
 
 /* Copy the FP64 coefficient array U_k (n_time x n_space, time-major) of a

@@ -1396,7 +1396,8 @@ __device__ __forceinline__ double with_sign(double x, unsigned sign_hi) {
 // FMAs per node; coef = -1 enters as a sign flip of the B-spline values.
 template <int D> __device__ __forceinline__ double comp_add(const CombComp& cc, int j, const int P[3], int s,
                                                             int nts, int c, const double* __restrict__ tbv,
-                                                            const int* __restrict__ tspan, bool interior, double v) {
+                                                            const int* __restrict__ tspan, bool interior, bool lift,
+                                                            double v) {
   const int sh = cc.jx - j;  // >= 0: injection from a finer component grid
   const int N = 1 << cc.jx, n = N - 1, nt = (1 << cc.jt) + 1;
   const unsigned sg = cc.coef > 0 ? 0u : 0x80000000u;
@@ -1418,7 +1419,7 @@ template <int D> __device__ __forceinline__ double comp_add(const CombComp& cc, 
       v = fma(with_sign(tb[t], sg), u, v);
     }
   }
-  if (cc.lift != nullptr) {
+  if (lift && cc.lift != nullptr) {
     int64_t ia = 0, sa = 1;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
@@ -1457,7 +1458,7 @@ template <int D>
 __global__ void __launch_bounds__(kBlock) k_comb_level(int j, const double* __restrict__ Yprev,
                                                        const CombComp* __restrict__ comps, int c0, int c1,
                                                        const double* __restrict__ tbv, const int* __restrict__ tspan,
-                                                       int nts, double* __restrict__ Y, FastDiv dQ1) {
+                                                       int nts, int nlift, double* __restrict__ Y, FastDiv dQ1) {
   const int s = blockIdx.y;
   const int Nj = 1 << j, Nc = Nj >> 1;
   int64_t ncs = 1, nsp = 1;
@@ -1521,7 +1522,7 @@ __global__ void __launch_bounds__(kBlock) k_comb_level(int j, const double* __re
     }
     if (!inside) continue;
     double v = f[e];
-    for (int c = c0; c < c1; ++c) v = comp_add<D>(comps[c], j, P, s, nts, c, tbv, tspan, interior, v);
+    for (int c = c0; c < c1; ++c) v = comp_add<D>(comps[c], j, P, s, nts, c, tbv, tspan, interior, s < nlift, v);
     Y[(int64_t)s * nsp + pidx] = v;
   }
 }
@@ -2024,6 +2025,35 @@ void launch_gemm_right(const double* X, const double* Phi, double* Y, int nt, in
   k_gemm_right<<<grid, block, 0, s>>>(X, Phi, Y, nt, nx, accumulate, first);
 }
 
+// Tables of the energy's combination levels, one thread per component and time:
+// row b holds the B-spline values of component c at times[b], row nb + b their
+// first derivatives.
+__global__ void __launch_bounds__(128) k_energy_tables(const CombComp* __restrict__ comps,
+                                                       const double* __restrict__ times, int nb, double T,
+                                                       double* __restrict__ tb, int* __restrict__ span) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
+  if (b >= nb) return;
+  const int Nt = 1 << comps[c].jt;
+  const double t = times[b];
+  const int k = min(Nt - 1, max(0, (int)floor(t * Nt / T)));
+  double v[3], d1[3], d2[3];
+  bs_local(Nt, T, k, t, v, d1, d2);
+  const int64_t row = (int64_t)c * 2 * nb + b;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    tb[row * 3 + a] = v[a];
+    tb[(row + nb) * 3 + a] = d1[a];
+  }
+  span[row] = k;
+  span[row + nb] = k;
+}
+
+void launch_energy_tables(const CombComp* comps, int nc, const double* times, int nb, double T, double* tb, int* span,
+                          cudaStream_t s) {
+  count(1);
+  k_energy_tables<<<dim3((nb + 127) / 128, nc), 128, 0, s>>>(comps, times, nb, T, tb, span);
+}
+
 // Energy of Section 6.3 on the cells of one level: for every time b,
 // part[b][block] = 1/2 sum over the block's cells e of
 //   z_e^T Me z_e + c2_e y_e^T Ke y_e,
@@ -2203,15 +2233,16 @@ bool launch_time_band_solve(const double* ab, const int* piv, double* Y, int nt,
 }
 
 void launch_comb_level(int d, int j, const double* Yprev, const CombComp* comps, int c0, int c1, const double* tbv,
-                       const int* tspan, int nts, double* Y, cudaStream_t s) {
+                       const int* tspan, int nts, double* Y, cudaStream_t s, int nlift) {
   count(1);
+  if (nlift < 0) nlift = nts;
   int64_t ncs = 1;  // one thread per node of level j-1 (each writes up to 2^d level-j nodes)
   for (int k = 0; k < d; ++k) ncs *= ((1 << j) / 2 + 1);
   dim3 grid(blocks_for(ncs), nts);
   const FastDiv f = make_fastdiv((unsigned)((1 << j) / 2 + 1));
-  if (d == 1) k_comb_level<1><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, Y, f);
-  else if (d == 2) k_comb_level<2><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, Y, f);
-  else k_comb_level<3><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, Y, f);
+  if (d == 1) k_comb_level<1><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f);
+  else if (d == 2) k_comb_level<2><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f);
+  else k_comb_level<3><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f);
 }
 
 template <typename R>

@@ -171,8 +171,13 @@ struct CombComp {
 // coef * u_k(., t_s) on the (2^j+1)^d nodes of level j, for every target time.
 // tbv[c][s][0..2]: the three B-spline values of component c at target time s,
 // tspan[c][s] their interval.  Yprev (level j-1, all nodes x nts) may be null.
+// The lifts enter the first nlift rows s (all of them by default).
 void launch_comb_level(int d, int j, const double* Yprev, const CombComp* comps, int c0, int c1, const double* tbv,
-                       const int* tspan, int nts, double* Y, cudaStream_t s);
+                       const int* tspan, int nts, double* Y, cudaStream_t s, int nlift = -1);
+// The tables of launch_comb_level for values (rows 0..nb-1) and time derivatives
+// (rows nb..2nb-1) at nb times in [0, T] (device).
+void launch_energy_tables(const CombComp* comps, int nc, const double* times, int nb, double T, double* tb, int* span,
+                          cudaStream_t s);
 // The same level in double-single arithmetic (combine_ds.cu): Yprev and, below
 // the target level, Y hold float pairs (8 bytes per value); the target level
 // (final_level) is written as FP64.  comps: per component its coefficient

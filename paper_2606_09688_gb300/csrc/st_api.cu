@@ -378,6 +378,33 @@ struct st_handle {
     int max_nt = 1;
   } rec;
 
+  // Workspace of st_energy, kept between calls up to 72 MiB.
+  struct Workspace {
+    static constexpr size_t kMax = (size_t)72 << 20;
+    unsigned char* p = nullptr;
+    size_t n = 0;
+    // At least bytes, or null where that is beyond kMax or not to be had.  No
+    // work that uses the old block may be pending.
+    unsigned char* get(size_t bytes) {
+      if (bytes <= n) return p;
+      if (bytes > kMax) return nullptr;
+      if (p != nullptr) cudaFree(p);
+      p = nullptr;
+      n = 0;
+      void* q = nullptr;
+      if (cudaMalloc(&q, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      p = (unsigned char*)q;
+      n = bytes;
+      return p;
+    }
+    ~Workspace() {
+      if (p != nullptr) cudaFree(p);
+    }
+  } energy_ws;
+
   // Optional per-kernel-class timing: CUDA events recorded on the handle's
   // stream around every launch, with the algorithmic bytes and flops of it.
   struct ProfRec {
@@ -2975,9 +3002,10 @@ st_status st_energy(st_handle* h, const double* times, int ntimes, int jx_eval, 
     if (!(times[i] >= 0.0 && times[i] <= p.T)) return fail(h, ST_ERR_ARG, "times must lie in [0, T]");
   const SpaceLevel& sl = *h->space[jx_eval];
   const int d = p.d, N = 1 << jx_eval;
-  int64_t nall = 1, ncell = 1;
+  int64_t nall = 1, ncoarse = 1, ncell = 1;
   for (int k = 0; k < d; ++k) {
     nall *= N + 1;
+    ncoarse *= N / 2 + 1;
     ncell *= N;
   }
   // components in level order; the combination levels evaluate u^CF and d_t u^CF
@@ -2989,87 +3017,64 @@ st_status st_energy(st_handle* h, const double* times, int ntimes, int jx_eval, 
   std::vector<int> first(jx_eval + 2, nc);
   for (int o = nc - 1; o >= 0; --o) first[h->comps[order[o]]->jx] = o;
   for (int lev = jx_eval; lev >= 0; --lev) first[lev] = std::min(first[lev], first[lev + 1]);
-  std::vector<CombComp> cv(nc), cd(nc);
+  std::vector<CombComp> cv(nc);
   for (int o = 0; o < nc; ++o) {
     const Component& k = *h->comps[order[o]];
     cv[o] = CombComp{k.U, k.sl->lift, k.jx, k.jt, k.coef, 0};
-    cd[o] = CombComp{k.U, nullptr, k.jx, k.jt, k.coef, 0};
   }
-  const int64_t budget = (int64_t)256 << 20;  // device bytes for the level arrays of one batch
-  const int B = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)ntimes, 256, budget / (nall * 8 * 4)}));
-  const unsigned nblk = (unsigned)((ncell + 255) / 256);
+  // Bound by launches and host work on small grids, so a batch is as many times
+  // as fit the budget, its B-spline tables are formed on the device, every level is
+  // one launch for values and time derivatives, and two buffers serve all levels:
+  // 1D n = 13, 800 times, 1.15 -> 0.15 ms against batches of 256 with host tables,
+  // two launches a level and call-local allocations.  The budget keeps a batch's
+  // levels in L2; a workspace within it stays with the handle, a larger one (a
+  // single time of a large grid) or that of a handle with a memory cap is call-local.
+  const int64_t budget = (int64_t)64 << 20;
+  const int B = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)ntimes, 16384, budget / ((nall + ncoarse) * 16)}));
+  const int64_t nblk = (ncell + 255) / 256;
   cudaStream_t st = h->stream;
-  // call-local device memory, stream-ordered
-  std::vector<void*> bufs;
-  auto dalloc = [&](size_t bytes) -> void* {
-    void* q = nullptr;
-    if (cudaMallocAsync(&q, bytes, st) != cudaSuccess) return nullptr;
-    bufs.push_back(q);
-    return q;
+  size_t total = 0;
+  auto part_of = [&](size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 255) & ~(size_t)255;
+    return at;
   };
-  auto release = [&]() {
-    for (void* q : bufs) cudaFreeAsync(q, st);
-    bufs.clear();
-  };
-  CombComp* dcv = (CombComp*)dalloc(sizeof(CombComp) * nc);
-  CombComp* dcd = (CombComp*)dalloc(sizeof(CombComp) * nc);
-  double* tbv = (double*)dalloc(sizeof(double) * 3 * nc * B);
-  double* tbd = (double*)dalloc(sizeof(double) * 3 * nc * B);
-  int* tsp = (int*)dalloc(sizeof(int) * nc * B);
-  double* part = (double*)dalloc(sizeof(double) * (size_t)nblk * B);
-  double* eout = (double*)dalloc(sizeof(double) * ntimes);
-  std::vector<double*> Yv(jx_eval + 1, nullptr), Yd(jx_eval + 1, nullptr);
-  bool ok = dcv && dcd && tbv && tbd && tsp && part && eout;
-  for (int lev = jmin; lev <= jx_eval && ok; ++lev) {
-    int64_t nsp = 1;
-    for (int k = 0; k < d; ++k) nsp *= (1 << lev) + 1;
-    Yv[lev] = (double*)dalloc(sizeof(double) * nsp * B);
-    Yd[lev] = (double*)dalloc(sizeof(double) * nsp * B);
-    ok = Yv[lev] && Yd[lev];
+  const size_t o_comps = part_of(sizeof(CombComp) * nc), o_times = part_of(sizeof(double) * ntimes);
+  const size_t o_out = part_of(sizeof(double) * ntimes), o_tb = part_of(sizeof(double) * 6 * nc * B);
+  const size_t o_span = part_of(sizeof(int) * 2 * nc * B), o_part = part_of(sizeof(double) * (size_t)nblk * B);
+  const size_t o_fine = part_of(sizeof(double) * 2 * (size_t)nall * B);
+  const size_t o_coarse = part_of(sizeof(double) * 2 * (size_t)ncoarse * B);
+  unsigned char* ws = h->opt.mem_cap_bytes > 0 ? nullptr : h->energy_ws.get(total);
+  void* local = nullptr;
+  if (ws == nullptr) {
+    if (cudaMallocAsync(&local, total, st) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(h, ST_ERR_OOM, "device allocation failed");
+    }
+    ws = (unsigned char*)local;
   }
-  if (!ok) {
-    cudaGetLastError();
-    release();
-    return fail(h, ST_ERR_OOM, "device allocation failed");
-  }
-  ST_CUDA(h, cudaMemcpyAsync(dcv, cv.data(), sizeof(CombComp) * nc, cudaMemcpyHostToDevice, st));
-  ST_CUDA(h, cudaMemcpyAsync(dcd, cd.data(), sizeof(CombComp) * nc, cudaMemcpyHostToDevice, st));
+  CombComp* comps = (CombComp*)(ws + o_comps);
+  double *dt = (double*)(ws + o_times), *eout = (double*)(ws + o_out), *tb = (double*)(ws + o_tb);
+  double* part = (double*)(ws + o_part);
+  int* span = (int*)(ws + o_span);
+  double* Y[2] = {(double*)(ws + o_fine), (double*)(ws + o_coarse)};  // by the distance from the finest level, even / odd
+  cudaError_t e = cudaMemcpyAsync(comps, cv.data(), sizeof(CombComp) * nc, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dt, times, sizeof(double) * ntimes, cudaMemcpyHostToDevice, st);
   const ElemK me = element_mass(d, sl.h), ke = element_stiffness(d, sl.h);
-  std::vector<double> hv((size_t)3 * nc * B), hd((size_t)3 * nc * B);
-  std::vector<int> hs((size_t)nc * B);
-  for (int t0 = 0; t0 < ntimes; t0 += B) {
+  for (int t0 = 0; t0 < ntimes && e == cudaSuccess; t0 += B) {
     const int nb = std::min(B, ntimes - t0);
-    for (int o = 0; o < nc; ++o) {
-      const Component& k = *h->comps[order[o]];
-      const int Nt = 1 << k.jt;
-      for (int b = 0; b < nb; ++b) {
-        const double t = times[t0 + b];
-        const int span = std::min(Nt - 1, std::max(0, (int)std::floor(t * Nt / p.T)));
-        double v[3], d1[3], d2[3];
-        bspline_local(Nt, p.T, span, t, v, d1, d2);
-        for (int a = 0; a < 3; ++a) {
-          hv[((size_t)o * nb + b) * 3 + a] = v[a];
-          hd[((size_t)o * nb + b) * 3 + a] = d1[a];
-        }
-        hs[(size_t)o * nb + b] = span;
-      }
-    }
-    ST_CUDA(h, cudaMemcpyAsync(tbv, hv.data(), sizeof(double) * 3 * nc * nb, cudaMemcpyHostToDevice, st));
-    ST_CUDA(h, cudaMemcpyAsync(tbd, hd.data(), sizeof(double) * 3 * nc * nb, cudaMemcpyHostToDevice, st));
-    ST_CUDA(h, cudaMemcpyAsync(tsp, hs.data(), sizeof(int) * nc * nb, cudaMemcpyHostToDevice, st));
+    launch_energy_tables(comps, nc, dt + t0, nb, p.T, tb, span, st);
     for (int lev = jmin; lev <= jx_eval; ++lev) {
-      const double* pv = lev > jmin ? Yv[lev - 1] : nullptr;
-      const double* pd = lev > jmin ? Yd[lev - 1] : nullptr;
-      launch_comb_level(d, lev, pv, dcv, first[lev], first[lev + 1], tbv, tsp, nb, Yv[lev], st);
-      launch_comb_level(d, lev, pd, dcd, first[lev], first[lev + 1], tbd, tsp, nb, Yd[lev], st);
+      double* y = Y[(jx_eval - lev) & 1];
+      launch_comb_level(d, lev, lev > jmin ? Y[(jx_eval - lev + 1) & 1] : nullptr, comps, first[lev], first[lev + 1], tb,
+                        span, 2 * nb, y, st, nb);
     }
-    launch_energy_cells(d, N, sl.c2d, Yv[jx_eval], Yd[jx_eval], nall, nb, me, ke, part, eout + t0, st);
-    // the host tables are overwritten by the next batch: wait for this batch's copies
-    ST_CUDA(h, cudaStreamSynchronize(st));
+    launch_energy_cells(d, N, sl.c2d, Y[0], Y[0] + (size_t)nall * nb, nall, nb, me, ke, part, eout + t0, st);
   }
-  ST_CUDA(h, cudaMemcpyAsync(energy_out, eout, sizeof(double) * ntimes, cudaMemcpyDeviceToHost, st));
-  release();
-  ST_CUDA(h, cudaStreamSynchronize(st));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(energy_out, eout, sizeof(double) * ntimes, cudaMemcpyDeviceToHost, st);
+  if (local != nullptr) cudaFreeAsync(local, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  ST_CUDA(h, e);
   h->d2h_bytes += (int64_t)(sizeof(double) * ntimes);
   return check_launch(h, "energy");
 }
