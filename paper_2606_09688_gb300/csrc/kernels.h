@@ -9,6 +9,36 @@
 
 namespace st {
 
+// Launches that overlap the kernel before them on the stream (programmatic
+// dependent launch): the blocks are placed once every block of that kernel has
+// passed grid_start() or ended, and wait in it for its end and its writes.  A
+// kernel launched so calls grid_start() in every thread, before any return and
+// before it reads or writes what the kernel before it touches; what older kernels
+// wrote may be read ahead of it.  Pointers to what the kernel before writes are
+// not const __restrict__: such loads may take the read-only path, which the wait
+// does not order.
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_start() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+template <typename... Params, typename... Args>
+void launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       Args... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 enum StencilOp { OP_APPLY = 0, OP_RESID = 1, OP_JACOBI = 2, OP_JACOBI_ZERO = 3 };
 
 // Per-mode state of the batched COCG iteration (device memory).

@@ -410,16 +410,20 @@ __global__ void __launch_bounds__(kThreads)
 // row, so the matrix is read once, coalesced over the rows; the warps' sums
 // meet in shared memory in a fixed order.  The inputs (own right-hand side
 // minus the children's updates, and on the way down the boundary's solution)
-// are gathered into shared memory by every task of the front.
-template <typename R, bool UP>
+// are gathered into shared memory by every task of the front.  AHEAD: launched
+// with launch_overlapped, the first matrix entries are read while the depth
+// before ends: a depth waits on dependent loads, and these leave the chain.  FP32
+// components alone, three sweeps: 63^2 3 modes 256 -> 203 us, 31^2 5 modes
+// 177 -> 149 us, 127^2 17 modes 1.25 -> 1.06 ms; FP64 (bound by its instructions)
+// gained nothing.
+template <typename R, bool UP, bool AHEAD>
 __global__ void __launch_bounds__(512)
     k_nd_level(NdLevel L, int leaf, int64_t cu, int cbmax, int g, int chunks, int kmax, const int* __restrict__ idx,
                const int* __restrict__ map, int64_t nidx, const int* __restrict__ nbs,
-               const cx<R>* __restrict__ mats, int64_t mstride, const cx<R>* __restrict__ b, cx<R>* x, cx<R>* u,
-               int64_t ustride, const CocgScal* __restrict__ scal, int64_t vstride) {
+               const cx<R>* __restrict__ mats, int64_t mstride, const cx<R>* b, cx<R>* x, cx<R>* u, int64_t ustride,
+               const CocgScal* scal, int64_t vstride) {
   extern __shared__ __align__(16) unsigned char smem_nd[];
   const int q = blockIdx.y;
-  if (scal != nullptr && !scal[q].active) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tp = (blockDim.x >> 5) / g;  // tasks per CTA
   const int tk = warp / g, wg = warp - tk * g;
@@ -436,6 +440,20 @@ __global__ void __launch_bounds__(512)
   cx<R>* uq = u + (int64_t)q * ustride;
   const int64_t c0 = cu + (int64_t)(2 * v) * cbmax, c1 = c0 + cbmax;  // the children's updates
   const int K = !live ? 0 : (UP ? L.s : L.s + nb);
+  // this lane's row of the matrix, its first entries read while the kernel before ends
+  const int rows = UP ? nb : L.s, ldm = UP ? L.bmax : L.s;
+  const cx<R>* M = mats + (int64_t)q * mstride +
+                   (UP ? L.g + (int64_t)v * L.s * L.bmax : L.h + (int64_t)v * L.ld * L.s) + r;
+  const bool out = live && r < rows;
+  cx<R> m[8];
+  if constexpr (AHEAD) {
+    if (out && wg + 7 * g < K) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) m[t] = M[(int64_t)(wg + t * g) * ldm];
+    }
+    grid_start();
+  }
+  if (scal != nullptr && !scal[q].active) return;
   for (int k = wg * 32 + lane; k < K; k += 32 * g) {
     cx<R> val;
     if (k < L.s) {
@@ -451,18 +469,15 @@ __global__ void __launch_bounds__(512)
     in[k] = val;
   }
   __syncthreads();
-  const int rows = UP ? nb : L.s, ldm = UP ? L.bmax : L.s;
-  const cx<R>* M = mats + (int64_t)q * mstride +
-                   (UP ? L.g + (int64_t)v * L.s * L.bmax : L.h + (int64_t)v * L.ld * L.s) + r;
   cx<R> acc = mk<R>(0, 0);
-  const bool out = live && r < rows;
   if (out) {
     cx<R> a2 = mk<R>(0, 0);
     int k = wg;
     for (; k + 7 * g < K; k += 8 * g) {
-      cx<R> m[8];
+      if (!AHEAD || k != wg) {
 #pragma unroll
-      for (int t = 0; t < 8; ++t) m[t] = M[(int64_t)(k + t * g) * ldm];
+        for (int t = 0; t < 8; ++t) m[t] = M[(int64_t)(k + t * g) * ldm];
+      }
 #pragma unroll
       for (int t = 0; t < 8; t += 2) {
         acc = fma_c(m[t], in[k + t * g], acc);
@@ -504,11 +519,22 @@ void nd_level(const NdPlan& p, int t, const cx<R>* mats, const cx<R>* b, cx<R>* 
   const size_t smem = ((size_t)tp * kmax + threads) * sizeof(cx<R>);
   const int64_t cu = leaf ? 0 : p.lv[t + 1].u;
   const int cb = leaf ? 0 : p.lv[t + 1].bmax;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_nd_level<R, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_nd_level<R, UP><<<dim3((unsigned)cdiv64(tasks, tp), nmodes), threads, smem, s>>>(
-      L, leaf ? 1 : 0, cu, cb, g, chunks, kmax, p.idx, p.map, p.nidx, p.nb, mats, p.mstride, b, x, u, p.ustride, scal,
-      vstride);
+  const dim3 grid((unsigned)cdiv64(tasks, tp), nmodes);
+  // FP32 solves of whole components, at depths of at most one CTA of 256 threads an
+  // SM: 2D n = 8 (nine components) 478 -> 397 us, an ensemble of them 12.7 ms either
+  // way.  At every depth the early CTAs take room from other components: the
+  // ensemble 13.3 ms, 2D n = 12 17.8 -> 18.2 ms; at up to two CTAs an SM the
+  // ensemble 13.0 ms.
+  const bool ahead = sizeof(R) == 4 && scal == nullptr && (int64_t)grid.x * grid.y * threads <= 152 * 256;
+  auto kern = ahead ? k_nd_level<R, UP, sizeof(R) == 4> : k_nd_level<R, UP, false>;
+  if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int lf = leaf ? 1 : 0;
+  if (ahead)
+    launch_overlapped(kern, grid, threads, smem, s, L, lf, cu, cb, g, chunks, kmax, p.idx, p.map, p.nidx, p.nb, mats,
+                      p.mstride, b, x, u, p.ustride, scal, vstride);
+  else
+    kern<<<grid, threads, smem, s>>>(L, lf, cu, cb, g, chunks, kmax, p.idx, p.map, p.nidx, p.nb, mats, p.mstride, b, x,
+                                     u, p.ustride, scal, vstride);
 }
 
 }  // namespace
