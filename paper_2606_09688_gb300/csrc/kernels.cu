@@ -275,6 +275,139 @@ __global__ void __launch_bounds__(256) k_stencil_tile2(Geo g, StencilCoefT<R> sc
   }
 }
 
+// 3D variant streaming along the third direction (FP32): a CTA owns a column of
+// 32 x 8 interior nodes of one mode and walks `rows` planes.  A plane of x, with
+// its halo of one node, is in shared memory; a thread reads its 3 x 3 values once
+// and adds their part of the stencil to the three planes they belong to: the
+// running sums of planes p (ak0) and p + 1 (ak1), the finished plane p - 1 leaves.
+// The weights towards the cell layer between two planes serve both of them
+// (the element matrix is even in each direction), and the mass is the tensor
+// (1, 4, 1)^3 m0.  Loads of x, b and c^2 run one plane ahead.  The one-thread-a-node
+// kernel is bound by its 27 loads a node and mode (1.3 TB/s and 11 TFLOP/s of a
+// Jacobi sweep on 127^3); here a node costs 9 shared-memory reads, one load each of
+// x and b and about 140 instructions.  3D n = 10, FP32: component (7,3), 127^3 and
+// 5 modes, 42.7 -> 32.0 ms, (6,4), 63^3 and 9 modes, 33.1 -> 29.3 ms.
+constexpr int kPlaneX = 32, kPlaneY = 8, kPlaneMin = 24;
+template <typename R, int OP>
+__global__ void __launch_bounds__(kPlaneX * kPlaneY, 3)
+    k_stencil_plane3(Geo g, StencilCoefT<R> sc, const R* __restrict__ c2, const cx<R>* __restrict__ x,
+                     const cx<R>* __restrict__ b, cx<R>* __restrict__ y, const cx<R>* __restrict__ lam,
+                     const CocgScal* __restrict__ scal, int64_t stride, R omega, int tiles_x, int rows) {
+  constexpr int HX = kPlaneX + 2, HY = kPlaneY + 2, NH = 2 * HX + 2 * kPlaneY;  // halo nodes of a plane
+  __shared__ cx<R> xs[2][HY][HX];
+  const int q = blockIdx.z;
+  if (scal != nullptr && !scal[q].active) return;
+  const int n = g.n, N = g.N, tid = threadIdx.x, tx = tid % kPlaneX, ty = tid / kPlaneX;
+  const int x0 = (blockIdx.x % tiles_x) * kPlaneX, y0 = (blockIdx.x / tiles_x) * kPlaneY;
+  const int ix = x0 + tx, iy = y0 + ty;
+  const int z0 = blockIdx.y * rows, z1 = min(z0 + rows, n);
+  const bool node = ix < n && iy < n;
+  // the halo node that threads 0 .. NH-1 also load: rows y0 - 1 and y0 + kPlaneY, then the two side columns
+  int hx = 0, hy = 0;
+  if (tid < HX) {
+    hx = tid;
+  } else if (tid < 2 * HX) {
+    hx = tid - HX;
+    hy = HY - 1;
+  } else {
+    const int t = tid - 2 * HX;
+    hx = t < kPlaneY ? 0 : HX - 1;
+    hy = 1 + t % kPlaneY;
+  }
+  const bool halo = tid < NH;
+  const bool hok = halo && x0 + hx >= 1 && x0 + hx <= n && y0 + hy >= 1 && y0 + hy <= n;
+  const int64_t np = (int64_t)n * n;
+  const cx<R>* xq = x + (int64_t)q * stride;
+  const int64_t on = (int64_t)iy * n + ix, oh = (int64_t)(y0 + hy - 1) * n + (x0 + hx - 1);
+  const cx<R>* bq = b + (int64_t)q * stride + on;
+  cx<R>* yq = y + (int64_t)q * stride + on;
+  const cx<R> zero = mk<R>(0, 0), l = lam[q];
+  auto ldx = [&](bool ok, int64_t o, int p) -> cx<R> { return (ok && p >= 0 && p < n) ? xq[p * np + o] : zero; };
+  // the four cells around the node's edge in cell layer p (between node planes p - 1 and p)
+  auto ldc = [&](int p, R c[4]) {
+    const bool ok = node && p >= 0 && p < N;
+    const R* cp = c2 + ((int64_t)p * N + iy) * N + ix;
+    c[0] = ok ? __ldg(cp) : R(0);
+    c[1] = ok ? __ldg(cp + 1) : R(0);
+    c[2] = ok ? __ldg(cp + N) : R(0);
+    c[3] = ok ? __ldg(cp + N + 1) : R(0);
+  };
+  // sums of the cells shared with each of the 3 x 3 neighbours, times weights k
+  auto weights = [](const R c[4], const R* k, R w[9]) {
+    const R lo = c[0] + c[1], hi = c[2] + c[3];
+    w[0] = k[0] * c[0];
+    w[1] = k[1] * lo;
+    w[2] = k[2] * c[1];
+    w[3] = k[3] * (c[0] + c[2]);
+    w[4] = k[4] * (lo + hi);
+    w[5] = k[5] * (c[1] + c[3]);
+    w[6] = k[6] * c[2];
+    w[7] = k[7] * hi;
+    w[8] = k[8] * c[3];
+  };
+  auto dot9 = [](const R w[9], const cx<R> v[9], cx<R> a0) -> cx<R> {
+    const cx<R> s0 = fma_s(w[2], v[2], fma_s(w[1], v[1], fma_s(w[0], v[0], a0)));
+    const cx<R> s1 = fma_s(w[5], v[5], fma_s(w[4], v[4], w[3] * v[3]));
+    const cx<R> s2 = fma_s(w[8], v[8], fma_s(w[7], v[7], w[6] * v[6]));
+    return (s0 + s1) + s2;
+  };
+  // plane z0 - 1 into buffer 0; its lower layer's sums are never used
+  xs[0][ty + 1][tx + 1] = ldx(node, on, z0 - 1);
+  if (halo) xs[0][hy][hx] = ldx(hok, oh, z0 - 1);
+  R cl[4], cu[4], wl[9];
+  ldc(z0 - 1, cl);
+  ldc(z0, cu);
+  weights(cl, sc.ke, wl);
+  const R m0 = sc.mtot[0], mc = sc.mtot[13], m4 = R(4) * m0;
+  cx<R> ak0 = zero, ak1 = zero, h0 = zero, h1 = zero, xc = zero, bn = zero;
+  R kc = R(0);  // stiffness diagonal of plane p - 1
+  __syncthreads();
+  for (int p = z0 - 1; p <= z1; ++p) {
+    const int buf = (p - z0 + 1) & 1;
+    // one plane ahead: x of plane p + 1, b of plane p, the cells above plane p + 1
+    const cx<R> xn = ldx(node && p < z1, on, p + 1), xh = ldx(hok && p < z1, oh, p + 1);
+    const cx<R> bp = (OP != OP_APPLY && node && p >= z0 && p < z1) ? bq[p * np] : zero;
+    R cn[4];
+    ldc(p + 2, cn);
+    cx<R> v[9];
+#pragma unroll
+    for (int s = 0; s < 9; ++s) v[s] = xs[buf][ty + s / 3][tx + s % 3];
+    const cx<R> r0 = fma_s(R(4), v[1], v[0] + v[2]), r1 = fma_s(R(4), v[4], v[3] + v[5]),
+                r2 = fma_s(R(4), v[7], v[6] + v[8]);
+    const cx<R> h = fma_s(R(4), r1, r0 + r2);
+    const cx<R> fin = dot9(wl, v, ak0);
+    if (p > z0 && node) {
+      const int64_t o = (int64_t)(p - 1) * np;
+      const cx<R> am = fma_s(m4, h1, m0 * (h0 + h));
+      const cx<R> Ax = fma_c(l, am, fin);
+      if (OP == OP_APPLY) yq[o] = Ax;
+      else if (OP == OP_RESID) yq[o] = bn - Ax;
+      else yq[o] = xc + scaled_div(omega, bn - Ax, fma_s(mc, l, mk<R>(kc, R(0))));
+    }
+    R wm[9];
+    {
+      const R cs[4] = {cl[0] + cu[0], cl[1] + cu[1], cl[2] + cu[2], cl[3] + cu[3]};
+      weights(cs, sc.ke + 9, wm);
+    }
+    weights(cu, sc.ke, wl);  // towards plane p + 1, and from there back
+    ak0 = dot9(wm, v, ak1);
+    ak1 = dot9(wl, v, zero);
+    h0 = h1;
+    h1 = h;
+    xc = v[4];
+    kc = wm[4];
+    bn = bp;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      cl[k] = cu[k];
+      cu[k] = cn[k];
+    }
+    xs[buf ^ 1][ty + 1][tx + 1] = xn;
+    if (halo) xs[buf ^ 1][hy][hx] = xh;
+    __syncthreads();
+  }
+}
+
 // 2D variant streaming down columns: a warp owns 30 consecutive columns of
 // interior nodes (its lanes 0 and 31 hold the halo columns) and walks a strip
 // of `rows` rows (as many strips as fill the device once).  The x values of
@@ -575,6 +708,35 @@ template <typename R> bool mass_separable(const StencilCoefT<R>& sc) {
   return true;
 }
 
+// The plane-streaming 3D kernel's assumptions: mass in tensor form, element
+// stiffness even in the third direction.  Taken for every launch shape from
+// kPlaneMin nodes a side: 31^3 leaves one of 32 lanes idle, coarser grids more than
+// half of the 32 x 8 tile.
+template <typename R> bool plane3_ok(const Geo& g, const StencilCoefT<R>& sc) {
+  if (sizeof(R) != 4 || g.d != 3 || g.n < kPlaneMin) return false;
+  const R m0 = sc.mtot[0];
+  const R w[3] = {R(1), R(4), R(1)};
+  for (int s = 0; s < 27; ++s)
+    if (sc.mtot[s] != m0 * w[s % 3] * w[s / 3 % 3] * w[s / 9]) return false;
+  for (int s = 0; s < 9; ++s)
+    if (sc.ke[s] != sc.ke[s + 18]) return false;
+  return true;
+}
+
+template <typename R>
+void stencil_plane3(int op, const Geo& g, const StencilCoefT<R>& sc, const R* c2, const cx<R>* x, const cx<R>* b,
+                    cx<R>* y, const cx<R>* lam, const CocgScal* scal, int nmodes, int64_t stride, double omega,
+                    cudaStream_t s) {
+  const int tx = (g.n + kPlaneX - 1) / kPlaneX, ty = (g.n + kPlaneY - 1) / kPlaneY;
+  // planes per CTA: a chunk pays two more planes, so long ones, but some six CTAs per SM
+  int rows = g.n;
+  while (rows > 8 && (int64_t)tx * ty * nmodes * ((g.n + rows - 1) / rows) < 6 * 152) rows = (rows + 1) / 2;
+  const dim3 grid(tx * ty, (g.n + rows - 1) / rows, nmodes);
+  auto kern = op == OP_APPLY ? k_stencil_plane3<R, OP_APPLY>
+                             : (op == OP_RESID ? k_stencil_plane3<R, OP_RESID> : k_stencil_plane3<R, OP_JACOBI>);
+  kern<<<grid, kPlaneX * kPlaneY, 0, s>>>(g, sc, c2, x, b, y, lam, scal, stride, (R)omega, tx, rows);
+}
+
 // block == 0 selects the shared-memory tile kernel, block == kColBlockCode the
 // column-streaming kernel (both 2D, operations that read x).
 constexpr int kColBlockCode = 64;
@@ -594,6 +756,12 @@ void stencil_launch_shape(int op, const Geo& g, const StencilCoefT<R>& sc, const
     else if (sh.mq == 2) stencil_col2_mq<R, 2>(op, g, sc, c2, x, b, y, lam, scal, nmodes, stride, omega, s);
     else stencil_col2_mq<R, 1>(op, g, sc, c2, x, b, y, lam, scal, nmodes, stride, omega, s);
     return;
+  }
+  if constexpr (D == 3 && sizeof(R) == 4) {
+    if (op != OP_JACOBI_ZERO && plane3_ok(g, sc)) {
+      stencil_plane3(op, g, sc, c2, x, b, y, lam, scal, nmodes, stride, omega, s);
+      return;
+    }
   }
   if (sh.mq == 4 && D < 3)
     stencil_dispatch_mq<D, R, (D < 3 ? 4 : 1)>(op, g, sc, c2, x, b, y, lam, scal, nmodes, stride, omega, sh.block, s);
