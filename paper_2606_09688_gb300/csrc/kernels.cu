@@ -1480,66 +1480,131 @@ __global__ void k_gemm_right(const double* __restrict__ X, const double* __restr
   }
 }
 
-// Banded LU solve with partial pivoting (factor layout of band_lu, spatial
-// mode fastest), one thread per spatial mode, Y column a (stride nx) in place.
-// Banded LU solves (A + mu_a B) y_a = r_a, one spatial mode a per CTA: the
-// mode's factor (mode-major: column j of the band at j * ld, the diagonal
-// stored as its reciprocal), pivots and right-hand side are staged in shared
-// memory, then one thread runs the forward (row interchanges, unit lower
-// factor, kl sub-diagonals) and backward (upper factor, kl + ku
-// super-diagonals) recurrences on a register window of the rows in reach, so
-// each step waits on two shared-memory loads and its own multiply-adds.
+// Banded LU solves (A + mu_a B) y_a = r_a with partial pivoting (factor layout of
+// band_lu, spatial mode fastest in Y, in place), one spatial mode a per CTA: the
+// mode's factor (mode-major: column j of the band at j * ld, the diagonal stored
+// as its reciprocal), pivots and right-hand side are staged in shared memory, then
+// one thread runs the forward (row interchanges, unit lower factor, kl
+// sub-diagonals) and backward (upper factor, kl + ku super-diagonals) recurrences
+// on a register window of the rows in reach.  Bound by that chain: one dependent
+// multiply-add a row forward, a product and a multiply-add backward.  Its operands
+// are read a group of rows ahead (before the group's stores, which the compiler may
+// not move loads across), and rows of zeros on both sides stand in for the tests
+// at the ends: 1D n = 13 (1025 rows on the longest component) 674 -> 633 us a pass,
+// a component of 9 modes and 1025 rows alone 392 -> 363 us.
+constexpr int kTimeBandPad = 16;   // rows of zeros on either side
+constexpr int kTimeBandGroup = 4;  // rows whose operands are read ahead
 template <int KL, int KU>
 __global__ void __launch_bounds__(128) k_time_band_solve(const double* __restrict__ ab, const int* __restrict__ piv,
                                                          double* __restrict__ Y, int nt, int64_t nx) {
-  constexpr int KV = KL + KU, LD = 2 * KL + KU + 1;
+  constexpr int KV = KL + KU, LD = 2 * KL + KU + 1, PAD = kTimeBandPad, G = kTimeBandGroup;
+  static_assert(PAD >= 2 * G + KV, "the last group and the one read ahead of it stay within the padding");
   extern __shared__ __align__(16) unsigned char tb_smem[];
-  double* sa = reinterpret_cast<double*>(tb_smem);  // nt x LD
-  double* sy = sa + (size_t)nt * LD;                // nt
-  int* sp = reinterpret_cast<int*>(sy + nt);        // nt
+  const int rows = nt + 2 * PAD;
+  double* sa = reinterpret_cast<double*>(tb_smem);  // rows x LD
+  double* sy = sa + (size_t)rows * LD;              // rows
+  int* sp = reinterpret_cast<int*>(sy + rows);      // rows: interchange with row j + sp[j]
   const int64_t a = blockIdx.x;
   const double* aba = ab + a * (int64_t)nt * LD;
-  for (int e = threadIdx.x; e < nt * LD; e += blockDim.x) sa[e] = aba[e];
-  for (int j = threadIdx.x; j < nt; j += blockDim.x) {
-    sp[j] = piv[a * nt + j];
-    sy[j] = Y[(int64_t)j * nx + a];
+  for (int e = threadIdx.x; e < rows * LD; e += blockDim.x) {
+    const int s = e - PAD * LD;
+    sa[e] = (s >= 0 && s < nt * LD) ? aba[s] : 0.0;
+  }
+  for (int e = threadIdx.x; e < rows; e += blockDim.x) {
+    const int j = e - PAD;
+    const bool in = j >= 0 && j < nt;
+    sp[e] = in ? piv[a * nt + j] - j : 0;
+    sy[e] = in ? Y[(int64_t)j * nx + a] : 0.0;
   }
   __syncthreads();
+  sa += PAD * LD + KV;  // sa[j * LD + i - j] = A(i, j)
+  sy += PAD;
+  sp += PAD;
   if (threadIdx.x == 0) {
-    // forward: window w[0..KL] = rows j .. j+KL
-    double w[KL + 1];
+    {  // forward: window w[0..KL] = rows j .. j+KL
+      double w[KL + 1], c[G][KL], in[G];
+      int p[G];
 #pragma unroll
-    for (int t = 0; t <= KL; ++t) w[t] = t < nt ? sy[t] : 0.0;
-    for (int j = 0; j < nt; ++j) {
-      const int p = sp[j] - j;  // 0 .. KL
-      double yj = w[0];
+      for (int t = 0; t <= KL; ++t) w[t] = sy[t];
 #pragma unroll
-      for (int t = 1; t <= KL; ++t) {
-        const double wt = w[t];
-        w[t] = (p == t) ? yj : wt;
-        yj = (p == t) ? wt : yj;
+      for (int u = 0; u < G; ++u) {
+        p[u] = sp[u];
+        in[u] = sy[u + KL + 1];
+#pragma unroll
+        for (int t = 0; t < KL; ++t) c[u][t] = sa[u * LD + t + 1];
       }
-      const double* col = sa + (size_t)j * LD + KV;  // col[i - j] = A(i, j)
+      for (int j0 = 0; j0 < nt; j0 += G) {
+        double cn[G][KL], inn[G];
+        int pn[G];
 #pragma unroll
-      for (int t = 1; t <= KL; ++t) w[t] = (j + t < nt) ? fma(-col[t], yj, w[t]) : w[t];
-      sy[j] = yj;
+        for (int u = 0; u < G; ++u) {
+          const int j = j0 + G + u;
+          pn[u] = sp[j];
+          inn[u] = sy[j + KL + 1];
 #pragma unroll
-      for (int t = 0; t < KL; ++t) w[t] = w[t + 1];
-      w[KL] = (j + KL + 1 < nt) ? sy[j + KL + 1] : 0.0;
+          for (int t = 0; t < KL; ++t) cn[u][t] = sa[j * LD + t + 1];
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          double yj = w[0];
+#pragma unroll
+          for (int t = 1; t <= KL; ++t) {
+            const double wt = w[t];
+            w[t] = (p[u] == t) ? yj : wt;
+            yj = (p[u] == t) ? wt : yj;
+          }
+#pragma unroll
+          for (int t = 1; t <= KL; ++t) w[t] = fma(-c[u][t - 1], yj, w[t]);
+          sy[j0 + u] = yj;
+#pragma unroll
+          for (int t = 0; t < KL; ++t) w[t] = w[t + 1];
+          w[KL] = in[u];
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          p[u] = pn[u];
+          in[u] = inn[u];
+#pragma unroll
+          for (int t = 0; t < KL; ++t) c[u][t] = cn[u][t];
+        }
+      }
     }
-    // backward: window w[0..KV] = rows j, j-1, .., j-KV
-    double v[KV + 1];
+    {  // backward: window v[0..KV] = rows j, j-1, .., j-KV
+      double v[KV + 1], c[G][KV + 1], in[G];
 #pragma unroll
-    for (int t = 0; t <= KV; ++t) v[t] = (nt - 1 - t >= 0) ? sy[nt - 1 - t] : 0.0;
-    for (int j = nt - 1; j >= 0; --j) {
-      const double* col = sa + (size_t)j * LD + KV;  // col[i - j] = A(i, j), col[0] = 1 / A(j, j)
-      const double yj = v[0] * col[0];
-      sy[j] = yj;
+      for (int t = 0; t <= KV; ++t) v[t] = sy[nt - 1 - t];
 #pragma unroll
-      for (int t = 1; t <= KV; ++t) v[t] = (j - t >= 0) ? fma(-col[-t], yj, v[t]) : v[t];
+      for (int u = 0; u < G; ++u) {
+        in[u] = sy[nt - 1 - u - KV - 1];
 #pragma unroll
-      for (int t = 0; t < KV; ++t) v[t] = v[t + 1];
-      v[KV] = (j - KV - 1 >= 0) ? sy[j - KV - 1] : 0.0;
+        for (int t = 0; t <= KV; ++t) c[u][t] = sa[(nt - 1 - u) * LD - t];
+      }
+      for (int j0 = nt - 1; j0 >= 0; j0 -= G) {
+        double cn[G][KV + 1], inn[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          const int j = j0 - G - u;
+          inn[u] = sy[j - KV - 1];
+#pragma unroll
+          for (int t = 0; t <= KV; ++t) cn[u][t] = sa[j * LD - t];
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          const double yj = v[0] * c[u][0];  // the diagonal's reciprocal
+          sy[j0 - u] = yj;
+#pragma unroll
+          for (int t = 1; t <= KV; ++t) v[t] = fma(-c[u][t], yj, v[t]);
+#pragma unroll
+          for (int t = 0; t < KV; ++t) v[t] = v[t + 1];
+          v[KV] = in[u];
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          in[u] = inn[u];
+#pragma unroll
+          for (int t = 0; t <= KV; ++t) c[u][t] = cn[u][t];
+        }
+      }
     }
   }
   __syncthreads();
@@ -2388,7 +2453,9 @@ void launch_refine_decide(RefineRec* rec, const double* nrm2, const double* fn2,
   k_refine_decide<<<1, 32, 0, s>>>(rec, nrm2, fn2, snorm, tol, max_sweeps, scal, nsel, cerr, h, it);
 }
 
-size_t time_band_smem(int nt) { return (size_t)nt * (7 * sizeof(double) + sizeof(double) + sizeof(int)); }
+size_t time_band_smem(int nt) {
+  return (size_t)(nt + 2 * kTimeBandPad) * (7 * sizeof(double) + sizeof(double) + sizeof(int));
+}
 
 bool launch_time_band_solve(const double* ab, const int* piv, double* Y, int nt, int64_t nx, int kl, int ku,
                             cudaStream_t s) {
