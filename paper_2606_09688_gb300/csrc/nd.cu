@@ -520,12 +520,12 @@ void nd_level(const NdPlan& p, int t, const cx<R>* mats, const cx<R>* b, cx<R>* 
   const int64_t cu = leaf ? 0 : p.lv[t + 1].u;
   const int cb = leaf ? 0 : p.lv[t + 1].bmax;
   const dim3 grid((unsigned)cdiv64(tasks, tp), nmodes);
-  // FP32 solves of whole components, at depths of at most one CTA of 256 threads an
-  // SM: 2D n = 8 (nine components) 478 -> 397 us, an ensemble of them 12.7 ms either
-  // way.  At every depth the early CTAs take room from other components: the
-  // ensemble 13.3 ms, 2D n = 12 17.8 -> 18.2 ms; at up to two CTAs an SM the
+  // FP32, at depths of at most one CTA of 256 threads an SM: 2D n = 8 (nine
+  // components) 478 -> 397 us, and with the coarse solves of multigrid an ensemble
+  // 12.9 -> 12.4 ms.  At every depth the early CTAs take room from other components:
+  // the ensemble 13.3 ms, 2D n = 12 17.8 -> 18.2 ms; at up to two CTAs an SM the
   // ensemble 13.0 ms.
-  const bool ahead = sizeof(R) == 4 && scal == nullptr && (int64_t)grid.x * grid.y * threads <= 152 * 256;
+  const bool ahead = sizeof(R) == 4 && (int64_t)grid.x * grid.y * threads <= 152 * 256;
   auto kern = ahead ? k_nd_level<R, UP, sizeof(R) == 4> : k_nd_level<R, UP, false>;
   if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int lf = leaf ? 1 : 0;
