@@ -68,7 +68,7 @@ def parse():
     ap.add_argument("--inner-tol", type=float, default=0.0,
                     help="inner Krylov tolerance per refinement sweep (0 = library default)")
     ap.add_argument("--max-direct-rows", type=int, default=0,
-                    help="largest spatial grid solved by the banded direct method (0 = library default)")
+                    help="largest spatial grid solved directly (nested dissection) (0 = library default)")
     ap.add_argument("--only-component", type=int, default=-1,
                     help="profiling aid: each step solves only this component (no combination)")
     ap.add_argument("--target", default="",

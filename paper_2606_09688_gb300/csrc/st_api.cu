@@ -8,8 +8,8 @@
 // conjugate modes folded (U = sum_real V_q x_q + 2 Re sum_pairs V_q x_q).
 // Each spatial problem is complex symmetric; it is solved by COCG with a
 // geometric multigrid V-cycle whose coarsest grid resolves the mode's wave
-// number and is solved by a banded LDL^T, or by the banded LDL^T alone on
-// small grids.
+// number and is solved directly (nested dissection or an explicit inverse), or
+// by nested dissection alone on small grids.
 // Space eigenbasis method (fine time levels): K Phi = M Phi diag(mu),
 // Phi^T M Phi = I, so Y = F Phi, (A + mu_a B) c_a = y_a (banded LU),
 // U = C Phi^T.
@@ -857,7 +857,7 @@ int choose_coarse(const st_problem& p, const Component& c, int64_t max_direct) {
     const Geo g = make_geo(p.d, j);
     return g.nnodes <= kMaxCoarseRows && fits(j);
   };
-  int jmax = 1;  // largest level the coarse banded solve handles
+  int jmax = 1;  // largest level the coarse direct solve handles
   while (jmax + 1 <= c.jx && fits_coarse(jmax + 1)) ++jmax;
   if (jc >= c.jx) return jmax;
   return std::min(jc, jmax);
