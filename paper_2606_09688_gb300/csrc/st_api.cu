@@ -77,10 +77,10 @@ constexpr int kModeTMaxNt = 129;       // time eigenbasis used up to this many t
 constexpr double kKappaFP32 = 2.0e5;   // cond(V) above which inner solves stay in FP64
 constexpr double kThetaMG = 1.25;      // coarsest-grid resolution: k h_c <= theta
 // Smoother weights and the imaginary shift (x |Re lam|) of modes the coarsest grid
-// cannot resolve.  The Q1 stencil's symbol over its diagonal takes the values
-// [1, 2] (1D), [3/4, 3/2] (2D) and [1/2, 3/2] (3D) on the frequencies that the
-// coarse grid does not hold.  One Jacobi sweep (FP64): near 2 / (min + max), the
-// minimiser of the largest damping factor there.  Two sweeps (FP32): the roots of
+// cannot resolve.  On square cells the Q1 stencil's symbol over its diagonal takes
+// the values [1, 2] (1D), [3/4, 3/2] (2D) and [1/2, 3/2] (3D) on the frequencies
+// that the coarse grid does not hold.  One Jacobi sweep (FP64): near 2 / (min + max),
+// the minimiser of the largest damping factor there.  Two sweeps (FP32): the roots of
 // the Chebyshev polynomial of that interval, mirrored after the coarse correction
 // (in 3D the larger root is cut to 1.2).  Against the single weight 0.6 (3D 0.55):
 // 2D n = 12 FP64 44 -> 41.4 ms, FP32 20.3 -> 19.0 ms a step; 3D n = 10 101 -> 94 ms; and
@@ -89,11 +89,22 @@ constexpr double kThetaMG = 1.25;      // coarsest-grid resolution: k h_c <= the
 // spectrum that these weights amplify wins (3D 63^3 x 33 rows, k h_c = 4.8, FP32: no
 // convergence, against 88 iterations), so such components keep the damped
 // weights and the larger shift.
+// On other cells the largest eigenvalue s of one cell's stiffness over its diagonal
+// (cell_bound), which bounds the symbol for every c^2, tends to 3 (2D) and 9/2
+// (3D), and a sweep of weight w amplifies from s = 2 / w on.  The FP64 weight is
+// therefore cut to kStable64 / s and the FP32 pair scaled by kStable32 / s; where that
+// gains less than a tenth on the damped weights (2D: below 2 / 3, safe for every
+// cell) these are taken.  At the edge of stability a sweep damps too little, hence
+// bounds below 2.  Iterations of 127^2, 5 rows, variable c^2, FP64 / FP32, at cell
+// ratios 1.5, 2, 8/3: square weights 18 / 7, then none within 1000; damped weights
+// 15 / 5, 20 / 6, 26 / 8; this rule 14 / 4, 19 / 6, 26 / 8.  511^2 at 2: none -> 19 / 5; 3D plates
+// 1.5 : 1.5 : 1 of 31^3, 3 rows: 347 / none -> 14 / 4 (damped 15 / 4).
 struct Smoother {
-  double w64[3], w32[3][2], shift;
+  double w64, w32[2], shift;
 };
-constexpr Smoother kSmooth = {{0.667, 0.85, 0.9}, {{0.54, 0.872}, {0.72, 1.163}, {0.7, 1.2}}, 0.2};
-constexpr Smoother kSmoothWeak = {{0.6, 0.6, 0.55}, {{0.6, 0.6}, {0.6, 0.6}, {0.55, 0.55}}, 0.5};
+constexpr Smoother kSmooth[3] = {{0.667, {0.54, 0.872}, 0.2}, {0.85, {0.72, 1.163}, 0.2}, {0.9, {0.7, 1.2}, 0.2}};
+constexpr Smoother kSmoothWeak[3] = {{0.6, {0.6, 0.6}, 0.5}, {0.6, {0.6, 0.6}, 0.5}, {0.55, {0.55, 0.55}, 0.5}};
+constexpr double kStable64 = 1.6, kStable32 = 1.8;
 constexpr double kKappaWeak = 2.5;
 constexpr int kIterPerGraph = 4;  // COCG iterations between host convergence checks
 
@@ -266,7 +277,7 @@ struct Component {
   cx<double>* lamP64 = nullptr;
   cx<float>* lamP32 = nullptr;
   int nshifted = 0;
-  const Smoother* smooth = &kSmooth;
+  Smoother smooth{};
   double* abT = nullptr;  // LU of (A + mu B)^T per spatial mode (adjoint systems)
   int* pivT = nullptr;
   int kl = 2, ku = 2;
@@ -823,6 +834,40 @@ st_status setup_time_level(st_handle* h, int jt, TimeData& td) {
   return ST_OK;
 }
 
+// Largest eigenvalue of D^{-1} K of one Q1 cell of widths h, D the diagonal of its
+// stiffness K.  The eigenvectors are tensor products of constant and alternating
+// vectors: 1D stiffness 0 and 2 / h, 1D mass h / 2 and h / 6.
+double cell_bound(int d, const double* h) {
+  double diag = 0.0, best = 0.0;
+  for (int set = 1; set < (1 << d); ++set) {  // the alternating directions
+    double lam = 0.0;
+    for (int k = 0; k < d; ++k) {
+      if (!((set >> k) & 1)) continue;
+      double t = 2.0 / (h[k] * h[k]);
+      for (int l = 0; l < d; ++l)
+        if (l != k) t *= ((set >> l) & 1) ? 1.0 / 6.0 : 0.5;
+      lam += t;
+    }
+    best = std::max(best, lam);
+  }
+  for (int k = 0; k < d; ++k) diag += std::pow(3.0, 1 - d) / (h[k] * h[k]);
+  return best / diag;
+}
+
+// Smoother of a component whose modes reach k h_c = kappa on the coarsest grid.
+Smoother smoother_of(int d, const double* h, double kappa) {
+  const Smoother& weak = kSmoothWeak[d - 1];
+  if (kappa > kKappaWeak) return weak;
+  Smoother s = kSmooth[d - 1];
+  if (d == 1) return s;  // every 1D cell has the bound 2
+  const double bound = cell_bound(d, h), f = std::min(1.0, kStable32 / bound);
+  s.w64 = std::max(std::min(s.w64, kStable64 / bound), weak.w64);
+  for (int k = 0; k < 2; ++k) s.w32[k] *= f;
+  if (s.w32[0] + s.w32[1] < 1.1 * (weak.w32[0] + weak.w32[1]))
+    for (int k = 0; k < 2; ++k) s.w32[k] = weak.w32[k];
+  return s;
+}
+
 // Coarsest multigrid level of a time-eigenbasis component: the coarsest grid
 // must resolve the largest wave number k = sqrt(-Re lam / min c^2) of its
 // modes (k h_c <= theta); grids with at most max_direct unknowns (default
@@ -1055,13 +1100,13 @@ st_status setup_component(st_handle* h, Component& c) {
     double kmax = 0.0;
     for (int q = 0; q < c.nsel; ++q)
       kmax = std::max(kmax, std::sqrt(std::max(0.0, -c.td->eig.lam[q].real()) / c.sl->c2min));
-    c.smooth = kmax * hc > kKappaWeak ? &kSmoothWeak : &kSmooth;
+    c.smooth = smoother_of(p.d, c.sl->h, kmax * hc);
     for (int q = 0; q < c.nsel; ++q) {
       const std::complex<double> l = c.td->eig.lam[q];
       double im = l.imag();
       const double kq = std::sqrt(std::max(0.0, -l.real()) / c.sl->c2min);
       if (!c.direct && kq * hc > kThetaMG) {
-        im += (im >= 0.0 ? 1.0 : -1.0) * c.smooth->shift * std::fabs(l.real());
+        im += (im >= 0.0 ? 1.0 : -1.0) * c.smooth.shift * std::fabs(l.real());
         ++c.nshifted;
       }
       lp[q] = mk(l.real(), im);
@@ -1211,7 +1256,7 @@ template <typename R> st_status prepare_work(st_handle* h, Component& c) {
       MGLevel& lv = c.mg[l];
       cx<R>* dv = h->alloc<cx<R>>((size_t)c.nsel * lv.geo.nnodes);
       ST_NEED(h, dv);
-      launch_jacobi_dinv<R>(lv.geo, lv.sc, lv.c2d, c.lamP64, c.smooth->w64[lv.geo.d - 1], c.nsel, lv.geo.nnodes, dv, c.cs);
+      launch_jacobi_dinv<R>(lv.geo, lv.sc, lv.c2d, c.lamP64, c.smooth.w64, c.nsel, lv.geo.nnodes, dv, c.cs);
       lv.sc.dinv = dv;
     }
   }
@@ -1285,7 +1330,7 @@ cx<R>* vcycle(st_handle* h, Component& c, int l, const cx<R>* b, cx<R>* xa, cx<R
     }
     return xb;
   }
-  const double om = c.smooth->w64[lv.geo.d - 1];
+  const double om = c.smooth.w64;
   const R* c2 = c2_of<R>(lv);
   const double cb = (double)lv.geo.ncells * rs;
   const MGLevel& lc = c.mg[l + 1];
@@ -1310,7 +1355,7 @@ cx<R>* vcycle(st_handle* h, Component& c, int l, const cx<R>* b, cx<R>* xa, cx<R
     return xa;
   }
   // FP32 inner solves are bound by latency and launches: V(2,2), fewer iterations
-  const double w1 = c.smooth->w32[lv.geo.d - 1][0], w2 = c.smooth->w32[lv.geo.d - 1][1];
+  const double w1 = c.smooth.w32[0], w2 = c.smooth.w32[1];
   PROF(h, s, KC_JACOBI, (int64_t)(n), m * n * 2 * cs + cb, m * n * 30.0,
        launch_stencil<R>(OP_JACOBI_ZERO, lv.geo, coef_of<R>(lv), c2, nullptr, b, xa, lam, c.scal, c.nsel, n, w1, s));
   PROF(h, s, KC_JACOBI, (int64_t)(n), m * n * 3 * cs + cb, m * n * (fl + 30.0),
@@ -1404,7 +1449,7 @@ template <typename R> st_status tune_component(st_handle* h, Component& c) {
     const size_t bytes = (size_t)c.nsel * n * sizeof(cx<R>);
     ST_CUDAC(c, cudaMemsetAsync(x, 0, bytes, c.cs));
     ST_CUDAC(c, cudaMemsetAsync(b, 0, bytes, c.cs));
-    const double om = c.smooth->w64[lv.geo.d - 1];
+    const double om = c.smooth.w64;
     const R* c2 = c2_of<R>(lv);
     const int ops[4] = {OP_JACOBI_ZERO, OP_JACOBI, OP_RESID, OP_APPLY};
     for (int op : ops) {
