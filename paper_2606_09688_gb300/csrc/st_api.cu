@@ -23,6 +23,7 @@
 #include <cstdio>
 #include <cstring>
 #include <future>
+#include <limits>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -1387,6 +1388,22 @@ double inner_tol(const st_handle* h, size_t rsize) {
   return rsize == 8 ? 1e-11 : 1e-4;
 }
 
+// Backward error eta at which the refinement of a component stops.  FP32 factors
+// leave their error in the smooth, ill-conditioned part, which eta hardly sees: on
+// 255^2, after three sweeps with eta between 2.5e-16 and 9.9e-16, U is up to 6e-11 off,
+// and one sweep more, to eta = 2e-17, leaves 5e-15 (127^2: 1.5e-12 and 3e-15).  Grids of
+// 63^2 and 3D ones are at eta = 5e-17 and 1e-13 off after three.  So 2D and 3D components
+// solved by FP32 factors go on to the rounding unit by default: field of the layered
+// 2D medium, n = 12, FP32 + IR, four media, 4.3e-11 .. 2.0e-10 off -> 2.6e-12 .. 3.3e-11
+// (FP64 6.1e-12 .. 3.8e-11), for 17.5 -> 18.4 ms a pass; twelve media of n = 8 .. 11 12.1 ->
+// 13.0 ms.  1D ones lose more digits a sweep (2047 unknowns: three sweeps, 1.8e-10),
+// no more than with banded factors, and keep the target.
+double refine_tol(const st_handle* h, const Component& c) {
+  if (h->opt.tol > 0) return h->opt.tol;
+  const bool fp32_factors = c.method == 0 && c.direct && !c.inner64;
+  return fp32_factors && c.sl->geo.d > 1 ? std::numeric_limits<double>::epsilon() : 1e-14;
+}
+
 // COCG start: x = 0, r = g, z = B r, rho = r . z, p = z.
 template <typename R> void cocg_start(st_handle* h, Component& c) {
   Work<R>& w = work_of<R>(c);
@@ -1640,7 +1657,7 @@ st_status solve_one(st_handle* h, Component& c, const SolveIO& io, bool adjoint)
   // Refinement stops on the normwise backward error eta = ||R|| / (||S|| ||U|| + ||F||)
   // (the relative residual of an exact solution can be far above rounding
   // when S is ill-conditioned), or when a sweep no longer halves eta.
-  const double tol = h->opt.tol > 0 ? h->opt.tol : 1e-14;
+  const double tol = h->opt.tol > 0 ? h->opt.tol : 1e-14, stop = refine_tol(h, c);
   const int max_sweeps = h->opt.max_sweeps > 0 ? h->opt.max_sweeps : 8;
   c.info = st_solve_info{};
   c.info.status = ST_OK;
@@ -1682,7 +1699,7 @@ st_status solve_one(st_handle* h, Component& c, const SolveIO& io, bool adjoint)
       c.info.status = ST_ERR_NUMERIC;
       return cfail(c, ST_ERR_NUMERIC, "non-finite residual");
     }
-    if (eta <= tol || eta > 0.5 * eta_prev) break;
+    if (eta <= stop || eta > 0.5 * eta_prev) break;
     eta_prev = eta;
     Rin = c.Rv;
   }
@@ -1769,7 +1786,7 @@ template <typename R> st_status capture_direct_graph(st_handle* h, Component& c)
   step.host = c.rec_h;
   step.fn2 = c.fn2;
   step.snorm = c.Snorm;
-  step.tol = h->opt.tol > 0 ? h->opt.tol : 1e-14;
+  step.tol = refine_tol(h, c);
   step.max_sweeps = h->opt.max_sweeps > 0 ? h->opt.max_sweeps : 8;
   const SweepInput first_in{&c.rec->sweeps, io.rhs}, first_out{&c.rec->sweeps, nullptr};
   const char* where = "sweep node";
