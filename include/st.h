@@ -203,7 +203,8 @@ st_status st_combine(st_handle* h, int jx_star, int jt_star, double* out_dev);
  * the combination overlapped with the solves: each level of the hierarchical
  * combination is enqueued on the handle's stream as soon as the components it
  * adds have finished, so the coarse levels run while the largest components
- * are still being solved.  Same result, layout and errors as the two calls;
+ * are still being solved.  Same result, layout and errors as the two calls (when
+ * a solve fails, out_dev keeps what it held);
  * info (nullable) as for st_solve_component (the call then synchronises). */
 st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_dev, st_solve_info* info);
 

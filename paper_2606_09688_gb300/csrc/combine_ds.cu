@@ -39,7 +39,7 @@ template <int D, int NR, bool FINAL>
 __global__ void __launch_bounds__(kCombThreads, D == 3 ? 2 : 3)
     k_comb_ds(int j, const ds* __restrict__ Yprev, const CombCompDS* __restrict__ comps, int c0, int c1,
               const float* __restrict__ tbw, const int* __restrict__ tspan, int nts, int L, ds* __restrict__ Yp,
-              double* __restrict__ Yd, FastDiv dQ1) {
+              double* __restrict__ Yd, FastDiv dQ1, FailureGuard guard) {
   constexpr int NE = 1 << D;
   __shared__ float sw[NR > 0 ? NR : 1][kCombMaxChunk + 1][3];
   __shared__ int ssp[NR > 0 ? NR : 1][kCombMaxChunk + 1];
@@ -61,7 +61,9 @@ __global__ void __launch_bounds__(kCombThreads, D == 3 ? 2 : 3)
     sw[r][ds_][1] = tbw[row * 3 + 1];
     sw[r][ds_][2] = tbw[row * 3 + 2];
   }
+  const bool failed = FINAL && solve_failed(guard);
   __syncthreads();
+  if (FINAL && failed) return;
   const int64_t qi = (int64_t)blockIdx.x * kCombThreads + threadIdx.x;
   if (qi >= ncs) return;
   int Q[3] = {0, 0, 0};
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kCombThreads, D == 3 ? 2 : 3)
 template <int D>
 __global__ void __launch_bounds__(kCombThreads)
     k_comb_prep_ds(const double* __restrict__ U, const double* __restrict__ lift, int coef, int jx, int nt,
-                   ds* __restrict__ Uds, ds* __restrict__ Lds) {
+                   ds* __restrict__ Uds, ds* __restrict__ Lds, SolveFailure fail) {
   const int N = 1 << jx, n = N - 1;
   int64_t nx = 1, na = 1;
 #pragma unroll
@@ -216,6 +218,7 @@ __global__ void __launch_bounds__(kCombThreads)
     na *= (N + 1);
   }
   const int64_t e = (int64_t)blockIdx.x * kCombThreads + threadIdx.x;
+  if (e == 0) note_failure(fail);
   if (Uds != nullptr && e < nt * nx) {
     double v = U[e];
     if (lift != nullptr) {
@@ -237,20 +240,21 @@ __global__ void __launch_bounds__(kCombThreads)
 
 template <int D, int NR>
 void launch_ds(bool final_level, dim3 grid, int j, const ds* Yprev, const CombCompDS* comps, int c0, int c1,
-               const float* tbw, const int* tspan, int nts, int L, ds* Yp, double* Yd, FastDiv f, cudaStream_t s) {
+               const float* tbw, const int* tspan, int nts, int L, ds* Yp, double* Yd, FastDiv f, const FailureGuard& g,
+               cudaStream_t s) {
   if (final_level)
-    k_comb_ds<D, NR, true><<<grid, kCombThreads, 0, s>>>(j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f);
+    k_comb_ds<D, NR, true><<<grid, kCombThreads, 0, s>>>(j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, g);
   else
-    k_comb_ds<D, NR, false><<<grid, kCombThreads, 0, s>>>(j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f);
+    k_comb_ds<D, NR, false><<<grid, kCombThreads, 0, s>>>(j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, g);
 }
 
 template <int D>
 void launch_ds_d(int nr, bool final_level, dim3 grid, int j, const ds* Yprev, const CombCompDS* comps, int c0,
                  int c1, const float* tbw, const int* tspan, int nts, int L, ds* Yp, double* Yd, FastDiv f,
-                 cudaStream_t s) {
-  if (nr == 0) launch_ds<D, 0>(final_level, grid, j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, s);
-  else if (nr == 1) launch_ds<D, 1>(final_level, grid, j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, s);
-  else launch_ds<D, 2>(final_level, grid, j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, s);
+                 const FailureGuard& g, cudaStream_t s) {
+  if (nr == 0) launch_ds<D, 0>(final_level, grid, j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, g, s);
+  else if (nr == 1) launch_ds<D, 1>(final_level, grid, j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, g, s);
+  else launch_ds<D, 2>(final_level, grid, j, Yprev, comps, c0, c1, tbw, tspan, nts, L, Yp, Yd, f, g, s);
 }
 
 }  // namespace
@@ -276,7 +280,7 @@ int comb_ds_chunk(int d, int j, int jt_star, const int* comp_jt, int ncomp_level
 }
 
 void launch_comb_prep_ds(int d, const double* U, const double* lift, int coef, int jx, int nt, ds* Uds, ds* Lds,
-                         cudaStream_t s) {
+                         cudaStream_t s, const SolveFailure& fail) {
   note_launches(1);
   int64_t nx = 1, na = 1;
   for (int k = 0; k < d; ++k) {
@@ -285,13 +289,14 @@ void launch_comb_prep_ds(int d, const double* U, const double* lift, int coef, i
   }
   const int64_t n = (Uds != nullptr && nt * nx > na) ? nt * nx : (Lds != nullptr ? na : nt * nx);
   const unsigned blocks = (unsigned)((n + kCombThreads - 1) / kCombThreads);
-  if (d == 1) k_comb_prep_ds<1><<<blocks, kCombThreads, 0, s>>>(U, lift, coef, jx, nt, Uds, Lds);
-  else if (d == 2) k_comb_prep_ds<2><<<blocks, kCombThreads, 0, s>>>(U, lift, coef, jx, nt, Uds, Lds);
-  else k_comb_prep_ds<3><<<blocks, kCombThreads, 0, s>>>(U, lift, coef, jx, nt, Uds, Lds);
+  if (d == 1) k_comb_prep_ds<1><<<blocks, kCombThreads, 0, s>>>(U, lift, coef, jx, nt, Uds, Lds, fail);
+  else if (d == 2) k_comb_prep_ds<2><<<blocks, kCombThreads, 0, s>>>(U, lift, coef, jx, nt, Uds, Lds, fail);
+  else k_comb_prep_ds<3><<<blocks, kCombThreads, 0, s>>>(U, lift, coef, jx, nt, Uds, Lds, fail);
 }
 
 void launch_comb_level_ds(int d, int j, const void* Yprev, const CombCompDS* comps, int c0, int c1, const float* tbw,
-                          const int* tspan, int nts, int L, void* Y, bool final_level, cudaStream_t s) {
+                          const int* tspan, int nts, int L, void* Y, bool final_level, cudaStream_t s,
+                          const FailureGuard& guard) {
   note_launches(1);
   int64_t ncs = 1;  // one thread per node of level j-1 (each writes up to 2^d level-j nodes)
   for (int k = 0; k < d; ++k) ncs *= ((1 << j) / 2 + 1);
@@ -302,9 +307,9 @@ void launch_comb_level_ds(int d, int j, const void* Yprev, const CombCompDS* com
   const ds* Yp = static_cast<const ds*>(Yprev);
   ds* Ypair = final_level ? nullptr : static_cast<ds*>(Y);
   double* Yd = final_level ? static_cast<double*>(Y) : nullptr;
-  if (d == 1) launch_ds_d<1>(nr, final_level, grid, j, Yp, comps, c0, c1, tbw, tspan, nts, L, Ypair, Yd, f, s);
-  else if (d == 2) launch_ds_d<2>(nr, final_level, grid, j, Yp, comps, c0, c1, tbw, tspan, nts, L, Ypair, Yd, f, s);
-  else launch_ds_d<3>(nr, final_level, grid, j, Yp, comps, c0, c1, tbw, tspan, nts, L, Ypair, Yd, f, s);
+  if (d == 1) launch_ds_d<1>(nr, final_level, grid, j, Yp, comps, c0, c1, tbw, tspan, nts, L, Ypair, Yd, f, guard, s);
+  else if (d == 2) launch_ds_d<2>(nr, final_level, grid, j, Yp, comps, c0, c1, tbw, tspan, nts, L, Ypair, Yd, f, guard, s);
+  else launch_ds_d<3>(nr, final_level, grid, j, Yp, comps, c0, c1, tbw, tspan, nts, L, Ypair, Yd, f, guard, s);
 }
 
 }  // namespace st

@@ -1324,7 +1324,10 @@ __device__ __forceinline__ void refine_step(const RefineStep& p, double rr, doub
     more = st == RR_OK && !(r.eta <= p.tol || r.eta > 0.5 * eta_prev) && r.sweeps < p.max_sweeps;
     r.status = st;
   }
-  if (!more) *p.host = r;  // page-locked: the host reads it once the graph has ended
+  if (!more) {
+    p.rec[1] = r;
+    *p.host = r;  // page-locked: the host reads it once the graph has ended
+  }
   *p.rec = more ? r : RefineRec{};
   cudaGraphSetConditional(p.cond, more ? 1u : 0u);
 }
@@ -1691,7 +1694,9 @@ template <int D>
 __global__ void __launch_bounds__(kBlock) k_comb_level(int j, const double* __restrict__ Yprev,
                                                        const CombComp* __restrict__ comps, int c0, int c1,
                                                        const double* __restrict__ tbv, const int* __restrict__ tspan,
-                                                       int nts, int nlift, double* __restrict__ Y, FastDiv dQ1) {
+                                                       int nts, int nlift, double* __restrict__ Y, FastDiv dQ1,
+                                                       FailureGuard guard) {
+  if (solve_failed(guard)) return;
   const int s = blockIdx.y;
   const int Nj = 1 << j, Nc = Nj >> 1;
   int64_t ncs = 1, nsp = 1;
@@ -2467,17 +2472,29 @@ bool launch_time_band_solve(const double* ab, const int* piv, double* Y, int nt,
   return true;
 }
 
+__global__ void k_note_failures(const RefineRec* const* __restrict__ recs, int n, SolveFailure f) {
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    f.rec = recs[k];
+    note_failure(f);
+  }
+}
+
+void launch_note_failures(const RefineRec* const* recs, int n, const SolveFailure& f, cudaStream_t s) {
+  count(1);
+  k_note_failures<<<1, 32, 0, s>>>(recs, n, f);
+}
+
 void launch_comb_level(int d, int j, const double* Yprev, const CombComp* comps, int c0, int c1, const double* tbv,
-                       const int* tspan, int nts, double* Y, cudaStream_t s, int nlift) {
+                       const int* tspan, int nts, double* Y, cudaStream_t s, int nlift, const FailureGuard& guard) {
   count(1);
   if (nlift < 0) nlift = nts;
   int64_t ncs = 1;  // one thread per node of level j-1 (each writes up to 2^d level-j nodes)
   for (int k = 0; k < d; ++k) ncs *= ((1 << j) / 2 + 1);
   dim3 grid(blocks_for(ncs), nts);
   const FastDiv f = make_fastdiv((unsigned)((1 << j) / 2 + 1));
-  if (d == 1) k_comb_level<1><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f);
-  else if (d == 2) k_comb_level<2><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f);
-  else k_comb_level<3><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f);
+  if (d == 1) k_comb_level<1><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f, guard);
+  else if (d == 2) k_comb_level<2><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f, guard);
+  else k_comb_level<3><<<grid, kBlock, 0, s>>>(j, Yprev, comps, c0, c1, tbv, tspan, nts, nlift, Y, f, guard);
 }
 
 template <typename R>

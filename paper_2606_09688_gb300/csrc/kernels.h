@@ -121,8 +121,8 @@ struct RefineRec {
 enum { RR_OK = 0, RR_NUMERIC = 1, RR_ITER_LIMIT = 2, RR_TIMEOUT = 3 };
 // The refinement test of a component without an inner iteration, taken by the
 // last block of the residual (launch_residual): rec (device) keeps the record
-// between sweeps and is zero between solves, host (page-locked) receives it when
-// the refinement ends; fn2 = ||F||^2 (device).
+// between sweeps and is zero between solves, rec[1] and host (page-locked) receive
+// it when the refinement ends; fn2 = ||F||^2 (device).
 struct RefineStep {
   RefineRec* rec = nullptr;  // null: no test
   RefineRec* host = nullptr;
@@ -131,6 +131,31 @@ struct RefineStep {
   int max_sweeps = 0;
   cudaGraphConditionalHandle cond{};
 };
+// A solve that failed, for the kernels that the host queues behind it before it
+// knows: launch_comb_prep_ds, on the component's stream, or launch_note_failures,
+// before the target level, set *word = call where a record tells of an error (a
+// status, or a backward error above fail_eta), and the target level of a combination
+// that finds its own call there writes nothing.  Words of earlier calls need no clearing.
+struct SolveFailure {
+  const RefineRec* rec = nullptr;  // null: the host has seen the solve succeed
+  double fail_eta = 0.0;
+  unsigned* word = nullptr;
+  unsigned call = 0;
+};
+struct FailureGuard {
+  const unsigned* word = nullptr;  // null: no test
+  unsigned call = 0;
+};
+// The same for n records (null entries are skipped; f.rec is not read).
+void launch_note_failures(const RefineRec* const* recs, int n, const SolveFailure& f, cudaStream_t s);
+#ifdef __CUDACC__
+__device__ __forceinline__ void note_failure(const SolveFailure& f) {
+  if (f.rec == nullptr) return;
+  const RefineRec r = *f.rec;
+  if (r.status != RR_OK || (r.sweeps > 0 && !(r.eta <= f.fail_eta))) *f.word = f.call;
+}
+__device__ __forceinline__ bool solve_failed(const FailureGuard& g) { return g.word != nullptr && *g.word == g.call; }
+#endif
 // What the first sweep of such a refinement does otherwise: *sweep == 0 (device)
 // makes a kernel read F instead of the residual, or overwrite its result instead
 // of adding to it, so that U = 0, R = F need no passes of their own.
@@ -203,7 +228,8 @@ struct CombComp {
 // tspan[c][s] their interval.  Yprev (level j-1, all nodes x nts) may be null.
 // The lifts enter the first nlift rows s (all of them by default).
 void launch_comb_level(int d, int j, const double* Yprev, const CombComp* comps, int c0, int c1, const double* tbv,
-                       const int* tspan, int nts, double* Y, cudaStream_t s, int nlift = -1);
+                       const int* tspan, int nts, double* Y, cudaStream_t s, int nlift = -1,
+                       const FailureGuard& guard = FailureGuard{});
 // The tables of launch_comb_level for values (rows 0..nb-1) and time derivatives
 // (rows nb..2nb-1) at nb times in [0, T] (device).
 void launch_energy_tables(const CombComp* comps, int nc, const double* times, int nb, double T, double* tb, int* span,
@@ -222,9 +248,10 @@ struct CombCompDS {
   int jx, jt;
 };
 void launch_comb_prep_ds(int d, const double* U, const double* lift, int coef, int jx, int nt, ds* Uds, ds* Lds,
-                         cudaStream_t s);
+                         cudaStream_t s, const SolveFailure& fail = SolveFailure{});
 void launch_comb_level_ds(int d, int j, const void* Yprev, const CombCompDS* comps, int c0, int c1, const float* tbw,
-                          const int* tspan, int nts, int L, void* Y, bool final_level, cudaStream_t s);
+                          const int* tspan, int nts, int L, void* Y, bool final_level, cudaStream_t s,
+                          const FailureGuard& guard = FailureGuard{});
 int comb_ds_chunk(int d, int j, int jt_star, const int* comp_jt, int ncomp_level);
 
 // Coarsest multigrid level by an explicit inverse (grids of at most a few

@@ -352,6 +352,9 @@ struct st_handle {
   // the count at the last st_solve_combine, sc_parity the pair buffer its
   // successor uses, sc_done_ev[p] the end of the levels of the last call that
   // used buffer p.
+  // sc_fail[p]: the call (its api_seq) of a failed solve whose levels were queued
+  // before the host knew (SolveFailure); like buffer p it is reused only after the
+  // levels that read it.
   // nodal parametrisation of c^2 and of the first source term's g (copies)
   std::vector<double> c2_nodal, g_nodal;
   int64_t api_seq = 0;
@@ -359,8 +362,10 @@ struct st_handle {
   int sc_parity = 0;
   cudaEvent_t sc_done_ev[2] = {nullptr, nullptr};
   bool sc_done_rec[2] = {false, false};
+  unsigned* sc_fail = nullptr;
   struct CombTables {
     CombComp* comps = nullptr;  // components ordered by combination level
+    const RefineRec** recs = nullptr;  // their records, or nullptr for host-driven solves
     double* tb = nullptr;
     float* tbw = nullptr;       // the same weights as floats (exact when ds_ok)
     CombCompDS* dcomps[2] = {nullptr, nullptr};  // the components' pair arrays (two buffers), table order
@@ -1771,7 +1776,7 @@ template <typename R> st_status capture_direct_graph(st_handle* h, Component& c)
   const SolveIO io = forward_io(c);
   if (c.method == 1 && time_band_smem(c.nt) > kTimeBandMaxSmem)
     return fail(h, ST_ERR_ARG, "device solve: time band solve of this size not supported");
-  c.rec = h->alloc<RefineRec>(1);
+  c.rec = h->alloc<RefineRec>(2);  // between the sweeps, and of the last solve
   c.fn2 = h->alloc<double>(1);
   ST_NEED(h, c.rec);
   ST_NEED(h, c.fn2);
@@ -1951,6 +1956,14 @@ st_status enqueue_graph_solve(st_handle* h, Component& c) {
   return ccheck(c, "solve graph");
 }
 
+// Device record of the last graph solve.
+const RefineRec* solve_record(const Component& c) {
+  return c.g_solve == nullptr ? nullptr : (c.rec_direct ? c.rec + 1 : c.rec);
+}
+
+// The backward error above which a solve has failed.
+double fail_eta(const st_handle* h) { return std::max(1e3 * (h->opt.tol > 0 ? h->opt.tol : 1e-14), 1e-12); }
+
 // Status of a graph solve, once the host has synchronised with an event that
 // follows the record's copy: the same outcomes as the host-driven loop.
 st_status finish_graph_solve(st_handle* h, Component& c) {
@@ -1962,13 +1975,12 @@ st_status finish_graph_solve(st_handle* h, Component& c) {
   c.info.max_inner_iters = r.max_iters;
   c.info.rel_residual = r.rel;
   c.info.backward_error = r.eta;
-  const double tol = h->opt.tol > 0 ? h->opt.tol : 1e-14;
   st_status st = ST_OK;
   if (r.status == RR_TIMEOUT) st = cfail(c, ST_ERR_TIMEOUT, "a bounded copy wait in the banded solve timed out");
   else if (r.status == RR_ITER_LIMIT) st = cfail(c, ST_ERR_NOT_CONVERGED, "COCG reached its iteration limit");
   else if (r.status != RR_OK) st = cfail(c, ST_ERR_NUMERIC, "COCG breakdown or non-finite value");
   c.solved = r.status == RR_OK;
-  if (st == ST_OK && r.sweeps > 0 && r.eta > 1e3 * tol && r.eta > 1e-12)
+  if (st == ST_OK && r.sweeps > 0 && r.eta > fail_eta(h))
     st = cfail(c, ST_ERR_NOT_CONVERGED, "refinement did not reach the backward-error target");
   c.info.status = st;
   return st;
@@ -2262,13 +2274,16 @@ st_status comb_tables(st_handle* h, int jx_star, int jt_star, uint64_t mask, con
       }
       for (int b = 0; b < 2; ++b) dc[b][o] = CombCompDS{k.Uds[b], k.Lds, k.jx, k.jt};
     }
+  std::vector<const RefineRec*> recs(nc);
+  for (int o = 0; o < nc; ++o) recs[o] = solve_record(*h->comps[order[o]]);
+  t.recs = h->alloc<const RefineRec*>(nc);
   t.comps = h->alloc<CombComp>(nc);
   t.tb = h->alloc<double>(tb.size());
   t.tbw = h->alloc<float>(tbw.size());
   t.dcomps[0] = h->alloc<CombCompDS>(nc);
   t.dcomps[1] = h->alloc<CombCompDS>(nc);
   t.span = h->alloc<int>(tsp.size());
-  if (!t.comps || !t.tb || !t.tbw || !t.dcomps[0] || !t.dcomps[1] || !t.span)
+  if (!t.recs || !t.comps || !t.tb || !t.tbw || !t.dcomps[0] || !t.dcomps[1] || !t.span)
     return fail(h, ST_ERR_OOM, "device allocation failed");
   t.Y.assign(jx_star + 1, nullptr);
   for (int lev = t.jmin; lev < jx_star; ++lev) {
@@ -2277,6 +2292,7 @@ st_status comb_tables(st_handle* h, int jx_star, int jt_star, uint64_t mask, con
     t.Y[lev] = h->alloc<double>((size_t)nsp * nts);
     if (!t.Y[lev]) return fail(h, ST_ERR_OOM, "device allocation failed");
   }
+  ST_CUDA(h, cudaMemcpyAsync(t.recs, recs.data(), nc * sizeof(recs[0]), cudaMemcpyHostToDevice, h->stream));
   ST_CUDA(h, cudaMemcpyAsync(t.comps, cc.data(), nc * sizeof(CombComp), cudaMemcpyHostToDevice, h->stream));
   ST_CUDA(h, cudaMemcpyAsync(t.tb, tb.data(), tb.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   ST_CUDA(h, cudaMemcpyAsync(t.tbw, tbw.data(), tbw.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
@@ -2291,9 +2307,11 @@ st_status comb_tables(st_handle* h, int jx_star, int jt_star, uint64_t mask, con
 // One level of the hierarchical combination on the handle's stream.
 // buf: the pair buffer the level reads; prepped: the components' pairs were
 // already written into it on their own streams (st_solve_combine), otherwise
-// they are converted here on the handle's stream.
+// they are converted here on the handle's stream.  guard: no target values where
+// it finds a failed solve.
 void enqueue_comb_level(st_handle* h, const st_handle::CombTables& t, int lev, int jx_star, int jt_star,
-                        double* out_dev, int buf = 0, bool prepped = false) {
+                        double* out_dev, int buf = 0, bool prepped = false,
+                        const FailureGuard& guard = FailureGuard{}) {
   const st_problem& p = h->prob;
   const int nts = (1 << jt_star) + 1;
   const int c0 = t.first[lev], c1 = t.first[lev + 1];
@@ -2315,10 +2333,11 @@ void enqueue_comb_level(st_handle* h, const st_handle::CombTables& t, int lev, i
     const int L = comb_ds_chunk(p.d, lev, jt_star, t.jt.data() + c0, c1 - c0);
     PROF(h, h->stream, KC_COMBINE, (int64_t)(nsp), outb + inb, flops,
          launch_comb_level_ds(p.d, lev, Yp, t.dcomps[buf], c0, c1, t.tbw, t.span, nts, L, Y, lev == jx_star,
-                              h->stream));
+                              h->stream, guard));
   } else {
     PROF(h, h->stream, KC_COMBINE, (int64_t)(nsp), outb + inb, flops,
-         launch_comb_level(p.d, lev, Yp, t.comps, c0, c1, t.tb, t.span, nts, Y, h->stream));
+         launch_comb_level(p.d, lev, Yp, t.comps, c0, c1, t.tb, t.span, nts, Y, h->stream, -1,
+                           lev == jx_star ? guard : FailureGuard{}));
   }
 }
 
@@ -2490,11 +2509,13 @@ st_status st_setup(const st_problem* problem, const st_options* options, st_hand
   hp->scalar = hp->alloc<double>(1);
   hp->dev_err = hp->alloc<int>(1);
   hp->solve_err = hp->alloc<int>(1);
-  if (!hp->part || !hp->scalar || !hp->dev_err || !hp->solve_err) {
+  hp->sc_fail = hp->alloc<unsigned>(2);
+  if (!hp->part || !hp->scalar || !hp->dev_err || !hp->solve_err || !hp->sc_fail) {
     g_create_error = "device allocation failed";
     return ST_ERR_OOM;
   }
-  if (cudaMemsetAsync(hp->solve_err, 0, sizeof(int), hp->stream) != cudaSuccess) {
+  if (cudaMemsetAsync(hp->solve_err, 0, sizeof(int), hp->stream) != cudaSuccess ||
+      cudaMemsetAsync(hp->sc_fail, 0, 2 * sizeof(unsigned), hp->stream) != cudaSuccess) {
     g_create_error = "cudaMemset failed";
     return ST_ERR_CUDA;
   }
@@ -2848,11 +2869,19 @@ st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_d
   std::vector<char> done(nc, 0);
   std::mutex mu;
   std::condition_variable cv;
+  // graph solves report after the levels are queued: the target level looks for
+  // itself (where the levels run in FP64, after one small launch in front of it: 2D box
+  // n = 9 0.441 -> 0.452 ms; such a launch behind every component's graph took it to
+  // 0.64 ms, and waiting for the records here would leave the host's round trip
+  // between the last solve and the level)
+  const FailureGuard guard{h->sc_fail + buf, (unsigned)h->api_seq};
   auto run = [&](int i) {
     Component& c = *h->comps[i];
     st_status r = solve_one(h, c, forward_io(c), false);
+    SolveFailure fail;
+    if (c.rec_pending) fail = SolveFailure{solve_record(c), fail_eta(h), h->sc_fail + buf, guard.call};
     if (r == ST_OK && overlap) {
-      launch_comb_prep_ds(h->prob.d, c.U, c.sl->lift, c.coef, c.jx, c.nt, c.Uds[buf], nullptr, c.cs);
+      launch_comb_prep_ds(h->prob.d, c.U, c.sl->lift, c.coef, c.jx, c.nt, c.Uds[buf], nullptr, c.cs, fail);
       r = ccheck(c, "combination pairs");
     }
     if (r == ST_OK && cudaEventRecord(c.done, c.cs) != cudaSuccess) r = cfail(c, ST_ERR_CUDA, "event record failed");
@@ -2898,7 +2927,9 @@ st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_d
     if (failed) break;
     cudaEvent_t lb = trace.t0 ? trace.make("level " + std::to_string(lev) + " combination start") : nullptr;
     if (lb != nullptr) cudaEventRecord(lb, h->stream);
-    enqueue_comb_level(h, *t, lev, jx_star, jt_star, out_dev, buf, overlap);
+    if (lev == jx_star && !overlap && !byc.empty())
+      launch_note_failures(t->recs, nc, SolveFailure{nullptr, fail_eta(h), h->sc_fail + buf, guard.call}, h->stream);
+    enqueue_comb_level(h, *t, lev, jx_star, jt_star, out_dev, buf, overlap, guard);
     cudaEvent_t le = trace.t0 ? trace.make("level " + std::to_string(lev) + " combination end") : nullptr;
     if (le != nullptr) cudaEventRecord(le, h->stream);
   }
