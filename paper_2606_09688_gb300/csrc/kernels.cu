@@ -2525,9 +2525,9 @@ int receiver_group(int64_t n, int ncomp) {
 }
 
 void launch_receiver_eval(const CombComp* comps, int ncomp, const RecCorner* rc, int nrec, int ncorner,
-                          const double* tbv, const int* tspan, int nts, double* part, double* out, cudaStream_t s) {
+                          const double* tbv, const int* tspan, int nts, double* part, int grp, double* out,
+                          cudaStream_t s) {
   const int64_t n = (int64_t)nts * nrec;
-  const int grp = receiver_group(n, ncomp);
   for (int c0 = 0; c0 < ncomp; c0 += grp) {
     const int nc = std::min(grp, ncomp - c0);
     count(2);

@@ -278,11 +278,12 @@ struct ElemK {
   double k[64];
 };
 // out[s][r] = sum_c coef_c u_c(x_r, t_s) for all target times s (nts) and
-// receivers r; part: scratch of receiver_group(nts x nrec, ncomp) x nts x nrec
-// doubles (at most 64 MB, or one component's values where those are more).
+// receivers r, the components in groups of grp; part: scratch of grp x nts x nrec
+// doubles.  receiver_group(nts x nrec, ncomp): the group that at most 64 MB hold, or 1.
 int receiver_group(int64_t n, int ncomp);
 void launch_receiver_eval(const CombComp* comps, int ncomp, const RecCorner* rc, int nrec, int ncorner,
-                          const double* tbv, const int* tspan, int nts, double* part, double* out, cudaStream_t s);
+                          const double* tbv, const int* tspan, int nts, double* part, int grp, double* out,
+                          cudaStream_t s);
 // wm[s][r] = w_s (vals - dobs)[s][r] with trapezoid weights on [0, T]; J = 1/2 sum w_s e^2 -> Jout[0].
 void launch_misfit(const double* vals, const double* dobs, int nts, int nrec, double T, double* wm, double* Jout,
                    cudaStream_t s);

@@ -380,6 +380,9 @@ struct st_handle {
   std::map<std::tuple<int, int, uint64_t>, CombTables> comb;  // per target level pair and component set
 
   // Receiver tables of the misfit gradient (one receiver set cached).
+  // Receiver tables of the last set of receivers and target times.  All of them lie in
+  // one block that grows with the largest set and serves every later one; a set
+  // whose block is not to be had leaves the tables of the set before in force.
   struct RecTables {
     int jt = -1, nrec = 0, ncorner = 0, nts = 0;
     std::vector<double> x;        // receiver coordinates (nrec x d)
@@ -391,8 +394,11 @@ struct st_handle {
     double* wm = nullptr;         // weighted misfit, nts x nrec
     double* J = nullptr;          // 1
     double* part = nullptr;       // receiver values of a group of components
+    int group = 1;                // components a group
     AdjComp* adj = nullptr;       // adjoint right-hand sides, in component order (first gradient)
     int max_nt = 1;
+    unsigned char* block = nullptr;
+    size_t bytes = 0;
   } rec;
 
   // Workspace of st_energy, kept between calls up to 72 MiB.
@@ -2141,17 +2147,54 @@ st_status build_receivers(st_handle* h, int jt_star, const double* x, int nrec) 
       sp[(size_t)c * nts + s] = span;
     }
   }
-  R.comps = h->upload(cc);
-  R.rc = h->upload(rc);
-  R.tb = h->upload(tb);
-  R.span = h->upload(sp);
-  R.vals = h->alloc<double>((size_t)nts * nrec);
-  R.wm = h->alloc<double>((size_t)nts * nrec);
-  R.J = h->alloc<double>(1);
-  R.part = h->alloc<double>((size_t)receiver_group((int64_t)nts * nrec, ncomp) * nts * nrec);
+  const size_t n = (size_t)nts * nrec;
+  size_t off[8];
+  auto layout = [&](int group) {
+    const size_t part[8] = {sizeof(CombComp) * cc.size(), sizeof(RecCorner) * rc.size(), sizeof(double) * tb.size(),
+                            sizeof(int) * sp.size(),      sizeof(double) * n,            sizeof(double) * n,
+                            sizeof(double),               sizeof(double) * n * group};
+    size_t total = 0;
+    for (int k = 0; k < 8; ++k) {
+      off[k] = total;
+      total += (part[k] + 255) & ~(size_t)255;
+    }
+    return total;
+  };
+  int group = receiver_group((int64_t)n, ncomp);
+  if (layout(group) > R.bytes) {
+    // a block of at least twice the old one, which stays behind (so that all blocks
+    // together take at most twice the largest), else of the size needed, else one
+    // component at a time
+    size_t want = std::max(layout(group), 2 * R.bytes);
+    unsigned char* block = h->alloc<unsigned char>(want);
+    if (block == nullptr) block = h->alloc<unsigned char>(want = layout(group));
+    if (block == nullptr && layout(group = 1) > R.bytes) {
+      block = h->alloc<unsigned char>(want = layout(group));
+      if (block == nullptr) return fail(h, ST_ERR_OOM, "device allocation failed");
+    }
+    if (block != nullptr) {
+      R.block = block;
+      R.bytes = want;
+    }
+  }
+  layout(group);
+  R.jt = -1;  // the tables are neither the old set's nor the new one's until all copies are queued
+  R.comps = (CombComp*)(R.block + off[0]);
+  R.rc = (RecCorner*)(R.block + off[1]);
+  R.tb = (double*)(R.block + off[2]);
+  R.span = (int*)(R.block + off[3]);
+  R.vals = (double*)(R.block + off[4]);
+  R.wm = (double*)(R.block + off[5]);
+  R.J = (double*)(R.block + off[6]);
+  R.part = (double*)(R.block + off[7]);
+  R.group = group;
+  ST_CUDA(h, cudaMemcpyAsync(R.comps, cc.data(), sizeof(CombComp) * cc.size(), cudaMemcpyHostToDevice, h->stream));
+  ST_CUDA(h, cudaMemcpyAsync(R.rc, rc.data(), sizeof(RecCorner) * rc.size(), cudaMemcpyHostToDevice, h->stream));
+  ST_CUDA(h, cudaMemcpyAsync(R.tb, tb.data(), sizeof(double) * tb.size(), cudaMemcpyHostToDevice, h->stream));
+  ST_CUDA(h, cudaMemcpyAsync(R.span, sp.data(), sizeof(int) * sp.size(), cudaMemcpyHostToDevice, h->stream));
+  h->h2d_bytes += (int64_t)(sizeof(CombComp) * cc.size() + sizeof(RecCorner) * rc.size() + sizeof(double) * tb.size() +
+                            sizeof(int) * sp.size());
   R.max_nt = max_nt;
-  if (!R.comps || !R.rc || !R.tb || !R.span || !R.vals || !R.wm || !R.J || !R.part)
-    return fail(h, ST_ERR_OOM, "device allocation failed");
   R.jt = jt_star;
   R.nrec = nrec;
   R.ncorner = nc;
@@ -2986,7 +3029,8 @@ st_status st_receiver_values(st_handle* h, int jt_star, const double* x_rec, int
   st_status s = build_receivers(h, jt_star, x_rec, n_rec);
   if (s != ST_OK) return s;
   const st_handle::RecTables& R = h->rec;
-  launch_receiver_eval(R.comps, (int)h->comps.size(), R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.part, out_dev, h->stream);
+  launch_receiver_eval(R.comps, (int)h->comps.size(), R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.part,
+                       R.group, out_dev, h->stream);
   return check_launch(h, "receiver values");
 }
 
@@ -3007,7 +3051,8 @@ st_status st_misfit_gradient(st_handle* h, int jt_star, const double* x_rec, int
   if (s != ST_OK) return s;
   st_handle::RecTables& R = h->rec;
   const int ncomp = (int)h->comps.size();
-  launch_receiver_eval(R.comps, ncomp, R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.part, R.vals, h->stream);
+  launch_receiver_eval(R.comps, ncomp, R.rc, n_rec, R.ncorner, R.tb, R.span, R.nts, R.part, R.group,
+                       R.vals, h->stream);
   launch_misfit(R.vals, d_obs_dev, R.nts, n_rec, p.T, R.wm, R.J, h->stream);
   // adjoint right-hand sides G_k = coef_k E_k^T (w * e)
   for (int c = 0; c < ncomp; ++c) {
