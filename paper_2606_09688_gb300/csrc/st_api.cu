@@ -2306,15 +2306,16 @@ st_status comb_tables(st_handle* h, int jx_star, int jt_star, uint64_t mask, con
   if (t.ds_ok)
     for (int o = 0; o < nc; ++o) {
       Component& k = *h->comps[order[o]];
-      if (k.Uds[0] == nullptr) {
-        k.Uds[0] = h->alloc<ds>((size_t)k.nt * k.nx);
-        k.Uds[1] = h->alloc<ds>((size_t)k.nt * k.nx);
-        if (k.sl->lift != nullptr) k.Lds = h->alloc<ds>((size_t)k.sl->nall);
-        if (k.Uds[0] == nullptr || k.Uds[1] == nullptr || (k.sl->lift != nullptr && k.Lds == nullptr))
-          return fail(h, ST_ERR_OOM, "device allocation failed");
+      // each by itself: a call after one that ran out of memory goes on where that stopped
+      for (int b = 0; b < 2; ++b)
+        if (k.Uds[b] == nullptr) k.Uds[b] = h->alloc<ds>((size_t)k.nt * k.nx);
+      if (k.sl->lift != nullptr && k.Lds == nullptr) {
+        k.Lds = h->alloc<ds>((size_t)k.sl->nall);
         if (k.Lds != nullptr)
           launch_comb_prep_ds(p.d, nullptr, k.sl->lift, k.coef, k.jx, k.nt, nullptr, k.Lds, h->stream);
       }
+      if (k.Uds[0] == nullptr || k.Uds[1] == nullptr || (k.sl->lift != nullptr && k.Lds == nullptr))
+        return fail(h, ST_ERR_OOM, "device allocation failed");
       for (int b = 0; b < 2; ++b) dc[b][o] = CombCompDS{k.Uds[b], k.Lds, k.jx, k.jt};
     }
   std::vector<const RefineRec*> recs(nc);
@@ -3058,12 +3059,11 @@ st_status st_misfit_gradient(st_handle* h, int jt_star, const double* x_rec, int
   for (int c = 0; c < ncomp; ++c) {
     Component& k = *h->comps[c];
     const size_t n = (size_t)k.nt * k.nx;
-    if (k.Gadj == nullptr) {
-      k.Gadj = h->alloc<double>(n);
-      k.Lam = h->alloc<double>(n);
-      k.gv = h->alloc<double>((size_t)k.nx);
-      if (!k.Gadj || !k.Lam || !k.gv) return fail(h, ST_ERR_OOM, "device allocation failed");
-    }
+    // each by itself: a call after one that ran out of memory goes on where that stopped
+    if (k.Gadj == nullptr) k.Gadj = h->alloc<double>(n);
+    if (k.Lam == nullptr) k.Lam = h->alloc<double>(n);
+    if (k.gv == nullptr) k.gv = h->alloc<double>((size_t)k.nx);
+    if (!k.Gadj || !k.Lam || !k.gv) return fail(h, ST_ERR_OOM, "device allocation failed");
     ST_CUDA(h, cudaMemsetAsync(k.Gadj, 0, n * sizeof(double), h->stream));
   }
   if (R.adj == nullptr) {
