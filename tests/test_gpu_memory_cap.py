@@ -82,3 +82,37 @@ def test_misfit_gradient_is_refused_or_works(torch):
                       mem_cap_bytes=16 << 20)
     results, refusals = _sweep(make, lambda s: s.misfit_gradient(su.jt_star, su.receivers, obs, 3)[0], 5)
     assert refusals >= 4 and np.isfinite(results[0]) and results[0] > 0 and len(set(results)) == 1
+
+
+def _pool_high(reset=False):
+    """Most memory that the device's default pool has held since the last reset."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, v = ctypes.c_void_p(), ctypes.c_uint64(0)
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    reserved_high = 6
+    if reset:
+        assert cu.cuMemPoolSetAttribute(pool, reserved_high, ctypes.byref(v)) == 0
+    assert cu.cuMemPoolGetAttribute(pool, reserved_high, ctypes.byref(v)) == 0
+    return v.value
+
+
+def test_set_up_under_a_cap_holds_one_workspace_at_a_time(torch):
+    """The factorisation's workspaces are not part of the handle's memory, so the cap covers
+    the largest of them, not their sum: a set-up of all components takes no more from the
+    pool than the largest one alone (64 MB: twice the pool's granularity)."""
+    import dataclasses
+
+    from paper_2606_09688_gb300 import Solver
+    p = W.layered_2d(11, 2)
+
+    def high(q):
+        torch.cuda.synchronize()
+        _pool_high(reset=True)
+        with Solver(q, mem_cap_bytes=64 << 30) as s:
+            comps = [(c.jx, c.jt) for c in s.components()]
+        return _pool_high(), comps
+    total, comps = high(p)
+    single = max(high(dataclasses.replace(p, J=0, mx=jx, mt=jt))[0] for jx, jt in comps if jx in (7, 8))
+    assert single > 256 << 20
+    assert total <= single + (64 << 20), (total >> 20, single >> 20)
