@@ -1,6 +1,8 @@
 // Banded complex-symmetric LDL^T: assembly, factorisation and the solve of
-// the spatial problems (K + lam_q M) x = b on grids small enough for a direct
-// method (whole component grids, or the coarsest multigrid level).
+// the spatial problems (K + lam_q M) x = b.  Its solves form the explicit inverses of
+// coarsest multigrid grids of at most 1024 unknowns at set-up (half bandwidths up
+// to 64; larger grids are solved by nested dissection, nd.cu), and its bounded copy
+// waits carry the fault injection of the timeout tests (129 to 256).
 //
 // Storage (per mode q, at q * mstride): row k of F holds column k of L,
 // F[k][t] = L_{k+t,k} (t = 1..bw) and F[k][0] = 1/d_k; row k of G holds row k of L,
@@ -347,95 +349,47 @@ __global__ void __launch_bounds__(32) k_band_solve_w(const cx<R>* __restrict__ F
   }
 }
 
-// Variant for bw = 32 * SLOTS (every 2D grid: bw = 2^j): rows keep their
-// register slot for their whole life (row r in lane r mod 32, register
-// (r mod bw) / 32), so no data moves between lanes except the broadcast of
-// the finished row.  Chunks are 32 rows, one group of 32 unrolled steps in
-// which every band offset is a compile-time constant; SG = chunk mod SLOTS is
-// the register that holds the rows finished during the chunk.
-template <typename R, int SLOTS, int PASS, int SG>
-__device__ __forceinline__ void band_group32(const cx<R>* __restrict__ st, int c, int nrow, int ld, int lane,
-                                             cx<R> (&v)[SLOTS], const cx<R>& bcur, cx<R>& y,
-                                             cx<R>* __restrict__ dst) {
-  constexpr int bw = 32 * SLOTS;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const cx<R>* row = st + (size_t)(PASS == 0 ? i : 31 - i) * ld;
-    if (lane == i) {
-      const int kp = 32 * c + i;
-      const int k = PASS == 0 ? kp : nrow - 1 - kp;
-      dst[k] = PASS == 0 ? y * row[0] : y;
-    }
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      if (s == SG) {
-        // lanes after i hold rows kp + (lane - i); lanes before i already hold
-        // rows entered during this chunk (t = lane - i + bw); lane i takes row kp + bw
-        const int t = lane - i + (lane <= i ? bw : 0);
-        const cx<R> a = row[t];
-        const cx<R> base = lane == i ? bcur : v[s];
-        v[s] = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, base.re)), fma(-a.re, y.im, fma(-a.im, y.re, base.im)));
-      } else {
-        const int d = (s - SG + SLOTS) % SLOTS;
-        const cx<R> a = row[lane - i + 32 * d];
-        v[s] = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, v[s].re)), fma(-a.re, y.im, fma(-a.im, y.re, v[s].im)));
-      }
-    }
-    const int nslot = (i < 31) ? SG : (SG + 1) % SLOTS;
-    y.re = __shfl_sync(0xffffffffu, v[nslot].re, (i + 1) & 31);
-    y.im = __shfl_sync(0xffffffffu, v[nslot].im, (i + 1) & 31);
-  }
-}
-
-// One step with a run-time step index (the last, partial chunk).
-template <typename R, int SLOTS, int PASS>
-__device__ __forceinline__ void band_step_rt(const cx<R>* __restrict__ row, int i, int sg, int c, int nrow,
-                                             int lane, cx<R> (&v)[SLOTS], const cx<R>& bcur, cx<R>& y,
-                                             cx<R>* __restrict__ dst) {
-  constexpr int bw = 32 * SLOTS;
+// Variant for bw = 32 (the 31^2 grid, the largest with an explicit inverse in 2D):
+// a row stays in its lane (row r in lane r mod 32) for its whole life, so no data
+// moves between lanes except the broadcast of the finished row.  Chunks are 32 rows,
+// one group of 32 unrolled steps in which every band offset is a compile-time
+// constant; the last, partial chunk runs the same step with its index at run time.
+template <typename R, int PASS>
+__device__ __forceinline__ void band_step32(const cx<R>* __restrict__ row, int i, int c, int nrow, int lane, cx<R>& v,
+                                            const cx<R>& bcur, cx<R>& y, cx<R>* __restrict__ dst) {
   if (lane == i) {
     const int kp = 32 * c + i;
     const int k = PASS == 0 ? kp : nrow - 1 - kp;
     dst[k] = PASS == 0 ? y * row[0] : y;
   }
+  // lanes after i hold rows kp + (lane - i); lanes before i already hold rows
+  // entered during this chunk (t = lane - i + 32); lane i takes row kp + 32
+  const cx<R> a = row[lane - i + (lane <= i ? 32 : 0)];
+  const cx<R> base = lane == i ? bcur : v;
+  v = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, base.re)), fma(-a.re, y.im, fma(-a.im, y.re, base.im)));
+  y.re = __shfl_sync(0xffffffffu, v.re, (i + 1) & 31);
+  y.im = __shfl_sync(0xffffffffu, v.im, (i + 1) & 31);
+}
+
+template <typename R, int PASS>
+__device__ __forceinline__ void band_chunk32(const cx<R>* __restrict__ st, int cnt, int c, int nrow, int ld, int lane,
+                                             cx<R>& v, const cx<R>& bcur, cx<R>& y, cx<R>* __restrict__ dst) {
+  if (cnt == 32) {
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s) {
-    int t;
-    cx<R> base = v[s];
-    if (s == sg) {
-      t = lane - i + (lane <= i ? bw : 0);
-      if (lane == i) base = bcur;
-    } else {
-      t = lane - i + 32 * ((s - sg + SLOTS) % SLOTS);
-    }
-    const cx<R> a = row[t];
-    v[s] = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, base.re)), fma(-a.re, y.im, fma(-a.im, y.re, base.im)));
+    for (int i = 0; i < 32; ++i)
+      band_step32<R, PASS>(st + (size_t)(PASS == 0 ? i : 31 - i) * ld, i, c, nrow, lane, v, bcur, y, dst);
+  } else {
+    for (int i = 0; i < cnt; ++i)
+      band_step32<R, PASS>(st + (size_t)(PASS == 0 ? i : cnt - 1 - i) * ld, i, c, nrow, lane, v, bcur, y, dst);
   }
-  const int nslot = (i < 31) ? sg : (sg + 1) % SLOTS;
-  cx<R> src = v[0];
-#pragma unroll
-  for (int s = 1; s < SLOTS; ++s)
-    if (s == nslot) src = v[s];
-  y.re = __shfl_sync(0xffffffffu, src.re, (i + 1) & 31);
-  y.im = __shfl_sync(0xffffffffu, src.im, (i + 1) & 31);
 }
 
-template <typename R, int SLOTS, int PASS>
-__device__ __forceinline__ void band_group_dispatch(const cx<R>* st, int c, int nrow, int ld, int lane,
-                                                    cx<R> (&v)[SLOTS], const cx<R>& bcur, cx<R>& y, cx<R>* dst) {
-  const int sg = c % SLOTS;
-  if (SLOTS == 1 || sg == 0) band_group32<R, SLOTS, PASS, 0>(st, c, nrow, ld, lane, v, bcur, y, dst);
-  else if (SLOTS >= 2 && sg == 1) band_group32<R, SLOTS, PASS, (SLOTS >= 2 ? 1 : 0)>(st, c, nrow, ld, lane, v, bcur, y, dst);
-  else if (SLOTS >= 4 && sg == 2) band_group32<R, SLOTS, PASS, (SLOTS >= 4 ? 2 : 0)>(st, c, nrow, ld, lane, v, bcur, y, dst);
-  else if (SLOTS >= 4 && sg == 3) band_group32<R, SLOTS, PASS, (SLOTS >= 4 ? 3 : 0)>(st, c, nrow, ld, lane, v, bcur, y, dst);
-}
-
-template <typename R, int SLOTS>
+template <typename R>
 __global__ void __launch_bounds__(32) k_band_solve_p2(const cx<R>* __restrict__ F, const cx<R>* __restrict__ G,
                                                       BandLayout L, const cx<R>* __restrict__ b,
                                                       cx<R>* __restrict__ x, const CocgScal* __restrict__ scal,
                                                       int64_t vstride, int* err) {
-  constexpr int C = 32, bw = 32 * SLOTS;
+  constexpr int C = 32, bw = 32;
   extern __shared__ __align__(128) unsigned char smem[];
   const int q = blockIdx.x;
   if (scal != nullptr && !scal[q].active) return;
@@ -479,13 +433,11 @@ __global__ void __launch_bounds__(32) k_band_solve_p2(const cx<R>* __restrict__ 
       issue(0);
       if (nchunks > 1) issue(1);
     }
-    cx<R> v[SLOTS];
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) v[s] = at(lane + 32 * s);
+    cx<R> v = at(lane);
     cx<R> bcur = at(lane + bw), bnext = at(C + lane + bw);
     cx<R> y;
-    y.re = __shfl_sync(0xffffffffu, v[0].re, 0);
-    y.im = __shfl_sync(0xffffffffu, v[0].im, 0);
+    y.re = __shfl_sync(0xffffffffu, v.re, 0);
+    y.im = __shfl_sync(0xffffffffu, v.im, 0);
     bool ok = true;
     for (int c = 0; c < nchunks; ++c) {
       ok = mbar_wait_bounded(&bar[c & 1], phase[c & 1]);
@@ -498,17 +450,8 @@ __global__ void __launch_bounds__(32) k_band_solve_p2(const cx<R>* __restrict__ 
       int klo, cnt;
       chunk(c, klo, cnt);
       const cx<R>* st = (c & 1) ? stage1 : stage0;
-      if (cnt == C) {
-        if (pass == 0) band_group_dispatch<R, SLOTS, 0>(st, c, nrow, ld, lane, v, bcur, y, dst);
-        else band_group_dispatch<R, SLOTS, 1>(st, c, nrow, ld, lane, v, bcur, y, dst);
-      } else {
-        const int sg = c % SLOTS;
-        for (int i = 0; i < cnt; ++i) {
-          const cx<R>* row = st + (size_t)(pass == 0 ? i : cnt - 1 - i) * ld;
-          if (pass == 0) band_step_rt<R, SLOTS, 0>(row, i, sg, c, nrow, lane, v, bcur, y, dst);
-          else band_step_rt<R, SLOTS, 1>(row, i, sg, c, nrow, lane, v, bcur, y, dst);
-        }
-      }
+      if (pass == 0) band_chunk32<R, 0>(st, cnt, c, nrow, ld, lane, v, bcur, y, dst);
+      else band_chunk32<R, 1>(st, cnt, c, nrow, ld, lane, v, bcur, y, dst);
       bcur = bnext;
       bnext = bnn;
       __syncwarp();
@@ -525,162 +468,6 @@ __global__ void __launch_bounds__(32) k_band_solve_p2(const cx<R>* __restrict__ 
   }
 }
 
-// FP64 variant of the fixed-slot solve: GB300 issues FP64 at a small
-// fraction of the FP32 rate per SM sub-partition, so one warp per mode is
-// bound by the FP64 pipe of its sub-partition.  Here each of SLOTS warps owns
-// one register slot (lanes hold rows r with (r mod bw) / 32 = warp), so the
-// per-row complex FMAs of a mode spread over SLOTS sub-partitions; the
-// finished row is passed through shared memory with one block barrier per row.
-// (ybuf is written by other threads between the barriers, so it must not be a
-// restrict pointer: that would let the compiler reuse an earlier load of it.)
-template <typename R, int SLOTS, int PASS, int SG>
-__device__ __forceinline__ void band_group32_mw(const cx<R>* __restrict__ st, int c, int nrow, int ld, int lane,
-                                                int warp, cx<R>& v, const cx<R>& bcur, cx<R>& y,
-                                                cx<R>* ybuf, cx<R>* __restrict__ dst) {
-  constexpr int bw = 32 * SLOTS;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const cx<R>* row = st + (size_t)(PASS == 0 ? i : 31 - i) * ld;
-    if (warp == SG && lane == i) {
-      const int kp = 32 * c + i;
-      const int k = PASS == 0 ? kp : nrow - 1 - kp;
-      dst[k] = PASS == 0 ? y * row[0] : y;
-    }
-    if (warp == SG) {
-      const int t = lane - i + (lane <= i ? bw : 0);
-      const cx<R> a = row[t];
-      const cx<R> base = lane == i ? bcur : v;
-      v = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, base.re)), fma(-a.re, y.im, fma(-a.im, y.re, base.im)));
-    } else {
-      const int d = (warp - SG + SLOTS) % SLOTS;
-      const cx<R> a = row[lane - i + 32 * d];
-      v = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, v.re)), fma(-a.re, y.im, fma(-a.im, y.re, v.im)));
-    }
-    const int nslot = (i < 31) ? SG : (SG + 1) % SLOTS;
-    if (warp == nslot && lane == ((i + 1) & 31)) ybuf[i & 1] = v;
-    __syncthreads();
-    y = ybuf[i & 1];
-  }
-}
-
-template <typename R, int SLOTS>
-__global__ void __launch_bounds__(32 * SLOTS) k_band_solve_mw(const cx<R>* __restrict__ F, const cx<R>* __restrict__ G,
-                                                              BandLayout L, const cx<R>* __restrict__ b,
-                                                              cx<R>* __restrict__ x, const CocgScal* __restrict__ scal,
-                                                              int64_t vstride, int* err) {
-  constexpr int C = 32, bw = 32 * SLOTS;
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int q = blockIdx.x;
-  if (scal != nullptr && !scal[q].active) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ld = L.ld, nrow = (int)L.nrow;
-  const size_t stage_elems = (size_t)C * ld;
-  cx<R>* stage0 = reinterpret_cast<cx<R>*>(smem);
-  cx<R>* stage1 = stage0 + stage_elems;
-  cx<R>* ybuf = stage1 + stage_elems;  // 2 entries
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ybuf + 2);
-  if (threadIdx.x == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  unsigned phase[2] = {0u, 0u};
-  const int nchunks = (nrow + C - 1) / C;
-  cx<R>* dst = x + (int64_t)q * vstride;
-  const cx<R> zero = mk<R>(0, 0);
-  for (int pass = 0; pass < 2; ++pass) {
-    const cx<R>* Mq = (pass == 0 ? F : G) + (int64_t)q * L.mstride;
-    const cx<R>* src = pass == 0 ? b + (int64_t)q * vstride : dst;
-    auto chunk = [&](int c, int& klo, int& cnt) {
-      const int k0 = c * C;
-      cnt = min(C, nrow - k0);
-      klo = pass == 0 ? k0 : nrow - k0 - cnt;
-    };
-    auto issue = [&](int c) {
-      int klo, cnt;
-      chunk(c, klo, cnt);
-      cx<R>* st = (c & 1) ? stage1 : stage0;
-      const unsigned bytes = (unsigned)((size_t)cnt * ld * sizeof(cx<R>));
-      mbar_expect_tx(&bar[c & 1], bytes);
-      bulk_g2s(st, Mq + (int64_t)klo * ld, bytes, &bar[c & 1]);
-    };
-    auto at = [&](int rp) -> cx<R> {
-      if (rp >= nrow) return zero;
-      return src[pass == 0 ? rp : nrow - 1 - rp];
-    };
-    if (threadIdx.x == 0) {
-      issue(0);
-      if (nchunks > 1) issue(1);
-    }
-    cx<R> v = at(lane + 32 * warp);
-    cx<R> bcur = at(lane + bw), bnext = at(C + lane + bw);
-    if (threadIdx.x == 0) ybuf[1] = v;  // row 0 (lane 0 of warp 0)
-    __syncthreads();
-    cx<R> y = ybuf[1];
-    bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
-      ok = mbar_wait_bounded(&bar[c & 1], phase[c & 1]);
-      if (!__syncthreads_and(ok)) {
-        ok = false;
-        break;
-      }
-      phase[c & 1] ^= 1u;
-      const cx<R> bnn = at((c + 2) * C + lane + bw);
-      int klo, cnt;
-      chunk(c, klo, cnt);
-      const cx<R>* st = (c & 1) ? stage1 : stage0;
-      const int sg = c % SLOTS;
-      if (cnt == C) {
-#define ST_MW_GROUP(P, S)                                                                            \
-  if (sg == S) band_group32_mw<R, SLOTS, P, (S < SLOTS ? S : 0)>(st, c, nrow, ld, lane, warp, v, bcur, y, \
-                                                                  ybuf, dst);
-        if (pass == 0) {
-          ST_MW_GROUP(0, 0) ST_MW_GROUP(0, 1) ST_MW_GROUP(0, 2) ST_MW_GROUP(0, 3)
-        } else {
-          ST_MW_GROUP(1, 0) ST_MW_GROUP(1, 1) ST_MW_GROUP(1, 2) ST_MW_GROUP(1, 3)
-        }
-#undef ST_MW_GROUP
-      } else {
-        for (int i = 0; i < cnt; ++i) {
-          const cx<R>* row = st + (size_t)(pass == 0 ? i : cnt - 1 - i) * ld;
-          if (warp == sg && lane == i) {
-            const int kp = 32 * c + i;
-            const int k = pass == 0 ? kp : nrow - 1 - kp;
-            dst[k] = pass == 0 ? y * row[0] : y;
-          }
-          int t;
-          cx<R> base = v;
-          if (warp == sg) {
-            t = lane - i + (lane <= i ? bw : 0);
-            if (lane == i) base = bcur;
-          } else {
-            t = lane - i + 32 * ((warp - sg + SLOTS) % SLOTS);
-          }
-          const cx<R> a = row[t];
-          v = mk<R>(fma(-a.re, y.re, fma(a.im, y.im, base.re)), fma(-a.re, y.im, fma(-a.im, y.re, base.im)));
-          const int nslot = (i < 31) ? sg : (sg + 1) % SLOTS;
-          if (warp == nslot && lane == ((i + 1) & 31)) ybuf[i & 1] = v;
-          __syncthreads();
-          y = ybuf[i & 1];
-        }
-      }
-      bcur = bnext;
-      bnext = bnn;
-      __syncthreads();
-      if (threadIdx.x == 0 && c + 2 < nchunks) issue(c + 2);
-    }
-    if (!ok) {
-      if (threadIdx.x == 0) {
-        atomicExch(err, 2);
-        for (int c2 = 0; c2 < 2; ++c2) mbar_wait_bounded(&bar[c2], phase[c2]);
-      }
-      return;
-    }
-    __syncthreads();
-  }
-}
-
 std::mutex g_attr_mu;  // launches come from several host threads (one per component)
 
 template <typename R, int SLOTS> void set_smem_attr(size_t bytes) {
@@ -692,20 +479,11 @@ template <typename R, int SLOTS> void set_smem_attr(size_t bytes) {
   }
 }
 
-template <typename R, int SLOTS> void set_smem_attr_mw(size_t bytes) {
+template <typename R> void set_smem_attr_p2(size_t bytes) {
   static size_t done = 0;
   std::lock_guard<std::mutex> lock(g_attr_mu);
   if (bytes > done) {
-    cudaFuncSetAttribute(k_band_solve_mw<R, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    done = bytes;
-  }
-}
-
-template <typename R, int SLOTS> void set_smem_attr_p2(size_t bytes) {
-  static size_t done = 0;
-  std::lock_guard<std::mutex> lock(g_attr_mu);
-  if (bytes > done) {
-    cudaFuncSetAttribute(k_band_solve_p2<R, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaFuncSetAttribute(k_band_solve_p2<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     done = bytes;
   }
 }
@@ -762,18 +540,14 @@ void launch_band_factor(cx<R>* F, cx<R>* G, const BandLayout& L, int nmodes, int
     const int RI = (L.bw + 31) / 32 * 32, NP = RI >= 256 ? 1 : 256 / RI;
     set_smem_attr_ldlt<R>(win_bytes);
     k_band_ldlt_win<R><<<nmodes, RI * NP, win_bytes, s>>>(F, L, RI, NP, err);
-  } else if (L.bw <= 256 && dsm_bytes(L.bw, 4, sizeof(cx<R>)) <= kMaxWindowBytes) {
-    // the window over a cluster of 4 CTAs (FP64, half bandwidth 128)
+  } else if (L.bw <= 256) {
+    // over a cluster of 4 (FP32) or 8 CTAs (FP64): half bandwidths 129 to 256, which only
+    // the fault injection of the single-warp solve takes (the 15^3 and 255^2 grids)
+    constexpr int NC = sizeof(R) == 8 ? 8 : 4;
     const int RI = (L.bw + 31) / 32 * 32, NP = 256 / RI;
-    const size_t bytes = dsm_bytes(L.bw, 4, sizeof(cx<R>));
-    set_smem_attr_ldlt_dsm<R, 4>(bytes);
-    k_band_ldlt_dsm<R, 4><<<nmodes * 4, RI * NP, bytes, s>>>(F, L, RI, NP, err);
-  } else if (L.bw <= 256 && dsm_bytes(L.bw, 8, sizeof(cx<R>)) <= kMaxWindowBytes) {
-    // over 8 CTAs (FP64, half bandwidth 241: the 15^3 grid)
-    const int RI = (L.bw + 31) / 32 * 32, NP = 256 / RI;
-    const size_t bytes = dsm_bytes(L.bw, 8, sizeof(cx<R>));
-    set_smem_attr_ldlt_dsm<R, 8>(bytes);
-    k_band_ldlt_dsm<R, 8><<<nmodes * 8, RI * NP, bytes, s>>>(F, L, RI, NP, err);
+    const size_t bytes = dsm_bytes(L.bw, NC, sizeof(cx<R>));
+    set_smem_attr_ldlt_dsm<R, NC>(bytes);
+    k_band_ldlt_dsm<R, NC><<<nmodes * NC, RI * NP, bytes, s>>>(F, L, RI, NP, err);
   }
   k_band_rows<R><<<dim3(blocks_for(L.nrow * L.ld), nmodes), kBlock, 0, s>>>(F, G, L);
   note_launches(2);
@@ -788,24 +562,10 @@ int band_chunk_rows(const BandLayout& L, size_t elem) {
 template <typename R>
 bool launch_band_solve(const cx<R>* F, const cx<R>* G, const BandLayout& L, const cx<R>* b, cx<R>* x,
                        const CocgScal* scal, int nmodes, int64_t vstride, int* err, cudaStream_t s) {
-  // power-of-two bandwidths (the 2D grids): fixed-slot kernel with 32-row chunks
-  const size_t smem32 = 2 * (size_t)32 * L.ld * sizeof(cx<R>) + 2 * sizeof(uint64_t);
-  if (sizeof(R) == 8 && smem32 + 2 * sizeof(cx<R>) <= 160 * 1024 && L.bw == 64) {
-    // FP64: spread each mode over bw / 32 warps (one FP64 pipe per warp)
-    const size_t sm = smem32 + 2 * sizeof(cx<R>);
-    set_smem_attr_mw<R, 2>(sm);
-    k_band_solve_mw<R, 2><<<nmodes, 64, sm, s>>>(F, G, L, b, x, scal, vstride, err);
-    note_launches(1);
-    return true;
-  }
-  if (smem32 <= 160 * 1024 && (L.bw == 32 || L.bw == 64)) {
-    if (L.bw == 32) {
-      set_smem_attr_p2<R, 1>(smem32);
-      k_band_solve_p2<R, 1><<<nmodes, 32, smem32, s>>>(F, G, L, b, x, scal, vstride, err);
-    } else {
-      set_smem_attr_p2<R, 2>(smem32);
-      k_band_solve_p2<R, 2><<<nmodes, 32, smem32, s>>>(F, G, L, b, x, scal, vstride, err);
-    }
+  if (L.bw == 32) {  // 31^2: chunks of 32 rows
+    const size_t smem32 = 2 * (size_t)32 * L.ld * sizeof(cx<R>) + 2 * sizeof(uint64_t);
+    set_smem_attr_p2<R>(smem32);
+    k_band_solve_p2<R><<<nmodes, 32, smem32, s>>>(F, G, L, b, x, scal, vstride, err);
     note_launches(1);
     return true;
   }
@@ -817,7 +577,7 @@ bool launch_band_solve(const cx<R>* F, const cx<R>* G, const BandLayout& L, cons
   } else if (L.bw <= 64) {
     set_smem_attr<R, 2>(smem);
     k_band_solve_w<R, 2><<<nmodes, 32, smem, s>>>(F, G, L, C, b, x, scal, vstride, err);
-  } else if (L.bw <= 256) {
+  } else if (L.bw <= 256) {  // fault injection only (launch_band_factor)
     set_smem_attr<R, 8>(smem);
     k_band_solve_w<R, 8><<<nmodes, 32, smem, s>>>(F, G, L, C, b, x, scal, vstride, err);
   } else {

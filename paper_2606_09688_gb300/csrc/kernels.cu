@@ -2396,12 +2396,11 @@ __global__ void k_refine_decide(RefineRec* __restrict__ rec, const double* __res
                                 const CocgScal* __restrict__ scal, int nsel, const int* __restrict__ cerr,
                                 cudaGraphConditionalHandle h, InnerTol itol) {
   int it = 0, worst = 0;  // worst: 2 = an iteration limit, 1 = another non-zero status word
-  if (scal != nullptr)
-    for (int q = threadIdx.x; q < nsel; q += 32) {
-      it = max(it, scal[q].iters);
-      const int sq = scal[q].status;
-      worst = max(worst, sq == 4 ? 2 : (sq != 0 ? 1 : 0));
-    }
+  for (int q = threadIdx.x; q < nsel; q += 32) {
+    it = max(it, scal[q].iters);
+    const int sq = scal[q].status;
+    worst = max(worst, sq == 4 ? 2 : (sq != 0 ? 1 : 0));
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     it = max(it, __shfl_xor_sync(0xffffffffu, it, o));
@@ -2412,7 +2411,7 @@ __global__ void k_refine_decide(RefineRec* __restrict__ rec, const double* __res
   r.sweeps += 1;
   r.max_iters = max(r.max_iters, it);
   int st = worst == 2 ? RR_ITER_LIMIT : (worst == 1 ? RR_NUMERIC : RR_OK);
-  if (cerr != nullptr && cerr[0] != 0) st = RR_TIMEOUT;
+  if (cerr[0] != 0) st = RR_TIMEOUT;
   const double rn = sqrt(nrm2[0]), un = sqrt(nrm2[1]), fn = sqrt(fn2[0]);
   const double rel = rn / fn, eta = rn / (snorm * un + fn);
   if (st == RR_OK && !(fabs(rel) <= 1.7e308)) st = RR_NUMERIC;

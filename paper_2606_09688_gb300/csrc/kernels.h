@@ -168,8 +168,8 @@ void launch_refine_init(RefineRec* rec, const double* fn2, cudaGraphConditionalH
                         cudaStream_t s);
 // After a sweep: nrm2 = (||R||^2, ||U||^2), fn2 = ||F||^2.  Stops on
 // eta = ||R|| / (snorm ||U|| + ||F||) <= tol, when eta no longer halves, after
-// max_sweeps, on a COCG status word (scal may be null), a copy timeout
-// (cerr[0] != 0, may be null) or a non-finite residual.
+// max_sweeps, on a COCG status word, a copy timeout (cerr[0] != 0) or a
+// non-finite residual.
 void launch_refine_decide(RefineRec* rec, const double* nrm2, const double* fn2, double snorm, double tol,
                           int max_sweeps, const CocgScal* scal, int nsel, const int* cerr,
                           cudaGraphConditionalHandle h, InnerTol it, cudaStream_t s);

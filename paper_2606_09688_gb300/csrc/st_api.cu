@@ -70,8 +70,8 @@ constexpr double kDirectFactorFlops = 2.5e10;
 // 41.5 / 19.9 ms); 1D and 3D 1024.
 constexpr int64_t kCoarseFloor = 1024, kCoarseFloor2D = 16384;
 constexpr int64_t kMaxDenseCoarse = 1024;  // coarsest multigrid grids up to this size use an explicit inverse
-constexpr int kMaxBandWidth = 1024;    // widest band the warp solve supports
-constexpr int kMaxCoarseBand = 256;    // widest band of a multigrid coarsest grid
+constexpr int kMaxBandWidth = 1024;    // grids of a wider band are not solved directly on request (max_direct_rows)
+constexpr int kMaxStallBand = 256;     // widest band of the single-warp banded solve (fault injection)
 constexpr int64_t kMaxCoarseRows = 32768;  // largest multigrid coarsest grid
 constexpr int kModeSMaxNx = 1024;      // dense spatial eigenbasis limit
 constexpr int kModeTMaxNt = 129;       // time eigenbasis used up to this many time unknowns
@@ -1143,7 +1143,7 @@ st_status setup_component(st_handle* h, Component& c) {
   // directly solved grids and coarsest grids too large for an explicit inverse
   // by nested dissection; the banded factors serve the explicit inverses and
   // the fault injection of the single-warp banded solve (bands above 128)
-  const bool stall = h->opt.inject_stall != 0 && c.bw > 128 && c.bw <= kMaxCoarseBand;
+  const bool stall = h->opt.inject_stall != 0 && c.bw > 128 && c.bw <= kMaxStallBand;
   if ((c.direct || c.nrowc > kMaxDenseCoarse) && !stall) {
     st_status s = nd_of(h, lc, c.nsel, c.inner64 ? 8 : 4, &c.nd);
     if (s != ST_OK) return s;
@@ -2396,10 +2396,10 @@ void largest_first(const st_handle* h, std::vector<int>& k) {
 
 // Forward (S U = F) or adjoint (S^T L = G) solves of components k0..k1-1.
 // Component streams start after the work already queued on the handle's
-// stream; independent components run concurrently, one host thread and one
-// stream each (one after the other with profiling on, so that event times are
-// not shared between overlapping kernels); the handle's stream then waits for
-// all of them.
+// stream; independent components run concurrently, one stream each, graph solves
+// queued by the calling thread and host-driven ones on a thread each (one after the
+// other with profiling on, so that event times are not shared between overlapping
+// kernels); the handle's stream then waits for all of them.
 st_status run_solves(st_handle* h, int k0, int k1, bool adjoint, st_solve_info* info) {
   ST_CUDA(h, cudaEventRecord(h->entry_ev, h->stream));
   std::vector<st_status> st(k1 - k0, ST_OK);
