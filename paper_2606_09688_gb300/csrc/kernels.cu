@@ -1696,7 +1696,10 @@ __global__ void __launch_bounds__(kBlock) k_comb_level(int j, const double* __re
                                                        const double* __restrict__ tbv, const int* __restrict__ tspan,
                                                        int nts, int nlift, double* __restrict__ Y, FastDiv dQ1,
                                                        FailureGuard guard) {
-  if (solve_failed(guard)) return;
+  if (guard.n > 0) {
+    const int k = threadIdx.x;
+    if (__syncthreads_or(k < guard.n && record_failed(guard.recs[k], guard.fail_eta))) return;
+  }
   const int s = blockIdx.y;
   const int Nj = 1 << j, Nc = Nj >> 1;
   int64_t ncs = 1, nsp = 1;
@@ -2469,18 +2472,6 @@ bool launch_time_band_solve(const double* ab, const int* piv, double* Y, int nt,
   cudaFuncSetAttribute(k_time_band_solve<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTimeBandMaxSmem);
   k_time_band_solve<2, 2><<<(unsigned)nx, 128, time_band_smem(nt), s>>>(ab, piv, Y, nt, nx);
   return true;
-}
-
-__global__ void k_note_failures(const RefineRec* const* __restrict__ recs, int n, SolveFailure f) {
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    f.rec = recs[k];
-    note_failure(f);
-  }
-}
-
-void launch_note_failures(const RefineRec* const* recs, int n, const SolveFailure& f, cudaStream_t s) {
-  count(1);
-  k_note_failures<<<1, 32, 0, s>>>(recs, n, f);
 }
 
 void launch_comb_level(int d, int j, const double* Yprev, const CombComp* comps, int c0, int c1, const double* tbv,

@@ -132,10 +132,11 @@ struct RefineStep {
   cudaGraphConditionalHandle cond{};
 };
 // A solve that failed, for the kernels that the host queues behind it before it
-// knows: launch_comb_prep_ds, on the component's stream, or launch_note_failures,
-// before the target level, set *word = call where a record tells of an error (a
-// status, or a backward error above fail_eta), and the target level of a combination
-// that finds its own call there writes nothing.  Words of earlier calls need no clearing.
+// knows: a record that tells of an error (a status, or a backward error above
+// fail_eta).  launch_comb_prep_ds, on the component's stream, sets *word = call where it
+// finds one, and the target level of a combination that finds its own call there
+// writes nothing (words of earlier calls need no clearing); a target level in FP64,
+// which the next call's solves never overlap, reads the n records itself.
 struct SolveFailure {
   const RefineRec* rec = nullptr;  // null: the host has seen the solve succeed
   double fail_eta = 0.0;
@@ -145,14 +146,16 @@ struct SolveFailure {
 struct FailureGuard {
   const unsigned* word = nullptr;  // null: no test
   unsigned call = 0;
+  const RefineRec* const* recs = nullptr;  // null entries: solves that the host has seen succeed
+  int n = 0;                               // at most 64
+  double fail_eta = 0.0;
 };
-// The same for n records (null entries are skipped; f.rec is not read).
-void launch_note_failures(const RefineRec* const* recs, int n, const SolveFailure& f, cudaStream_t s);
 #ifdef __CUDACC__
+__device__ __forceinline__ bool record_failed(const RefineRec* rec, double fail_eta) {
+  return rec != nullptr && (rec->status != RR_OK || (rec->sweeps > 0 && !(rec->eta <= fail_eta)));
+}
 __device__ __forceinline__ void note_failure(const SolveFailure& f) {
-  if (f.rec == nullptr) return;
-  const RefineRec r = *f.rec;
-  if (r.status != RR_OK || (r.sweeps > 0 && !(r.eta <= f.fail_eta))) *f.word = f.call;
+  if (record_failed(f.rec, f.fail_eta)) *f.word = f.call;
 }
 __device__ __forceinline__ bool solve_failed(const FailureGuard& g) { return g.word != nullptr && *g.word == g.call; }
 #endif

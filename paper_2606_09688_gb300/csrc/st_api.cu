@@ -2916,11 +2916,14 @@ st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_d
   std::mutex mu;
   std::condition_variable cv;
   // graph solves report after the levels are queued: the target level looks for
-  // itself (where the levels run in FP64, after one small launch in front of it: 2D box
-  // n = 9 0.441 -> 0.452 ms; such a launch behind every component's graph took it to
-  // 0.64 ms, and waiting for the records here would leave the host's round trip
-  // between the last solve and the level)
-  const FailureGuard guard{h->sc_fail + buf, (unsigned)h->api_seq};
+  // itself (a small launch behind every component's graph took the 2D box, n = 9,
+  // from 0.44 to 0.64 ms, one in front of the level to 0.452; waiting for the records
+  // here would leave the host's round trip between the last solve and the level)
+  FailureGuard guard;
+  if (!h->prof_on) {
+    if (overlap) guard = FailureGuard{h->sc_fail + buf, (unsigned)h->api_seq};
+    else guard = FailureGuard{nullptr, 0, t->recs, nc, fail_eta(h)};
+  }
   auto run = [&](int i) {
     Component& c = *h->comps[i];
     st_status r = solve_one(h, c, forward_io(c), false);
@@ -2973,8 +2976,6 @@ st_status st_solve_combine(st_handle* h, int jx_star, int jt_star, double* out_d
     if (failed) break;
     cudaEvent_t lb = trace.t0 ? trace.make("level " + std::to_string(lev) + " combination start") : nullptr;
     if (lb != nullptr) cudaEventRecord(lb, h->stream);
-    if (lev == jx_star && !overlap && !byc.empty())
-      launch_note_failures(t->recs, nc, SolveFailure{nullptr, fail_eta(h), h->sc_fail + buf, guard.call}, h->stream);
     enqueue_comb_level(h, *t, lev, jx_star, jt_star, out_dev, buf, overlap, guard);
     cudaEvent_t le = trace.t0 ? trace.make("level " + std::to_string(lev) + " combination end") : nullptr;
     if (le != nullptr) cudaEventRecord(le, h->stream);
